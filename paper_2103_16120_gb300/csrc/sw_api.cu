@@ -44,7 +44,8 @@ struct sw_grid_s {
     void *cmem;
     double *ax, *cx, *bx, *ay, *cy, *by, *C, *diag, *lf, *invD, *zz, *gam, *ec, *rowmax, *eta;
     double *gam32, *ec32;          // per row, of the FP32 zonal factors
-    bool f64_valid;                // the FP64 zonal factors match the coefficients and eta
+    double *wgt;                   // nine-point weights of the FP64 policy (NWGT fields)
+    bool f64_valid;                // the FP64 zonal factors and weights match the coefficients and eta
     float *wax, *wcx, *wbx, *way, *wcy, *wby, *wC, *wdiag, *lf32, *invD32, *zz32;
     // the zonal factors transposed per row for the warp-per-row solver (rows
     // of a power of two of at least 128 points; null otherwise)
@@ -142,7 +143,8 @@ extern "C" sw_status sw_grid_create(int nx, int ny, double radius, sw_grid *out)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device);
     size_t N = g->N;
     const bool wt = warp_rows_ok(nx);
-    size_t bytes = 11 * al(N * 8) + 5 * al((size_t)ny * 8) + al(8) + 11 * al(N * 4) + (wt ? 3 * (al(N * 8) + al(N * 4)) : 0);
+    size_t bytes = 11 * al(N * 8) + 5 * al((size_t)ny * 8) + al(8) + 11 * al(N * 4) + (wt ? 3 * (al(N * 8) + al(N * 4)) : 0) +
+                   al((size_t)NWGT * N * 8);
     if (e == cudaSuccess) e = cudaMalloc(&g->cmem, bytes);
     if (e == cudaSuccess) e = cudaMalloc((void **)&g->blk, sizeof(SolverBlock));
     if (e == cudaSuccess) e = cudaMalloc((void **)&g->desc, sizeof(EnsDesc));
@@ -181,6 +183,7 @@ extern "C" sw_status sw_grid_create(int nx, int ny, double radius, sw_grid *out)
         for (auto q : {&g->lfT, &g->invDT, &g->zzT}) { *q = (double *)p; p += al(N * 8); }
         for (auto q : {&g->lf32T, &g->invD32T, &g->zz32T}) { *q = (float *)p; p += al(N * 4); }
     }
+    g->wgt = (double *)p;
     *out = g;
     return SW_OK;
 }
@@ -310,7 +313,7 @@ static FactorArgs factor_args(const sw_grid_s *g)
 }
 
 // new coefficients or eta: the FP32 zonal factors (mixed solvers) now; the
-// FP64 ones when an FP64 solve or preconditioner needs them (ensure_f64)
+// FP64 ones and the nine-point weights when an FP64 solve or preconditioner needs them (ensure_f64)
 static sw_status refactor(sw_grid g, cudaStream_t s)
 {
     CK(launch_factor(factor_args(g), false, row_threads(g->nx), s));
@@ -318,7 +321,7 @@ static sw_status refactor(sw_grid g, cudaStream_t s)
     return SW_OK;
 }
 
-// the FP64 zonal factors, stream-ordered before the FP64 work that follows on
+// the FP64 zonal factors and weights, stream-ordered before the FP64 work that follows on
 // s.  Inside a CUDA graph capture they are always recorded: a replay cannot
 // know whether the coefficients changed since.
 static sw_status ensure_f64(sw_grid g, cudaStream_t s)
@@ -328,6 +331,7 @@ static sw_status ensure_f64(sw_grid g, cudaStream_t s)
     const bool recorded = (cap != cudaStreamCaptureStatusNone);
     if (g->f64_valid && !recorded) return SW_OK;
     CK(launch_factor(factor_args(g), true, row_threads(g->nx), s));
+    CK(launch_weights(WeightArgs{g->nx, g->ny, g->ax, g->cx, g->bx, g->ay, g->cy, g->by, g->C, g->wgt}, s));
     if (!recorded) g->f64_valid = true;
     return SW_OK;
 }
@@ -434,6 +438,7 @@ static void fill_member(sw_grid g, const sw_solve_opts *o, const double *R, doub
         M.wC = (const ct *)g->C; M.wdiag = (const ct *)g->diag;
         M.lf = (const ft *)g->lf; M.invD = (const ft *)g->invD; M.zz = (const ft *)g->zz;
         M.lfT = (const ft *)g->lfT; M.invDT = (const ft *)g->invDT; M.zzT = (const ft *)g->zzT;
+        M.wgt = (const ct *)g->wgt;
     }
     if constexpr (Pol::kMixed) { M.gam = g->gam32; M.ec = g->ec32; }
     else { M.gam = g->gam; M.ec = g->ec; }

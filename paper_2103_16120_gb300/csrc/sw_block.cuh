@@ -45,39 +45,52 @@ __device__ __forceinline__ float warp_max(float x)
     return x;
 }
 
-// Sum over the warp of 32 values per lane at once (transposed butterfly):
-// five exchange levels, each halving the values a lane keeps; lane l ends
-// with the total of value l.  The pairing, hence the rounding, is fixed.
-template <class T>
-__device__ __forceinline__ T warp_sum32(T (&v)[32])
+// Sum over the warp of P values per lane at once (P a power of two <= 32;
+// transposed butterfly): log2 P exchange levels, each halving the values a
+// lane keeps, then plain levels over the lanes that hold the same value; lane
+// l ends with the total of value l P / 32.  P - 1 + log2(32 / P) adds per
+// lane: an FP64 add costs 64 cycles, so the values are not padded to 32.  The
+// pairing, hence the rounding, is fixed.
+__host__ __device__ constexpr int pow2_from(int n) { return n <= 1 ? 1 : 2 * pow2_from((n + 1) / 2); }
+
+template <int O, int CNT, class T, int P>
+__device__ __forceinline__ void warp_sum_level(T (&v)[P])
 {
-    const int lane = threadIdx.x & 31;
+    if constexpr (CNT > 1) {
+        const bool hi = (threadIdx.x & O) != 0;
 #pragma unroll
-    for (int o = 16, cnt = 32; o > 0; o >>= 1, cnt >>= 1) {
-        const bool hi = (lane & o) != 0;
-#pragma unroll
-        for (int k = 0; k < cnt / 2; ++k) {
-            T send = hi ? v[k] : v[k + cnt / 2];
-            T keep = hi ? v[k + cnt / 2] : v[k];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        for (int k = 0; k < CNT / 2; ++k) {
+            T send = hi ? v[k] : v[k + CNT / 2];
+            T keep = hi ? v[k + CNT / 2] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
         }
+    } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
     }
+    if constexpr (O > 1) warp_sum_level<O / 2, (CNT > 1 ? CNT / 2 : 1)>(v);
+}
+
+template <class T, int P>
+__device__ __forceinline__ T warp_sum_many(T (&v)[P])
+{
+    warp_sum_level<16, P>(v);
     return v[0];
 }
 
-// Block sum of NV <= 32 values per thread; tot[q] (shared memory) receives
-// total q in FP64.  scratch: 32 doubles per warp.  Fixed order: a warp
-// butterfly in T, then the warps in index order in FP64.
-template <int NV, class T>
-__device__ __forceinline__ void block_sum_many(const T (&x)[NV], double *tot, double *scratch)
+// Block sum of the first NV <= 32 of a thread's values; tot[q] (shared
+// memory) receives total q in FP64.  scratch: 32 doubles per warp.  Fixed
+// order: a warp butterfly in T, then the warps in index order in FP64.
+template <int NV, class T, int NX>
+__device__ __forceinline__ void block_sum_many(const T (&x)[NX], double *tot, double *scratch)
 {
-    static_assert(NV <= 32, "");
+    static_assert(NV <= NX && NV <= 32, "");
+    constexpr int P = pow2_from(NV);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    T v[32];
+    T v[P];
 #pragma unroll
-    for (int q = 0; q < 32; ++q) v[q] = q < NV ? x[q] : T(0);
-    const T s = warp_sum32(v);
-    scratch[w * 32 + lane] = (double)s;
+    for (int q = 0; q < P; ++q) v[q] = q < NV ? x[q] : T(0);
+    const T s = warp_sum_many<T, P>(v);
+    if ((lane & (32 / P - 1)) == 0) scratch[w * 32 + lane * P / 32] = (double)s;
     __syncthreads();
     if (threadIdx.x < NV) {
         double t = 0;
@@ -106,18 +119,19 @@ __device__ __forceinline__ dfloat df_add(dfloat a, dfloat b)
     return dfloat{hi, e - (hi - s)};
 }
 
-// Block sum of NV <= 32 FP32 values per thread into double-float totals
-// tot[q] (shared memory): a warp butterfly in FP32, then the warps in index
-// order in double-float.  scratch: 32 floats per warp.
-template <int NV>
-__device__ __forceinline__ void block_sum_many_df(const float (&x)[NV], dfloat *tot, float *scratch)
+// Block sum of the first NV <= 32 of a thread's FP32 values into double-float
+// totals tot[q] (shared memory): a warp butterfly in FP32, then the warps in
+// index order in double-float, padded to P values.  scratch: 32 floats per warp.
+template <int NV, int P, int NX>
+__device__ __forceinline__ void block_sum_many_df(const float (&x)[NX], dfloat *tot, float *scratch)
 {
-    static_assert(NV <= 32, "");
+    static_assert(NV <= NX && NV <= P && P <= 32, "");
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    float v[32];
+    float v[P];
 #pragma unroll
-    for (int q = 0; q < 32; ++q) v[q] = q < NV ? x[q] : 0.f;
-    scratch[w * 32 + lane] = warp_sum32(v);
+    for (int q = 0; q < P; ++q) v[q] = q < NV ? x[q] : 0.f;
+    const float s = warp_sum_many<float, P>(v);
+    if ((lane & (32 / P - 1)) == 0) scratch[w * 32 + lane * P / 32] = s;
     __syncthreads();
     if (threadIdx.x < NV) {
         dfloat t{0.f, 0.f};

@@ -84,6 +84,12 @@ template <class T> __device__ __forceinline__ T ldcg(const T *p) { return __ldcg
 // ---------------------------------------------------------------------------
 // grid-level data of one member (one elliptic problem) -- immutable during a launch
 // ---------------------------------------------------------------------------
+// fields of the nine-point weights of the FP64 policy (k_weights):
+//   L x   = sum_k w_k (x_k - x_c) + W_SUM x_c, k over the eight neighbours
+//   P^M x = sum of the six N and S weights times their points
+//           + W_ME x_E + W_MW x_W + W_MC x_c
+enum Weight : int { W_N, W_S, W_NE, W_NW, W_SE, W_SW, W_E, W_W, W_SUM, W_ME, W_MW, W_MC, NWGT };
+
 template <class Pol>
 struct MemberDev {
     typedef typename Pol::coef coef_t;
@@ -103,6 +109,9 @@ struct MemberDev {
     const double *ax, *cx, *bx, *ay, *cy, *by, *C;
     // the same in the policy's coefficient type, and diag(L) (options 1, 2)
     const coef_t *wax, *wcx, *wbx, *way, *wcy, *wby, *wC, *wdiag;
+    // FP64 policy: the stencils of L and P^M as weights of the nine points
+    // (Weight), one field of nx*ny each; null in the mixed policies
+    const coef_t *wgt;
     // zonal factors of T = I - eta (P^Z - P^H): multipliers, inverse pivots,
     // Sherman-Morrison vector; per row gamma and the wrap coupling
     const fac_t *lf, *invD, *zz;

@@ -117,15 +117,36 @@ __device__ void phase_true(const MemberDev<Pol> &M, const RowView<Pol> &v, typen
     const int nx = M.nx, ny = M.ny;
     const size_t row = (size_t)j * nx;
     comp *sb = (comp *)(ws + sb_offset<Pol>(nx));
-    // FP64 coefficients: the policy's own (FP64 policy) or the FP64 copies
-    RowCoef<double> c;
-    if constexpr (Pol::kMixed) {
-        const size_t rs = j > 0 ? row - nx : row;
-        c = {M.ax + row, M.cx + row, M.bx + row, M.ay + row, M.cy + row, M.by + row,
-             M.ay + rs, M.cy + rs, M.by + rs, M.C + row};
-    } else {
-        c = coef_of(v);
+    if constexpr (!Pol::kMixed) {
+        // FP64 policy: the nine-point weights
+        double *ph = (double *)ws;
+        stage3_f64(ph, M.phi, nx, ny, j);
+        constexpr int UW = 2;
+        for (int i0 = threadIdx.x; i0 < nx; i0 += UW * blockDim.x) {
+            double Wt[UW][9], Rv[UW];
+#pragma unroll
+            for (int u = 0; u < UW; ++u) {
+                const int i = min(i0 + u * (int)blockDim.x, nx - 1);
+                load_weights<true>(v, i, Wt[u]);
+                Rv[u] = __ldg(M.R + row + i);
+            }
+#pragma unroll
+            for (int u = 0; u < UW; ++u) {
+                const int i = i0 + u * blockDim.x;
+                if (i >= nx) break;
+                const double rv = stencil9<true>(ph, ph + nx, ph + 2 * nx, i, nx, Wt[u]) - Rv[u];
+                v.r[i] = rv;
+                part[0] += rv * rv;
+                part[1] += Rv[u] * Rv[u];
+                sb[pidx(i)] = stage0_input(M, v, eta, rv, i);
+            }
+        }
+        stage0_finish(M, v, j, ws);
+        return;
     }
+    const size_t rs = j > 0 ? row - nx : row;
+    const RowCoef<double> c = {M.ax + row, M.cx + row, M.bx + row, M.ay + row, M.cy + row, M.by + row,
+                               M.ay + rs, M.cy + rs, M.by + rs, M.C + row};
     // the three Phi rows (FP64), unshifted, into the stage + raw region
     double *ph = (double *)ws;
     int src[3], sh[3];
@@ -236,6 +257,42 @@ __device__ void phase_le(const MemberDev<Pol> &M, const MemberCtl &c, const RowV
     stage3_q(ws, M, M.e, M.e32, M.e_s, j);
     SW_TRACE(101);
     const comp *stg = (const comp *)ws;
+    if constexpr (!Pol::kMixed) {
+        // FP64: L e from the nine-point weights, its products in the same loop
+        constexpr int UW = 2;
+        const double *Lpl[KM];
+#pragma unroll
+        for (int l = 0; l < KM; ++l) Lpl[l] = v.Lpb + (size_t)phys_slot(c, M.k, l < nd ? l : 0) * v.vstride;
+        for (int i0 = threadIdx.x; i0 < nx; i0 += UW * blockDim.x) {
+            double Wt[UW][9], rv[UW], lp[UW][KM];
+#pragma unroll
+            for (int u = 0; u < UW; ++u) {
+                const int i = min(i0 + u * (int)blockDim.x, nx - 1);
+                load_weights<true>(v, i, Wt[u]);
+                rv[u] = v.r[i];
+#pragma unroll
+                for (int l = 0; l < KM; ++l) lp[u][l] = l < nd ? Lpl[l][i] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < UW; ++u) {
+                const int i = i0 + u * blockDim.x;
+                if (i >= nx) break;
+                const double la = stencil9<true>(stg, stg + nx, stg + 2 * nx, i, nx, Wt[u]);
+                v.Le[i] = la;
+                part[0] += la * la;
+                part[1] += rv[u] * la;
+#pragma unroll
+                for (int l = 0; l < KM; ++l) {
+                    if (l < nd) {
+                        part[2 + l] += la * lp[u][l];
+                        part[2 + KM + l] += rv[u] * lp[u][l];
+                    }
+                }
+            }
+        }
+        __syncthreads();           // the block's next row is staged over these
+        return;
+    }
     // L e of the row, straight into the row's L e storage
     if (stencil4_ok(coef_of(v), nx) && ((uintptr_t)v.Le & 15) == 0)
         stencil_row4<comp, typename Pol::coef>(stg, stg + nx, stg + 2 * nx, nx, j, ny, coef_of(v), true, (comp *)v.Le,
@@ -793,8 +850,14 @@ __global__ void __launch_bounds__(MAX_THREADS, MINB) k_gcr(const EnsDesc *__rest
         const int ns = phase_slots(s_c.phase, s_c.nu + 1, slot);
         double *pbuf = partg + (size_t)par * NSLOT * ny;
         if (ns > 0) {
-            if constexpr (Pol::kMixed) block_sum_many_df<NP>(part, (dfloat *)s_blk, (float *)scratch);
-            else block_sum_many<NP, acc_t>(part, s_blk, scratch);
+            if constexpr (Pol::kMixed) {
+                // (the warp-per-row kernels measured 0.5 % slower with 16 values)
+                block_sum_many_df<NP, WARP ? 32 : pow2_from(NP)>(part, (dfloat *)s_blk, (float *)scratch);
+            } else {
+                // the update and the true residual use the slots before T_0 only
+                if (s_c.phase == PH_LE) block_sum_many<NP, acc_t, NP>(part, s_blk, scratch);
+                else block_sum_many<2 + KM, acc_t, NP>(part, s_blk, scratch);
+            }
             if (threadIdx.x < ns) {
                 const int g = slot[threadIdx.x];          // slot of tot; its place in part
                 const int at = g < S_T0 ? g : g - S_T0 + 2 + KM;
@@ -924,7 +987,7 @@ __global__ void __launch_bounds__(MAX_THREADS, MINB) k_gcr(const EnsDesc *__rest
             if (s_c.nR > 0.0)
                 for (int i = threadIdx.x; i < nx; i += blockDim.x) { double x = (double)r[i]; t += x * x; }
             double tv[1] = {t};
-            block_sum_many<1, double>(tv, s_blk, scratch);
+            block_sum_many<1, double, 1>(tv, s_blk, scratch);
             if (threadIdx.x == 0) M.rowres[j] = sqrt(s_blk[0]);
             __syncthreads();
         }

@@ -30,6 +30,13 @@ struct FaceArgs {
     double *rowmax;                                          // max |diag(P^M)| per row
 };
 
+// nine-point weights of L and P^M for the FP64 policy, from the faces
+struct WeightArgs {
+    int nx, ny;
+    const double *ax, *cx, *bx, *ay, *cy, *by, *C;
+    double *wgt;                                             // NWGT fields of nx*ny
+};
+
 struct FactorArgs {
     int nx, ny;
     double eta_explicit;            // > 0: use it; otherwise 1/max|diag(P^M)|
@@ -67,6 +74,7 @@ cudaError_t launch_split_refresh(const SplitRefreshArgs &a, cudaStream_t s);
 cudaError_t launch_split_residual(const SplitResidualArgs &a, cudaStream_t s);
 
 cudaError_t launch_faces(const FaceArgs &a, int threads, cudaStream_t s);
+cudaError_t launch_weights(const WeightArgs &a, cudaStream_t s);
 cudaError_t launch_factor(const FactorArgs &a, bool fp64, int threads, cudaStream_t s);
 size_t gcr_smem_bytes(int prec, int max_nx, int k, int cache_const, int cache_state);
 // shared memory of the warp-per-row mode (0 when nx does not allow it)

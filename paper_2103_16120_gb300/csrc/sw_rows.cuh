@@ -19,7 +19,8 @@ __host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~(size_t)15
 //   raw   mixed policies: the 16-bit / FP32 rows as copied from global memory
 //   sb    one padded row (tridiagonal buffer)
 //   red   reduction / scan scratch
-//   const 11 coefficient rows + 3 padded factor rows of the owned row (optional)
+//   const 11 coefficient rows (FP64: 12 weight rows and the diagonal) + 3
+//         padded factor rows of the owned row (optional)
 //   state r, L e, e copy, (k+1) p rows, (k+1) L p rows of the owned row (optional)
 // ---------------------------------------------------------------------------
 template <class Pol>
@@ -51,9 +52,12 @@ __host__ __device__ inline size_t work_bytes(int nx)
 }
 
 template <class Pol>
+__host__ __device__ constexpr int const_rows() { return Pol::kMixed ? 11 : NWGT + 1; }
+
+template <class Pol>
 __host__ __device__ inline size_t const_bytes(int nx)
 {
-    return al16(11 * (size_t)nx * sizeof(typename Pol::coef)) + al16(3 * (size_t)padded_len(nx) * sizeof(typename Pol::fac));
+    return al16(const_rows<Pol>() * (size_t)nx * sizeof(typename Pol::coef)) + al16(3 * (size_t)padded_len(nx) * sizeof(typename Pol::fac));
 }
 
 template <class Pol>
@@ -72,6 +76,8 @@ struct RowView {
     typedef typename Pol::vec VT;
     // constants (coefficient rows unpadded; factor rows padded when fpad)
     const CT *ax, *cx, *bx, *ay, *cy, *by, *ays, *cys, *bys, *C, *diag;
+    const CT *w;                    // FP64: weight W of point i at w[W * wstride + i]
+    size_t wstride;
     const FT *lf, *invD, *zz;
     bool fpad;
     double gam, ec;
@@ -103,6 +109,7 @@ __device__ __forceinline__ void view_const_global(const MemberDev<Pol> &M, int j
     v.ay = M.way + row; v.cy = M.wcy + row; v.by = M.wby + row;
     v.ays = M.way + rs; v.cys = M.wcy + rs; v.bys = M.wby + rs;
     v.C = M.wC + row; v.diag = M.wdiag + row;
+    if constexpr (!Pol::kMixed) { v.w = M.wgt + row; v.wstride = (size_t)M.nx * M.ny; }
     v.lf = M.lf + row; v.invD = M.invD + row; v.zz = M.zz + row;
     v.fpad = false;
     v.gam = M.gam[j]; v.ec = M.ec[j];
@@ -118,16 +125,24 @@ __device__ void view_const_cache(const MemberDev<Pol> &M, int j, unsigned char *
     RowView<Pol> g;
     view_const_global(M, j, g);
     CT *c = (CT *)slot;
-    const CT *src[11] = {g.ax, g.cx, g.bx, g.ay, g.cy, g.by, g.ays, g.cys, g.bys, g.C, g.diag};
-    for (int a = 0; a < 11; ++a)
-        for (int i = threadIdx.x; i < nx; i += blockDim.x) c[a * nx + i] = src[a][i];
+    if constexpr (Pol::kMixed) {
+        const CT *src[11] = {g.ax, g.cx, g.bx, g.ay, g.cy, g.by, g.ays, g.cys, g.bys, g.C, g.diag};
+        for (int a = 0; a < 11; ++a)
+            for (int i = threadIdx.x; i < nx; i += blockDim.x) c[a * nx + i] = src[a][i];
+        v.ax = c; v.cx = c + nx; v.bx = c + 2 * nx; v.ay = c + 3 * nx; v.cy = c + 4 * nx; v.by = c + 5 * nx;
+        v.ays = c + 6 * nx; v.cys = c + 7 * nx; v.bys = c + 8 * nx; v.C = c + 9 * nx; v.diag = c + 10 * nx;
+    } else {
+        for (int a = 0; a <= NWGT; ++a) {
+            const CT *src = a < NWGT ? g.w + a * g.wstride : g.diag;
+            for (int i = threadIdx.x; i < nx; i += blockDim.x) c[a * nx + i] = src[i];
+        }
+        v.w = c; v.wstride = nx; v.diag = c + NWGT * nx;
+    }
     const int pl = padded_len(nx);
-    FT *f = (FT *)(slot + al16(11 * (size_t)nx * sizeof(CT)));
+    FT *f = (FT *)(slot + al16(const_rows<Pol>() * (size_t)nx * sizeof(CT)));
     const FT *fs[3] = {g.lf, g.invD, g.zz};
     for (int a = 0; a < 3; ++a)
         for (int i = threadIdx.x; i < nx; i += blockDim.x) f[a * pl + pidx(i)] = fs[a][i];
-    v.ax = c; v.cx = c + nx; v.bx = c + 2 * nx; v.ay = c + 3 * nx; v.cy = c + 4 * nx; v.by = c + 5 * nx;
-    v.ays = c + 6 * nx; v.cys = c + 7 * nx; v.bys = c + 8 * nx; v.C = c + 9 * nx; v.diag = c + 10 * nx;
     v.lf = f; v.invD = f + pl; v.zz = f + 2 * pl;
     v.fpad = true;
     v.gam = g.gam; v.ec = g.ec;
@@ -314,6 +329,41 @@ __device__ __forceinline__ bool stencil4_ok(const RowCoef<CT> &c, int nx)
            al(c.ays) && al(c.cys) && al(c.bys);
 }
 
+// The nine-point form of the stencils, for the FP64 policy.  FP64 issues one
+// warp instruction per 64 cycles here, so the instruction count is the time:
+// the flux form above takes 30 (P^M) and 33 (L) per point, the weights 9 and
+// 17.  One FP64 iteration measured 398 against 577 us at 2048 x 1024,
+// 132 against 179 at 1024 x 512, 46 against 58 at 512 x 256 (the weights are 96
+// bytes a point more to hold, 16 more to read in a stage and in L).  L is written with the differences to the centre, which keeps the
+// cancellation of the flux form (a constant field gives W_SUM times it, the
+// fluxes' own b and C terms); P^M only enters multiplied by eta = 1 /
+// max|diag(P^M)| and added to the field it acts on, where the plain sum's
+// rounding is that of the field.  The weights of a point are loaded before
+// its sums start.  Wt[9]: the N, S, NE, NW, SE, SW weights, then E, W and the
+// centre's of the form.
+template <bool FULL, class RV>
+__device__ __forceinline__ void load_weights(const RV &v, int i, double (&Wt)[9])
+{
+#pragma unroll
+    for (int a = 0; a < 6; ++a) Wt[a] = v.w[a * v.wstride + i];
+    Wt[6] = v.w[(FULL ? W_E : W_ME) * v.wstride + i];
+    Wt[7] = v.w[(FULL ? W_W : W_MW) * v.wstride + i];
+    Wt[8] = v.w[(FULL ? W_SUM : W_MC) * v.wstride + i];
+}
+
+template <bool FULL>
+__device__ __forceinline__ double stencil9(const double *S, const double *X, const double *N, int i, int nx,
+                                           const double (&Wt)[9])
+{
+    const int ie = (i + 1 == nx) ? 0 : i + 1, iw = (i == 0) ? nx - 1 : i - 1;
+    const double xc = X[i], o = FULL ? xc : 0.0;
+    const double x[8] = {N[i], S[i], N[ie], N[iw], S[ie], S[iw], X[ie], X[iw]};
+    double s = Wt[8] * xc;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) s = fma(Wt[a], FULL ? x[a] - o : x[a], s);
+    return s;
+}
+
 template <class Pol>
 __device__ __forceinline__ bool in_band(const MemberDev<Pol> &M, int j)
 {
@@ -342,6 +392,25 @@ __device__ __forceinline__ typename Pol::comp q_load(const MemberDev<Pol> &M, co
     }
 }
 
+// stage rows j-1, j, j+1 of an FP64 field, the pole shift as two half-row copies
+__device__ __forceinline__ void stage3_f64(double *stg, const double *f, int nx, int ny, int j)
+{
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        int src, sh;
+        ghost_row(j - 1 + r, nx, ny, src, sh);
+        const double *sr = f + (size_t)src * nx;
+        double *d = stg + (size_t)r * nx;
+        if (sh == 0) {
+            row_copy_issue(d, sr, nx * 8);
+        } else {
+            row_copy_issue(d, sr + sh, (nx - sh) * 8);
+            row_copy_issue(d + (nx - sh), sr, sh * 8);
+        }
+    }
+    row_copy_wait();
+}
+
 // stage rows j-1, j, j+1 of a preconditioner field into stg: the three source
 // rows are copied as they are (one round trip), then converted with their
 // row scales and the pole shift in shared memory
@@ -355,20 +424,7 @@ __device__ __noinline__ void stage3_q(unsigned char *ws, const MemberDev<Pol> &M
     comp *stg = (comp *)ws;
     int src[3], sh[3];
     if constexpr (!Pol::kMixed) {
-        // FP64: straight into the stage, the pole shift as two half-row copies
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            ghost_row(j - 1 + r, nx, ny, src[r], sh[r]);
-            const qt *sr = h + (size_t)src[r] * nx;
-            comp *d = stg + (size_t)r * nx;
-            if (sh[r] == 0) {
-                row_copy_issue(d, sr, nx * (int)sizeof(qt));
-            } else {
-                row_copy_issue(d, sr + sh[r], (nx - sh[r]) * (int)sizeof(qt));
-                row_copy_issue(d + (nx - sh[r]), sr, sh[r] * (int)sizeof(qt));
-            }
-        }
-        row_copy_wait();
+        stage3_f64(stg, h, nx, ny, j);
         return;
     }
     unsigned char *raw = ws + raw_offset<Pol>(nx);
@@ -506,6 +562,32 @@ __device__ void precond_stage(const MemberDev<Pol> &M, const RowView<Pol> &v, ty
     SW_TRACE(301);
     const comp *S = stg, *X = stg + nx, *N = stg + 2 * nx;
     const bool opt3 = (M.pc >= 3);
+    if constexpr (!Pol::kMixed) {
+        constexpr int UW = 2;
+        for (int i0 = threadIdx.x; i0 < nx; i0 += UW * blockDim.x) {
+            double Wt[UW][9], rv[UW], dg[UW];
+#pragma unroll
+            for (int u = 0; u < UW; ++u) {
+                const int i = min(i0 + u * (int)blockDim.x, nx - 1);
+                if (opt3) load_weights<false>(v, i, Wt[u]); else load_weights<true>(v, i, Wt[u]);
+                rv[u] = v.r[i];
+                dg[u] = opt3 ? 1.0 : v.diag[i];
+            }
+#pragma unroll
+            for (int u = 0; u < UW; ++u) {
+                const int i = i0 + u * blockDim.x;
+                if (i >= nx) break;
+                if (opt3) sb[pidx(i)] = X[i] + eta * (stencil9<false>(S, X, N, i, nx, Wt[u]) - rv[u]);
+                else sb[pidx(i)] = X[i] + M.omega * (rv[u] - stencil9<true>(S, X, N, i, nx, Wt[u])) / dg[u];
+            }
+        }
+        __syncthreads();
+        SW_TRACE(302);
+        if (opt3) trisolve_view(sb, nx, v, sm);
+        SW_TRACE(303);
+        q_store_row(M, oh, of32, os, j, sb, last ? v.el : (comp *)nullptr, (float *)sm);
+        return;
+    }
     if (stencil4_ok(coef_of(v), nx))
         stencil_row4<comp, typename Pol::coef>(S, X, N, nx, j, ny, coef_of(v), !opt3, sb, true);
     else

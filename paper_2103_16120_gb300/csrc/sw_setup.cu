@@ -66,6 +66,44 @@ __global__ void __launch_bounds__(MAX_THREADS) k_faces(FaceArgs a)
     }
 }
 
+// The weights of the nine points in L and P^M (sw_common.cuh, Weight), the
+// face terms of a point gathered: with Fe = cx (xn + xne - xs - xse) + bx (xc
+// + xe) + ax (xe - xc) through the east face, and so on, L = Fe - Fw + Fn - Fs
+// - C xc.  20 FP64 operations a point, once per set of coefficients that an
+// FP64 solve or preconditioner uses.
+__global__ void __launch_bounds__(128) k_weights(WeightArgs a)
+{
+    const int nx = a.nx, ny = a.ny, j = blockIdx.x;
+    const int i = blockIdx.y * blockDim.x + threadIdx.x;
+    if (i >= nx) return;
+    const size_t row = (size_t)j * nx, id = row + i, iw = row + (i == 0 ? nx - 1 : i - 1), N = (size_t)nx * ny;
+    const double ax = a.ax[id], axw = a.ax[iw], cx = a.cx[id], cxw = a.cx[iw], bx = a.bx[id], bxw = a.bx[iw];
+    // the faces of the last row are zero; the row below the first has none
+    const double ay = a.ay[id], cy = a.cy[id], by = a.by[id];
+    const double ays = j > 0 ? a.ay[id - nx] : 0.0, cys = j > 0 ? a.cy[id - nx] : 0.0, bys = j > 0 ? a.by[id - nx] : 0.0;
+    const double cxd = cx - cxw, bd = (bx - bxw) + (by - bys), cyd = cy - cys;
+    const double me = bx + cyd, mw = -(bxw + cyd);
+    double *w = a.wgt + id;
+    w[W_N * N] = cxd + (ay + by);
+    w[W_S * N] = (ays - bys) - cxd;
+    w[W_NE * N] = cx + cy;
+    w[W_NW * N] = -(cxw + cy);
+    w[W_SE * N] = -(cx + cys);
+    w[W_SW * N] = cxw + cys;
+    w[W_E * N] = ax + me;
+    w[W_W * N] = axw + mw;
+    w[W_SUM * N] = 2.0 * bd - a.C[id];
+    w[W_ME * N] = me;
+    w[W_MW * N] = mw;
+    w[W_MC * N] = bd - (ay + ays);
+}
+
+cudaError_t launch_weights(const WeightArgs &a, cudaStream_t s)
+{
+    k_weights<<<dim3(a.ny, (a.nx + 127) / 128), 128, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 // 2x2 matrix [[m00, m01], [m10, m11]]
 template <class T> struct M2 { T m00, m01, m10, m11; };
 
