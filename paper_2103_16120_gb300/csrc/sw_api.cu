@@ -93,11 +93,30 @@ GridView sw::grid_view(const sw_grid_s *g)
     return GridView{g->nx, g->ny, g->device, g->sms, g->wax, g->way, g->wdiag};
 }
 
-// threads of the block that works on one row: about four values per thread,
-// at least nx/16 (the tridiagonal chunks live in registers, 16 values at most)
+// threads of the block that works on one row: four warps, one for each of the
+// SM's schedulers and FP64 pipes, which every row of up to 1024 points then
+// uses, and eight for longer rows; at least nx/16 (the tridiagonal chunks live
+// in registers, 16 values at most).  About four points a thread, as before,
+// leaves rows of 128 points with one warp and one FP64 pipe: us per iteration
+// FP64 / FP16 with 32-192 and with 128 threads: 128 x 64 48 / 36 and 31 / 28,
+// 256 x 128 42 / 32 and 32 / 27, 360 x 181 46 / 32 and 46 / 29, 768 x 384
+// 101 / 49 and 81 / 41, 1024 x 512 (FP64) 132 and 118.  2048 x 1024 (FP64)
+// takes 397 with 256 and 508 with 128; 1440 x 721 (FP16) 104 and 109.
 static int row_threads(int nx, int requested = 0)
 {
-    int t = requested > 0 ? requested : ((nx / 4 + 31) / 32) * 32;
+    int t = requested > 0 ? requested : (nx <= 1024 ? 128 : MAX_THREADS);
+    const int tmin = ((nx + 16 * 32 - 1) / (16 * 32)) * 32;
+    if (t < tmin) t = tmin;
+    if (t < 32) t = 32;
+    if (t > MAX_THREADS) t = MAX_THREADS;
+    return t;
+}
+
+// threads of the set-up kernels' blocks, one row each: about four points a
+// thread (the pivots' chunks set the rounding of the FP32 factors)
+static int setup_threads(int nx)
+{
+    int t = ((nx / 4 + 31) / 32) * 32;
     const int tmin = ((nx + 16 * 32 - 1) / (16 * 32)) * 32;
     if (t < tmin) t = tmin;
     if (t < 32) t = 32;
@@ -316,7 +335,7 @@ static FactorArgs factor_args(const sw_grid_s *g)
 // FP64 ones and the nine-point weights when an FP64 solve or preconditioner needs them (ensure_f64)
 static sw_status refactor(sw_grid g, cudaStream_t s)
 {
-    CK(launch_factor(factor_args(g), false, row_threads(g->nx), s));
+    CK(launch_factor(factor_args(g), false, setup_threads(g->nx), s));
     g->f64_valid = false;
     return SW_OK;
 }
@@ -330,7 +349,7 @@ static sw_status ensure_f64(sw_grid g, cudaStream_t s)
     CK(cudaStreamIsCapturing(s, &cap));
     const bool recorded = (cap != cudaStreamCaptureStatusNone);
     if (g->f64_valid && !recorded) return SW_OK;
-    CK(launch_factor(factor_args(g), true, row_threads(g->nx), s));
+    CK(launch_factor(factor_args(g), true, setup_threads(g->nx), s));
     CK(launch_weights(WeightArgs{g->nx, g->ny, g->ax, g->cx, g->bx, g->ay, g->cy, g->by, g->C, g->wgt}, s));
     if (!recorded) g->f64_valid = true;
     return SW_OK;
@@ -350,7 +369,7 @@ extern "C" sw_status sw_elliptic_set_coeffs(sw_grid g, const double *A11, const 
     a.ax = g->ax; a.cx = g->cx; a.bx = g->bx; a.ay = g->ay; a.cy = g->cy; a.by = g->by; a.C64 = g->C; a.diag = g->diag;
     a.wax = g->wax; a.wcx = g->wcx; a.wbx = g->wbx; a.way = g->way; a.wcy = g->wcy; a.wby = g->wby; a.wC = g->wC;
     a.wdiag = g->wdiag; a.rowmax = g->rowmax;
-    CK(launch_faces(a, row_threads(g->nx), s));
+    CK(launch_faces(a, setup_threads(g->nx), s));
     sw_status st = refactor(g, s);
     if (st) return st;
     g->has_coeffs = true;
@@ -565,13 +584,21 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     if (o->row_mode == 2 && !warp_possible)
         return fail(SW_ERR_INVALID_ARG, "row_mode 2 (one warp per row) needs grids with nx a power of two >= 128 "
                                         "and a preconditioner other than the learned one");
-    for (int lv = (o->pc == SW_PC_LEARNED ? 1 : 0); lv < 3 && !P.grid && o->row_mode != 2; ++lv) {
-        const size_t sm_l = gcr_smem_bytes(o->prec, max_nx, o->k, levels[lv][0], levels[lv][1]);
-        int bps = 0;
-        CK(gcr_occupancy(o->prec, o->k, 1, 0, P.threads, sm_l, &bps));
-        if (bps > 0 && rows_total <= (long)bps * sms) {
-            for (int m = 0; m < n; ++m) P.nb[m] = grids[m]->ny;
-            P.grid = (int)rows_total; P.cc = levels[lv][0]; P.cs = levels[lv][1]; P.smem = sm_l;
+    // one row per block where that fits, with row_threads' four warps or else
+    // with about four points a thread (members of an ensemble, or rows of few
+    // points, then still get a block each)
+    const int narrow = o->threads_per_row > 0 ? P.threads : setup_threads(max_nx);
+    const int shapes[2] = {P.threads, narrow};
+    for (int sh = 0; sh < (narrow < P.threads ? 2 : 1) && !P.grid && o->row_mode != 2; ++sh) {
+        for (int lv = (o->pc == SW_PC_LEARNED ? 1 : 0); lv < 3 && !P.grid; ++lv) {
+            const size_t sm_l = gcr_smem_bytes(o->prec, max_nx, o->k, levels[lv][0], levels[lv][1]);
+            int bps = 0;
+            CK(gcr_occupancy(o->prec, o->k, 1, 0, shapes[sh], sm_l, &bps));
+            if (bps > 0 && rows_total <= (long)bps * sms) {
+                for (int m = 0; m < n; ++m) P.nb[m] = grids[m]->ny;
+                P.threads = shapes[sh];
+                P.grid = (int)rows_total; P.cc = levels[lv][0]; P.cs = levels[lv][1]; P.smem = sm_l;
+            }
         }
     }
     // the automatic choice takes one warp per row for the mixed precisions;
@@ -655,6 +682,7 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
         // resident blocks
         P.smem = gcr_smem_bytes(o->prec, max_nx, o->k, 0, 0);
         P.cc = P.cs = 0;
+        if (n > 1) P.threads = narrow;
         int bps = 0, bps2 = 0;
         CK(gcr_occupancy(o->prec, o->k, 1, 0, P.threads, P.smem, &bps));
         CK(gcr_occupancy(o->prec, o->k, 2, 0, P.threads, P.smem, &bps2));
