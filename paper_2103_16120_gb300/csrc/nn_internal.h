@@ -50,6 +50,8 @@ struct ConvArgs {
     __nv_bfloat16 *y;           // [B][H][W][cout] (unless yf is set)
     float *yf;                  // FP32 output [B][H][W][yf_c] of channels < yf_c, or null
     int yf_c;
+    const __nv_bfloat16 *xc;    // tcgen05: first input channels, from the coarser level [B][H/2][W/2][.]
+    __nv_bfloat16 *yp;          // tcgen05: 2x2 mean of y [B][H/2][W/2][cout]
     const __nv_bfloat16 *mask;  // [B][H][W][cout]: zero the output where mask <= 0 (ReLU derivative), or null
     int B, H, W;
     int relu;
@@ -58,23 +60,28 @@ struct ConvArgs {
 struct WgradArgs {
     const __nv_bfloat16 *g;     // [B][H][W][cout]  gradient at the layer output (pre-activation)
     const __nv_bfloat16 *x;     // [B][H][W][cin]   layer input
+    const __nv_bfloat16 *xc;    // tcgen05: the first input channels, from the coarser level (x holds the others)
     float *dw;                  // [9][cout][cin]   accumulated (FP32)
     float *db;                  // [cout] accumulated, or null
     int B, H, W;
 };
 
 cudaError_t launch_conv(int cin, int cout, bool dgrad, const ConvArgs &a, int sms, cudaStream_t s);
-// the same convolution on tcgen05 (nn_tc.cu) where its rows are a multiple of
-// 128 points and the operands fit in shared memory; err (device) is set if a
+// the network's convolutions and input gradients on tcgen05 (nn_tc.cu), with
+// what follows them fused, for rows of a multiple of 128 points (the others
+// take launch_conv and the kernels of nn_ops.cu); err (device) is set if a
 // tensor-core wait ran out
-bool conv_tc_supported(int cin, int cout, bool dgrad, int W);
-cudaError_t launch_conv_tc(int cin, int cout, bool dgrad, const ConvArgs &a, int sms, int *err, cudaStream_t s);
-inline cudaError_t launch_conv_auto(int cin, int cout, bool dgrad, const ConvArgs &a, int sms, int *err,
-                                    cudaStream_t s)
-{
-    return conv_tc_supported(cin, cout, dgrad, a.W) ? launch_conv_tc(cin, cout, dgrad, a, sms, err, s)
-                                                    : launch_conv(cin, cout, dgrad, a, sms, s);
-}
+enum ConvStep : int {
+    CONV_C1, CONV_C2,   // x -> y, and its 2x2 mean -> yp
+    CONV_C3,            // x -> y
+    CONV_C4, CONV_C5,   // [up(xc), x] -> y
+    CONV_C6,            // x -> yf
+    CONV_D6,            // x -> y, zero where mask <= 0
+    CONV_D5, CONV_D4,   // x -> the adjoint of [up, skip]: coarse part (mask: coarse activation) -> y, skip part -> yf
+    CONV_D3, CONV_D2    // x -> yf
+};
+inline bool conv_tc_rows(int W) { return W % 128 == 0; }
+cudaError_t launch_conv_tc(ConvStep step, const ConvArgs &a, int sms, int *err, cudaStream_t s);
 cudaError_t launch_wgrad(int cin, int cout, const WgradArgs &a, int sms, cudaStream_t s);
 // the weight gradient on tcgen05 (nn_tc.cu) for the layers it takes
 bool wgrad_tc_supported(int cin, int cout, int W);

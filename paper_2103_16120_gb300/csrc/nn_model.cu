@@ -124,8 +124,8 @@ sw_status check_err(sw_model_s *M)
 
 ConvArgs conv_args(const bf16 *x, const bf16 *w, const float *bias, bf16 *y, int B, int H, int W, int relu)
 {
-    ConvArgs a;
-    a.x = x; a.w = w; a.bias = bias; a.y = y; a.yf = nullptr; a.yf_c = 0; a.mask = nullptr;
+    ConvArgs a{};
+    a.x = x; a.w = w; a.bias = bias; a.y = y;
     a.B = B; a.H = H; a.W = W; a.relu = relu;
     return a;
 }
@@ -144,19 +144,35 @@ sw_status forward(sw_model_s *M, int B, int H, int W, const float *x0, cudaStrea
 {
     Acts &A = M->A;
     const int H1 = H / 2, W1 = W / 2, H2 = H / 4, W2 = W / 4;
+    // a convolution and the pooling of its output
+    auto conv_pool = [&](ConvStep step, int l, const bf16 *x, bf16 *y, bf16 *yp, int h, int w) -> cudaError_t {
+        ConvArgs a = conv_args(x, M->wf[l], M->bias[l], y, B, h, w, 1);
+        a.yp = yp;
+        if (conv_tc_rows(w)) return launch_conv_tc(step, a, M->sms, M->err, s);
+        const cudaError_t e = launch_conv(LAYER[l].cin_pad, LAYER[l].cout_pad, false, a, M->sms, s);
+        return e != cudaSuccess ? e : launch_pool(y, yp, B, h, w, LAYER[l].cout_pad, s);
+    };
+    // a convolution of [up(coarse), skip]; cat: where it is stored for rows
+    // that the tcgen05 kernel does not take
+    auto conv_cat = [&](ConvStep step, int l, const bf16 *coarse, const bf16 *skip, int cs, bf16 *cat, bf16 *y, int h,
+                        int w) -> cudaError_t {
+        ConvArgs a = conv_args(skip, M->wf[l], M->bias[l], y, B, h, w, 1);
+        a.xc = coarse;
+        if (conv_tc_rows(w)) return launch_conv_tc(step, a, M->sms, M->err, s);
+        const cudaError_t e = launch_cat_up(coarse, 64, skip, cs, cat, B, h, w, s);
+        a.x = cat;
+        return e != cudaSuccess ? e : launch_conv(64 + cs, LAYER[l].cout_pad, false, a, M->sms, s);
+    };
     NCK(launch_pack_input(x0, A.x0b, B, H, W, s));
-    NCK(launch_conv_auto(16, 32, false, conv_args(A.x0b, M->wf[0], M->bias[0], A.a1, B, H, W, 1), M->sms, M->err, s));
-    NCK(launch_pool(A.a1, A.p1, B, H, W, 32, s));
-    NCK(launch_conv_auto(32, 64, false, conv_args(A.p1, M->wf[1], M->bias[1], A.a2, B, H1, W1, 1), M->sms, M->err, s));
-    NCK(launch_pool(A.a2, A.p2, B, H1, W1, 64, s));
-    NCK(launch_conv_auto(64, 64, false, conv_args(A.p2, M->wf[2], M->bias[2], A.a3, B, H2, W2, 1), M->sms, M->err, s));
-    NCK(launch_cat_up(A.a3, 64, A.a2, 64, A.cat4, B, H1, W1, s));
-    NCK(launch_conv_auto(128, 64, false, conv_args(A.cat4, M->wf[3], M->bias[3], A.a4, B, H1, W1, 1), M->sms, M->err, s));
-    NCK(launch_cat_up(A.a4, 64, A.a1, 32, A.cat5, B, H, W, s));
-    NCK(launch_conv_auto(96, 32, false, conv_args(A.cat5, M->wf[4], M->bias[4], A.a5, B, H, W, 1), M->sms, M->err, s));
+    NCK(conv_pool(CONV_C1, 0, A.x0b, A.a1, A.p1, H, W));
+    NCK(conv_pool(CONV_C2, 1, A.p1, A.a2, A.p2, H1, W1));
+    const ConvArgs c3 = conv_args(A.p2, M->wf[2], M->bias[2], A.a3, B, H2, W2, 1);
+    NCK(conv_tc_rows(W2) ? launch_conv_tc(CONV_C3, c3, M->sms, M->err, s) : launch_conv(64, 64, false, c3, M->sms, s));
+    NCK(conv_cat(CONV_C4, 3, A.a3, A.a2, 64, A.cat4, A.a4, H1, W1));
+    NCK(conv_cat(CONV_C5, 4, A.a4, A.a1, 32, A.cat5, A.a5, H, W));
     ConvArgs o = conv_args(A.a5, M->wf[5], M->bias[5], nullptr, B, H, W, 0);
     o.yf = A.y; o.yf_c = 1;
-    NCK(launch_conv_auto(32, 16, false, o, M->sms, M->err, s));
+    NCK(conv_tc_rows(W) ? launch_conv_tc(CONV_C6, o, M->sms, M->err, s) : launch_conv(32, 16, false, o, M->sms, s));
     return SW_OK;
 }
 
@@ -171,33 +187,55 @@ sw_status backward(sw_model_s *M, int B, int H, int W, const float *target, cuda
     }
     NCK(cudaMemsetAsync(A.scal + 1, 0, sizeof(double), s));
     NCK(launch_loss(A.y, target, A.gy16, A.scal + 1, B, H, W, s));
-    auto wg = [&](int l, const bf16 *g, const bf16 *x, int b_, int h_, int w_) {
-        WgradArgs a{g, x, M->dw[l], M->db[l], b_, h_, w_};
+    auto wg = [&](int l, const bf16 *g, const bf16 *x, int h_, int w_, const bf16 *coarse = nullptr,
+                  const bf16 *cat = nullptr) {
+        // a concatenated input is stored only where the forward pass stored it
+        WgradArgs a{g, x, coarse, M->dw[l], M->db[l], B, h_, w_};
+        if (cat && !conv_tc_rows(w_)) a.x = cat;
         return launch_wgrad_auto(LAYER[l].cin_pad, LAYER[l].cout_pad, a, M->sms, M->err, s);
     };
+    // input gradient with FP32 output
+    auto dgrad = [&](ConvStep step, int l, const bf16 *g, float *out, int h, int w) {
+        const int co = LAYER[l].cin_pad;
+        const ConvArgs a = dgrad_args(g, M->wd[l], out, co, B, h, w);
+        return conv_tc_rows(w) ? launch_conv_tc(step, a, M->sms, M->err, s)
+                               : launch_conv(LAYER[l].cout_pad, co, true, a, M->sms, s);
+    };
+    // input gradient of a convolution of [up(coarse), skip], split into the
+    // coarse level's gradient (times the ReLU derivative) and the skip's
+    auto dgrad_cat = [&](ConvStep step, int l, const bf16 *g, float *gcat, int cs, const bf16 *coarse, bf16 *gz,
+                         float *gskip, int h, int w) -> cudaError_t {
+        if (conv_tc_rows(w)) {
+            ConvArgs a = conv_args(g, M->wd[l], nullptr, gz, B, h, w, 0);
+            a.mask = coarse;
+            a.yf = gskip;
+            return launch_conv_tc(step, a, M->sms, M->err, s);
+        }
+        const cudaError_t e =
+            launch_conv(LAYER[l].cout_pad, 64 + cs, true, dgrad_args(g, M->wd[l], gcat, 64 + cs, B, h, w), M->sms, s);
+        return e != cudaSuccess ? e : launch_split_up_bwd(gcat, 64, cs, coarse, gz, gskip, B, h, w, s);
+    };
     // c6 (32 -> 1, padded to 16 outputs)
-    NCK(wg(5, A.gy16, A.a5, B, H, W));
+    NCK(wg(5, A.gy16, A.a5, H, W));
     ConvArgs d6 = conv_args(A.gy16, M->wd[5], nullptr, A.gz5, B, H, W, 0);
     d6.mask = A.a5;
-    NCK(launch_conv_auto(16, 32, true, d6, M->sms, M->err, s));
+    NCK(conv_tc_rows(W) ? launch_conv_tc(CONV_D6, d6, M->sms, M->err, s) : launch_conv(16, 32, true, d6, M->sms, s));
     // c5 (96 -> 32) on [up(a4), a1]
-    NCK(wg(4, A.gz5, A.cat5, B, H, W));
-    NCK(launch_conv_auto(32, 96, true, dgrad_args(A.gz5, M->wd[4], A.gcat5, 96, B, H, W), M->sms, M->err, s));
-    NCK(launch_split_up_bwd(A.gcat5, 64, 32, A.a4, A.gz4, A.gskip1, B, H, W, s));
+    NCK(wg(4, A.gz5, A.a1, H, W, A.a4, A.cat5));
+    NCK(dgrad_cat(CONV_D5, 4, A.gz5, A.gcat5, 32, A.a4, A.gz4, A.gskip1, H, W));
     // c4 (128 -> 64) on [up(a3), a2]
-    NCK(wg(3, A.gz4, A.cat4, B, H1, W1));
-    NCK(launch_conv_auto(64, 128, true, dgrad_args(A.gz4, M->wd[3], A.gcat4, 128, B, H1, W1), M->sms, M->err, s));
-    NCK(launch_split_up_bwd(A.gcat4, 64, 64, A.a3, A.gz3, A.gskip2, B, H1, W1, s));
+    NCK(wg(3, A.gz4, A.a2, H1, W1, A.a3, A.cat4));
+    NCK(dgrad_cat(CONV_D4, 3, A.gz4, A.gcat4, 64, A.a3, A.gz3, A.gskip2, H1, W1));
     // c3 (64 -> 64) on pool(a2)
-    NCK(wg(2, A.gz3, A.p2, B, H2, W2));
-    NCK(launch_conv_auto(64, 64, true, dgrad_args(A.gz3, M->wd[2], A.gp2, 64, B, H2, W2), M->sms, M->err, s));
+    NCK(wg(2, A.gz3, A.p2, H2, W2));
+    NCK(dgrad(CONV_D3, 2, A.gz3, A.gp2, H2, W2));
     NCK(launch_pool_bwd(A.gskip2, A.gp2, A.a2, A.gz2, B, H1, W1, 64, s));
     // c2 (32 -> 64) on pool(a1)
-    NCK(wg(1, A.gz2, A.p1, B, H1, W1));
-    NCK(launch_conv_auto(64, 32, true, dgrad_args(A.gz2, M->wd[1], A.gp1, 32, B, H1, W1), M->sms, M->err, s));
+    NCK(wg(1, A.gz2, A.p1, H1, W1));
+    NCK(dgrad(CONV_D2, 1, A.gz2, A.gp1, H1, W1));
     NCK(launch_pool_bwd(A.gskip1, A.gp1, A.a1, A.gz1, B, H, W, 32, s));
     // c1 (4 -> 32, inputs padded to 16)
-    NCK(wg(0, A.gz1, A.x0b, B, H, W));
+    NCK(wg(0, A.gz1, A.x0b, H, W));
     GradPtrs gp;
     for (int l = 0; l < NLAYERS; ++l) { gp.dw[l] = M->dw[l]; gp.db[l] = M->db[l]; }
     NCK(launch_flatten_grad(gp, M->gflat, s));

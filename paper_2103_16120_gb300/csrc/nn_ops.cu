@@ -74,17 +74,27 @@ __global__ void k_skip_bwd(const float *gcat, int cc, int cs, float *gskip, int 
     }
 }
 
-// gz = (g_skip + pool-adjoint of g_pooled) * (a > 0)
-__global__ void k_pool_bwd(const float *gskip, const float *gp, const __nv_bfloat16 *a, __nv_bfloat16 *gz,
-                           int B, int H, int W, int C)
+// gz = (g_skip + pool-adjoint of g_pooled) * (a > 0), C = 8 << lc8.  Bound by
+// its bytes (32-bit gradients of two levels, two 16-bit fields): a block takes
+// one row, a thread 8 channels of a point in 16-byte accesses.  At 32 x 256 x
+// 128 x 32 (268 MB) one value a thread with 64-bit index arithmetic took 157 us.
+__global__ void __launch_bounds__(256) k_pool_bwd(const float4 *gskip, const float4 *gp, const uint4 *a, uint4 *gz,
+                                                  int H, int W, int lc8)
 {
-    const size_t n = (size_t)B * H * W * C;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(q % C);
-        const size_t pix = q / C;
-        const int w = (int)(pix % W), h = (int)((pix / W) % H), b = (int)(pix / W / H);
-        const float g = gskip[q] + 0.25f * gp[(((size_t)b * (H / 2) + h / 2) * (W / 2) + w / 2) * C + c];
-        gz[q] = __float2bfloat16_rn(__bfloat162float(a[q]) > 0.f ? g : 0.f);
+    const int row = blockIdx.x, b = row / H, h = row - b * H, n = W << lc8;
+    const size_t at = (size_t)row * n, cat = ((size_t)b * (H / 2) + h / 2) * (W / 2) << lc8;
+    for (int q = threadIdx.x; q < n; q += 256) {
+        const size_t cq = cat + ((size_t)((q >> lc8) >> 1) << lc8) + (q & ((1 << lc8) - 1));
+        const float4 s0 = __ldg(gskip + 2 * (at + q)), s1 = __ldg(gskip + 2 * (at + q) + 1);
+        const float4 p0 = __ldg(gp + 2 * cq), p1 = __ldg(gp + 2 * cq + 1);
+        const uint4 av = __ldg(a + at + q);
+        const __nv_bfloat16 *act = (const __nv_bfloat16 *)&av;
+        const float g[8] = {s0.x + 0.25f * p0.x, s0.y + 0.25f * p0.y, s0.z + 0.25f * p0.z, s0.w + 0.25f * p0.w,
+                            s1.x + 0.25f * p1.x, s1.y + 0.25f * p1.y, s1.z + 0.25f * p1.z, s1.w + 0.25f * p1.w};
+        __nv_bfloat16 o[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o[k] = __float2bfloat16_rn(__bfloat162float(act[k]) > 0.f ? g[k] : 0.f);
+        gz[at + q] = *(const uint4 *)o;
     }
 }
 
@@ -153,7 +163,8 @@ struct LayerPtrs {
 // padded channels are zero
 __global__ void k_pack(PackArgs a, LayerPtrs lp)
 {
-    for (int l = 0; l < NLAYERS; ++l) {
+    {
+        const int l = blockIdx.y;                  // one layer's blocks
         const LayerShape S = lp.sh[l];
         const float *w = a.master + lp.off[l];
         const int nf = 9 * S.cout_pad * S.cin_pad;
@@ -178,7 +189,8 @@ __global__ void k_pack(PackArgs a, LayerPtrs lp)
 
 __global__ void k_flatten_grad(GradPtrs g, LayerPtrs lp, float *flat)
 {
-    for (int l = 0; l < NLAYERS; ++l) {
+    {
+        const int l = blockIdx.y;                  // one layer's blocks
         const LayerShape S = lp.sh[l];
         const int nw = S.cout * S.cin * 9;
         for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nw + S.cout; q += gridDim.x * blockDim.x) {
@@ -251,8 +263,10 @@ cudaError_t launch_split_up_bwd(const float *gcat, int cc, int cs, const __nv_bf
 cudaError_t launch_pool_bwd(const float *g_skip, const float *g_pooled, const __nv_bfloat16 *a,
                             __nv_bfloat16 *gz, int B, int H, int W, int C, cudaStream_t s)
 {
-    const size_t n = (size_t)B * H * W * C;
-    k_pool_bwd<<<blocks_for(n, 256), 256, 0, s>>>(g_skip, g_pooled, a, gz, B, H, W, C);
+    int lc8 = 0;
+    while ((8 << lc8) < C) ++lc8;
+    k_pool_bwd<<<B * H, 256, 0, s>>>((const float4 *)g_skip, (const float4 *)g_pooled, (const uint4 *)a, (uint4 *)gz,
+                                     H, W, lc8);
     return cudaGetLastError();
 }
 
@@ -273,13 +287,13 @@ cudaError_t launch_pack_input(const float *x0, __nv_bfloat16 *xb, int B, int H, 
 
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t s)
 {
-    k_pack<<<64, 256, 0, s>>>(a, layer_ptrs());
+    k_pack<<<dim3(64, NLAYERS), 256, 0, s>>>(a, layer_ptrs());
     return cudaGetLastError();
 }
 
 cudaError_t launch_flatten_grad(const GradPtrs &g, float *flat, cudaStream_t s)
 {
-    k_flatten_grad<<<64, 256, 0, s>>>(g, layer_ptrs(), flat);
+    k_flatten_grad<<<dim3(64, NLAYERS), 256, 0, s>>>(g, layer_ptrs(), flat);
     return cudaGetLastError();
 }
 

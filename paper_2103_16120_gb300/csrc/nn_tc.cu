@@ -1,6 +1,7 @@
-// nn_tc.cu -- the 3x3 convolution of nn_conv.cu on the fifth-generation
-// tensor cores (tcgen05): BF16 operands from shared memory, FP32 accumulator
-// in tensor memory (TMEM), one thread issuing the MMAs.
+// nn_tc.cu -- the 3x3 convolutions and weight gradients of nn_conv.cu on the
+// fifth-generation tensor cores (tcgen05), for rows of a multiple of 128
+// points: BF16 operands from shared memory, FP32 accumulator in tensor memory
+// (TMEM), one thread issuing the MMAs.
 //
 // Tile: 128 consecutive output points of one latitude row (M = 128) x all
 // output channels (N = COUT).  Operands use the no-swizzle K-major layout:
@@ -11,14 +12,10 @@
 // 16 ks + 15, A starts at row ky, plane 2 ks, point kx, and one
 // tcgen05.mma of K = 16 accumulates it.
 //
-// A block works down a strip of 16 rows of one 128-point column.  Input
-// rows sit in a ring of four shared-memory slots (plus the two shifted pole
-// rows of the input gradient), so every input row is staged once, and the
-// accumulator is double-buffered in TMEM.  While the tensor core computes
-// row h (thread 0 issues 9 * CIN / 16 MMAs, 12 * ... on a pole row, and
-// commits them to an mbarrier), the block reads row h-1 out of TMEM
-// (each warp its 32 lanes), stores it, and stages input row h+2 with
-// cp.async into the slot row h-2 used.  Every mbarrier wait is bounded.
+// A block works down strips of up to 8 rows of one 128-point column.  Input
+// rows sit in a ring of shared-memory slots (the shifted pole rows of the
+// input gradient among them), so every input row of a strip is staged once.
+// Every mbarrier wait is bounded.
 #include <cuda_bf16.h>
 #include <cstdint>
 
@@ -74,6 +71,35 @@ __device__ __forceinline__ void mma_bf16(unsigned dtmem, unsigned long long a, u
         : "memory");
 }
 
+// the same, issued by the lane with one != 0 of a warp that runs together: the
+// descriptors are then warp-uniform values
+__device__ __forceinline__ void mma_bf16_one(unsigned dtmem, unsigned long long a, unsigned long long b, unsigned id,
+                                             unsigned accumulate, unsigned one)
+{
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %4, 0;\n setp.ne.u32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "l"(a), "l"(b), "r"(id), "r"(accumulate), "r"(one)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_commit_one(unsigned mbar, unsigned one)
+{
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.u32 q, %1, 0;\n"
+        " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(mbar),
+        "r"(one)
+        : "memory");
+}
+
+// one lane of a converged warp: 1 in that lane, 0 in the others
+__device__ __forceinline__ unsigned elect_one()
+{
+    unsigned one;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(one));
+    return one;
+}
+
 __device__ __forceinline__ void mma_commit(unsigned mbar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
@@ -112,249 +138,464 @@ __device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8])
     for (int q = 0; q < 8; ++q) v[q] = __uint_as_float(r[q]);
 }
 
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, float *v)
+{
+    unsigned r[16];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr));
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
+}
+
+__device__ __forceinline__ void mbar_init(unsigned long long *b, unsigned count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(unsigned long long *b)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+
+// 16 of a thread's 32 (8 of 16) values as BF16: the upper half if hi; zero
+// where mask (if any) is not positive
+template <int N>
+__device__ __forceinline__ void store_half(const float (&v)[N], int hi, const __nv_bfloat16 *mask, __nv_bfloat16 *out)
+{
+#pragma unroll
+    for (int k = 0; k < N / 16; ++k) {
+        float x[8];
+#pragma unroll
+        for (int z = 0; z < 8; ++z) x[z] = hi ? v[N / 2 + 8 * k + z] : v[8 * k + z];
+        if (mask) {
+            const uint4 mq = __ldg((const uint4 *)mask + k);
+            const __nv_bfloat16 *mv = (const __nv_bfloat16 *)&mq;
+#pragma unroll
+            for (int z = 0; z < 8; ++z)
+                if (!(__bfloat162float(mv[z]) > 0.f)) x[z] = 0.f;
+        }
+        __nv_bfloat162 o2[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) o2[z] = __floats2bfloat162_rn(x[2 * z], x[2 * z + 1]);
+        ((uint4 *)out)[k] = *(const uint4 *)o2;
+    }
+}
+
 __host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : 256)); }
 
 } // namespace
 
-constexpr int TC_STRIP = 8;                 // rows of one work unit
-constexpr int TC_RING = 5;                  // ring slots of input rows
-// ring of 5 input rows, plus 2 shifted pole rows for the input gradient
-__host__ __device__ constexpr int tc_slots(bool dgrad) { return dgrad ? TC_RING + 2 : TC_RING; }
+// ---------------------------------------------------------------------------
+// forward and input-gradient convolution
+// ---------------------------------------------------------------------------
+// what the epilogue makes of an output row
+enum Epi : int {
+    EP_ACT,       // bias, ReLU, BF16
+    EP_ACT_POOL,  // the same, and the 2x2 mean of two rows for the next level
+    EP_Y,         // the network's output: channel 0 plus bias, FP32
+    EP_MASK,      // zero where mask <= 0 (ReLU derivative), BF16
+    EP_F32,       // FP32
+    EP_UP         // input gradient of [up(coarse), skip]: the first UP_C channels
+                  // summed over 2x2 points, zero where the coarse activation is
+                  // <= 0, BF16; the others FP32
+};
+constexpr int UP_C = 64;                    // channels of the coarse level in both concatenations
 
-template <int CIN, int COUT, bool DGRAD>
-__global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int *err)
+// ring slots of input rows, as many as fit beside the weights, at most 8
+template <int CIN, int COUT>
+struct ConvShape {
+    static constexpr int KC = CIN / 8;                            // 16-byte channel chunks of a point
+    static constexpr size_t WB = (size_t)9 * KC * COUT * 16;      // weights
+    static constexpr size_t SLOT = (size_t)KC * TC_P * 16;        // one staged row
+    static constexpr int FIT = (int)((215 * 1024 - WB) / SLOT);
+    static constexpr int RING = FIT > 8 ? 8 : FIT;
+    static constexpr size_t BYTES = WB + RING * SLOT;
+    // rows whose copies stay in flight behind the newest one's
+    static constexpr int DEPTH = RING >= 6 ? 4 : RING - 2;
+    static constexpr unsigned TCOLS = tmem_cols(COUT);            // columns of one accumulator
+    // groups of four epilogue warps: with 64 or more channels a row's stores
+    // and sums are more than four warps do beside the MMAs
+    static constexpr int EG = COUT >= 64 ? 2 : 1;
+    static constexpr int THREADS = 128 * EG + 160;                // epilogue, 4 producer warps, 1 MMA warp
+    // two blocks per SM where shared memory (with the static part and what the
+    // system keeps) and the epilogue's registers allow
+    static constexpr int MINB = 2 * (BYTES + 3072) <= 227 * 1024 && COUT <= 32 ? 2 : 1;
+};
+constexpr int ACCS = 4;                     // accumulators: three rows in progress, one read out
+
+// What bounds it: with one set of 128 threads that staged, issued and read out
+// in turn, a 128-point row of c5 (96 -> 32) took 4 us, of which the MMAs need
+// 0.9 (each reads a 4 KB A operand from shared memory) and the row's bytes
+// 0.6; the rest was one row's copies, MMAs and stores waiting for each other.
+// So the three jobs run in warps of their own, handing rows on through
+// mbarriers.  Producers copy input rows into a ring (cp.async), several rows
+// in flight.  One thread takes an input row as soon as it is there and issues
+// everything that reads it: kernel row ky of the weights adds it to output row
+// r + 1 - ky, so three output rows are in progress in TMEM, an input row's slot
+// is free after its own 9 CIN / 16 MMAs, and the whole ring but one slot holds
+// rows to come (which is what 128 input channels need: beside their weights
+// only four rows fit).  The epilogue warps read a finished accumulator while
+// the next rows run.  A block takes the COUT output channels of blockIdx.y;
+// with CS > 0 the first CS input channels come from the coarser level (nearest
+// neighbour) and the others from a second field, so the concatenation is never
+// stored.  us at 32 samples of 256 x 128, before (with the pooling, the
+// concatenation or its adjoint that is now part of the kernel) and now: c1 96,
+// 42; c2 59, 31; c4 354, 86; c5 298, 111; c6 84, 38; d6 96, 47; d5 481, 96; d4
+// 285, 85; d2 87, 35.  An N = 32 MMA takes 38 ns in c5, about twice its operands'
+// shared-memory time: the MMAs bound c4, c5 and d4, the bytes c1, c6 and d6.
+template <int CIN, int CS, int COUT, bool DGRAD, int EPI>
+__global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, COUT>::MINB) k_conv_tc(ConvArgs a, int strip, int *err)
 {
-    constexpr int KC = CIN / 8;                 // 16-byte channel chunks of an input point
-    constexpr unsigned TCOLS = tmem_cols(COUT);
+    typedef ConvShape<CIN, COUT> S;
+    constexpr int KC = S::KC, RING = S::RING, DEPTH = S::DEPTH, SLOT = (int)S::SLOT;
+    static_assert(RING >= DEPTH + 2, "a slot is freed once its row, handed over, is done");
+    static_assert(COUT % 16 == 0 && ACCS * S::TCOLS <= 512, "");
+    constexpr unsigned TCOLS = S::TCOLS;
     constexpr unsigned ID = idesc_bf16(TC_TW, COUT);
-    constexpr int SLOT = KC * TC_P * 16;        // bytes of one staged row
+    constexpr int EG = S::EG;
+    constexpr int CHUNK = EG > 1 || COUT < 32 ? 16 : 32;    // columns read out at once
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char *Ws = smem;                                         // [9][KC][COUT] x 16 B
-    unsigned char *Xs = Ws + (size_t)9 * KC * COUT * 16;              // [slot][KC][TC_P] x 16 B
-    __shared__ __align__(8) unsigned long long s_mbar[2];
+    unsigned char *Ws = smem;                       // [9][KC][COUT] x 16 B
+    unsigned char *Xs = Ws + S::WB;                 // [slot][KC][TC_P] x 16 B
+    __shared__ __align__(8) unsigned long long s_full[RING], s_empty[RING], s_accf[ACCS], s_acce[ACCS], s_done;
     __shared__ unsigned s_tmem;
     __shared__ int s_bad;
     __shared__ float s_bias[COUT];
     const int H = a.H, W = a.W;
     const int nseg = W / TC_TW;
-    const int nstrip = (H + TC_STRIP - 1) / TC_STRIP;
+    const int nstrip = (H + strip - 1) / strip;
     const long nunits = (long)a.B * nseg * nstrip;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+    const int n0 = blockIdx.y * COUT, ntot = gridDim.y * COUT;
 
     if (threadIdx.x == 0) {
         s_bad = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[0])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[1])) : "memory");
+        for (int q = 0; q < RING; ++q) {
+            mbar_init(&s_full[q], 128);
+            mbar_init(&s_empty[q], 1);
+        }
+        for (int q = 0; q < ACCS; ++q) {
+            mbar_init(&s_accf[q], 1);
+            mbar_init(&s_acce[q], 128 * EG);
+        }
+        mbar_init(&s_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        // two accumulators: the tensor core fills one while the other is read out
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
-                     "r"(2 * TCOLS)
+                     "r"(ACCS * TCOLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     for (int q = threadIdx.x; q < 9 * COUT * KC; q += blockDim.x) {
         const int c = q % KC, o = (q / KC) % COUT, tap = q / KC / COUT;
-        cp16(Ws + ((size_t)(tap * KC + c) * COUT + o) * 16, a.w + ((size_t)tap * COUT + o) * CIN + c * 8);
+        cp16(Ws + ((size_t)(tap * KC + c) * COUT + o) * 16, a.w + ((size_t)tap * ntot + n0 + o) * CIN + c * 8);
     }
-    for (int q = threadIdx.x; q < COUT; q += blockDim.x) s_bias[q] = a.bias ? a.bias[q] : 0.f;
+    for (int q = threadIdx.x; q < COUT; q += blockDim.x) s_bias[q] = a.bias ? a.bias[n0 + q] : 0.f;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = s_tmem;
-    unsigned par[2] = {0, 0};
+    volatile int *bad = &s_bad;
+    // a unit is `strip` output rows of one 128-point column of one sample.  Its
+    // ring entries, in order: forward, the input rows h0 - 1 .. h1 (beyond a
+    // pole, the pole row shifted by half a circle); gradient, the rows among
+    // them that exist, after the shifted pole row of the first strip and before
+    // that of the last.  Entry numbers run on over the block's units.
+    struct Unit { int b, w0, h0, h1, r0, south, north, nent; };
+    auto unit_of = [&](long u) {
+        Unit q;
+        q.w0 = (int)(u % nseg) * TC_TW;
+        q.h0 = (int)((u / nseg) % nstrip) * strip;
+        q.b = (int)(u / nseg / nstrip);
+        q.h1 = min(q.h0 + strip, H);
+        q.south = (DGRAD && q.h0 == 0) ? 1 : 0;
+        q.north = (DGRAD && q.h1 == H) ? 1 : 0;
+        q.r0 = q.h0 - 1 + q.south;                               // first row entry
+        q.nent = q.south + (q.h1 - q.north - q.r0 + 1) + q.north;
+        return q;
+    };
 
-    // stage input row hs (with halo; shift: across-pole ghost) into a slot;
-    // rows outside 0..H-1 give the sphere halo (forward) or zero (DGRAD)
-    auto stage = [&](int slot, int b, int w0, int hr, bool pole_shift) {
-        int hs = hr, shift = pole_shift ? W / 2 : 0;
-        bool zero = false;
-        if (!pole_shift && (hs < 0 || hs >= H)) {
-            if (DGRAD) zero = true;
-            else { hs = hs < 0 ? 0 : H - 1; shift = W / 2; }
-        }
-        unsigned char *base = Xs + (size_t)slot * SLOT;
-        for (int q = threadIdx.x; q < TC_P * KC; q += blockDim.x) {
-            const int c = q % KC, pt = q / KC;
-            unsigned char *dst = base + ((size_t)c * TC_P + pt) * 16;
-            if (zero) {
-                *(uint4 *)dst = make_uint4(0, 0, 0, 0);
-            } else {
-                int ws = (w0 - 1 + pt + shift) % W;
+    if (warp >= 4 * EG && warp < 4 * EG + 4) {
+        // ---- producers ----
+        // a thread's pieces (16 bytes, channel chunk c of point pt) are the same
+        // in every row: their places in the slot and in a row are kept
+        const int p = threadIdx.x - 128 * EG;
+        constexpr int NP = (TC_P * KC + 127) / 128;
+        int src[NP], cur_w0 = -1, cur_shift = 0;
+        auto place = [&](int w0, int shift) {    // offsets of the pieces in their source rows
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                const int z = p + 128 * k, c = z % KC;
+                int ws = w0 - 1 + z / KC + shift;
                 if (ws < 0) ws += W;
-                cp16(dst, a.x + (((size_t)b * H + hs) * W + ws) * CIN + c * 8);
+                else if (ws >= W) ws -= W;
+                src[k] = CS > 0 && c < CS / 8 ? (ws >> 1) * CS + c * 8 : ws * (CIN - CS) + (c - CS / 8) * 8;
+            }
+            cur_w0 = w0;
+            cur_shift = shift;
+        };
+        int e = 0, told = 0;
+        auto hand_over = [&](int upto) {         // entries [told, upto) are complete
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            for (; told < upto; ++told) mbar_arrive(&s_full[told % RING]);
+        };
+        for (long u = blockIdx.x; u < nunits && !*bad; u += gridDim.x) {
+            const Unit q = unit_of(u);
+            for (int k = 0; k < q.nent; ++k, ++e) {
+                const int slot = e % RING;
+                if (e >= RING && !mbar_wait(smem_u32(&s_empty[slot]), (e / RING - 1) & 1)) { *bad = 1; break; }
+                int hr = q.r0 + k - q.south, shift = 0;
+                if (DGRAD && (k < q.south || k - q.south > q.h1 - q.north - q.r0)) {
+                    hr = k < q.south ? 0 : H - 1;
+                    shift = W / 2;
+                } else if (hr < 0 || hr >= H) {
+                    hr = hr < 0 ? 0 : H - 1;
+                    shift = W / 2;
+                }
+                unsigned char *base = Xs + (size_t)slot * SLOT;
+                const __nv_bfloat16 *row = a.x + ((size_t)q.b * H + hr) * W * (CIN - CS);
+                const __nv_bfloat16 *crow =
+                    CS > 0 ? a.xc + ((size_t)q.b * (H / 2) + hr / 2) * (W / 2) * CS : nullptr;
+                if (q.w0 != cur_w0 || shift != cur_shift) place(q.w0, shift);
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                    const int z = p + 128 * k, c = z % KC;
+                    unsigned char *dst = base + (c * TC_P + z / KC) * 16;
+                    if (TC_P * KC % 128 != 0 && k == NP - 1 && z >= TC_P * KC) break;
+                    cp16(dst, (CS > 0 && c < CS / 8 ? crow : row) + src[k]);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                asm volatile("cp.async.wait_group %0;" ::"n"(DEPTH) : "memory");
+                if (e >= DEPTH) hand_over(e + 1 - DEPTH);
             }
         }
-    };
-    auto ready = [&]() {   // staged rows visible to the tensor core
         asm volatile("cp.async.wait_all;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    };
-    // read accumulator buf (row h of the unit) out of TMEM and store it
-    auto epilogue = [&](int buf, int b, int h, int w0) {
-        const int p = warp * 32 + lane;
-        const size_t pix = ((size_t)b * H + h) * W + w0 + p;
-        const unsigned trow = tmem + (unsigned)buf * TCOLS + ((unsigned)(warp * 32) << 16);
+        hand_over(e);
+    } else if (warp == 4 * EG + 4) {
+        // ---- MMAs ----
+        // the whole warp runs the role and one lane issues, so that everything
+        // but the issue is warp-uniform (a row of c5 took 3.1 us with one
+        // thread in a branch of its own)
+        {
+            const unsigned one = elect_one();
+            const unsigned long long A0 = sdesc(smem_u32(Xs), TC_P * 16, 128), B0 = sdesc(smem_u32(Ws), COUT * 16, 128);
+            int e = 0, t0 = 0;                      // ring entry; number of the unit's first output row
+            for (long u = blockIdx.x; u < nunits && !*bad; u += gridDim.x) {
+                const Unit q = unit_of(u);
+                unsigned begun = 0;                 // output rows (bit t % ACCS) that have been added to
+                // three taps of kernel row ky: slot's row into output row h
+                auto add = [&](int slot, int ky, int h) {
+                    const int t = t0 + h - q.h0, buf = t % ACCS;
+                    if (!(begun >> buf & 1) && t >= ACCS && !mbar_wait(smem_u32(&s_acce[buf]), (t / ACCS - 1) & 1))
+                        return false;
+                    if (!(begun >> buf & 1)) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const unsigned d = tmem + (unsigned)buf * TCOLS;
+                    unsigned acc = begun >> buf & 1;
 #pragma unroll
-        for (int c0 = 0; c0 < COUT; c0 += 8) {
-            float v[8];
-            tmem_ld8(trow + c0, v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    for (int kx = 0; kx < 3; ++kx) {
+                        const unsigned long long ad = A0 + (unsigned)(slot * (SLOT / 16) + kx);
+                        const unsigned long long bd = B0 + (unsigned)((ky * 3 + kx) * KC * COUT);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int co = c0 + q;
-                float x = v[q] + s_bias[co];
-                if (a.relu) x = fmaxf(x, 0.f);
-                if (a.mask && !(__bfloat162float(a.mask[pix * COUT + co]) > 0.f)) x = 0.f;
-                v[q] = x;
+                        for (int ks = 0; ks < CIN / 16; ++ks) {
+                            mma_bf16_one(d, ad + 2 * ks * TC_P, bd + 2 * ks * COUT, ID, acc, one);
+                            acc = 1;
+                        }
+                    }
+                    begun |= 1u << buf;
+                    return true;
+                };
+                auto finish = [&](int h) {          // output row h is complete
+                    const int buf = (t0 + h - q.h0) % ACCS;
+                    begun &= ~(1u << buf);
+                    mma_commit_one(smem_u32(&s_accf[buf]), one);
+                };
+                for (int k = 0; k < q.nent; ++k, ++e) {
+                    const int slot = e % RING;
+                    bool ok = mbar_wait(smem_u32(&s_full[slot]), (e / RING) & 1);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    // the adjoint of the ghost rows: the pole row collects what
+                    // the row beyond it had copied (kernel row 2 at the first
+                    // row, 0 at the last)
+                    if (DGRAD && k < q.south) {
+                        ok = ok && add(slot, 2, 0);
+                    } else if (DGRAD && q.north && k == q.nent - 1) {
+                        ok = ok && add(slot, 0, H - 1);
+                        finish(H - 1);
+                    } else {
+                        const int r = q.r0 + k - q.south;
+                        for (int ky = 2; ky >= 0; --ky) {
+                            const int h = r + 1 - ky;
+                            if (h >= q.h0 && h < q.h1) ok = ok && add(slot, ky, h);
+                        }
+                        if (r - 1 >= q.h0) finish(r - 1);
+                    }
+                    mma_commit_one(smem_u32(&s_empty[slot]), one);
+                    if (!ok) { *bad = 1; break; }
+                }
+                t0 += q.h1 - q.h0;
             }
-            if (a.yf) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (c0 + q < a.yf_c) a.yf[pix * a.yf_c + c0 + q] = v[q];
-            } else {
-                __nv_bfloat162 o2[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) o2[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
-                *(uint4 *)(a.y + pix * COUT + c0) = *(const uint4 *)o2;
-            }
+            // everything issued has completed before TMEM and the barriers go
+            mma_commit_one(smem_u32(&s_done), one);
+            if (!mbar_wait(smem_u32(&s_done), 0)) *bad = 1;
         }
-    };
-    auto wait_acc = [&](int buf) {
-        const bool okw = mbar_wait(smem_u32(&s_mbar[buf]), par[buf]);
-        par[buf] ^= 1;
-        if (!okw && lane == 0) atomicExch(&s_bad, 1);
-    };
-
-    for (long unit = blockIdx.x; unit < nunits && !s_bad; unit += gridDim.x) {
-        const int seg = (int)(unit % nseg);
-        const int strip = (int)((unit / nseg) % nstrip);
-        const int b = (int)(unit / nseg / nstrip);
-        const int w0 = seg * TC_TW;
-        const int h0 = strip * TC_STRIP, h1 = min(h0 + TC_STRIP, H);
-        // ring: input row hr lives in slot (hr + TC_RING) % TC_RING; the
-        // shifted pole rows (input gradient) in slots TC_RING and TC_RING + 1
-        auto slot_of = [](int hr) { return (hr + TC_RING) % TC_RING; };
-        for (int hr = h0 - 1; hr <= h0 + 1; ++hr) stage(slot_of(hr), b, w0, hr, false);
-        if (DGRAD && h0 == 0) stage(TC_RING, b, w0, 0, true);
-        if (DGRAD && h1 == H) stage(TC_RING + 1, b, w0, H - 1, true);
-        ready();
-        for (int h = h0; h < h1; ++h) {
-            const int buf = (h - h0) & 1;
-            // input row h+2 (for row h+1) goes into the slot that row h-3 held;
-            // the last MMAs to read it were row h-2's, complete since the
-            // previous iteration.  Its copy overlaps this iteration.
-            if (h + 2 <= h1) stage(slot_of(h + 2), b, w0, h + 2, false);
-            if (threadIdx.x == 0) {
-                const unsigned xs = smem_u32(Xs), ws0 = smem_u32(Ws);
-                const bool pole = DGRAD && (h == 0 || h == H - 1);
-                const int ntap = pole ? 12 : 9;
-                const unsigned d = tmem + (unsigned)buf * TCOLS;
-                unsigned acc = 0;
-                for (int t = 0; t < ntap; ++t) {
-                    int tap, slot;
-                    if (t < 9) { tap = t; slot = slot_of(h - 1 + t / 3); }
-                    else { tap = (h == 0 ? 6 : 0) + (t - 9); slot = h == 0 ? TC_RING : TC_RING + 1; }
-                    const int kx = tap % 3;
+        __syncwarp();
+    } else {
+        // ---- epilogue: thread = output point, warp w reads TMEM lanes 32 (w % 4)
+        // .. + 31, group w / 4 every EG-th chunk of columns ----
+        const int eg = warp / 4;
+        int t = 0;
+        // pair sums of the even row
+        float hold[EPI == EP_ACT_POOL || EPI == EP_UP ? (EPI == EP_UP && COUT > UP_C ? UP_C : COUT) / EG : 1];
+        for (long u = blockIdx.x; u < nunits && !*bad; u += gridDim.x) {
+            const Unit q = unit_of(u);
+            const int w = q.w0 + (warp & 3) * 32 + lane;
+            for (int h = q.h0; h < q.h1; ++h, ++t) {
+                const int buf = t % ACCS;
+                if (!mbar_wait(smem_u32(&s_accf[buf]), (t / ACCS) & 1)) *bad = 1;
+                if (__any_sync(0xffffffffu, *bad)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const unsigned trow = tmem + (unsigned)buf * TCOLS + ((unsigned)((warp & 3) * 32) << 16);
+                const size_t pix = ((size_t)q.b * H + h) * W + w;
+                const size_t cpix = ((size_t)q.b * (H / 2) + h / 2) * (W / 2) + w / 2;
 #pragma unroll
-                    for (int ks = 0; ks < CIN / 16; ++ks) {
-                        const unsigned aa = xs + (unsigned)slot * SLOT + ((unsigned)(2 * ks) * TC_P + kx) * 16;
-                        const unsigned ba = ws0 + (unsigned)(tap * KC + 2 * ks) * COUT * 16;
-                        mma_bf16(d, sdesc(aa, TC_P * 16, 128), sdesc(ba, COUT * 16, 128), ID, acc);
-                        acc = 1;
+                for (int ci = 0; ci < COUT / CHUNK; ci += EG) {
+                    const int c0 = (ci + eg) * CHUNK, hc = ci / EG * CHUNK;
+                    float v[CHUNK];
+#pragma unroll
+                    for (int k = 0; k < CHUNK; k += 16) {
+                        if (EPI == EP_Y) { tmem_ld8(trow, *(float (*)[8])v); break; }
+                        tmem_ld16(trow + c0 + k, v + k);
+                    }
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (ci + EG >= COUT / CHUNK) {
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        mbar_arrive(&s_acce[buf]);
+                    }
+                    if constexpr (EPI == EP_Y) {
+                        a.yf[pix] = v[0] + s_bias[0];
+                    } else if constexpr (EPI == EP_F32) {
+                        float4 *o = (float4 *)(a.yf + pix * ntot + n0 + c0);
+#pragma unroll
+                        for (int k = 0; k < CHUNK / 4; ++k)
+                            o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                    } else if constexpr (EPI == EP_UP) {
+                        const int col = n0 + c0;
+                        if (ci * CHUNK >= UP_C || col >= UP_C) {
+                            float4 *o = (float4 *)(a.yf + pix * (ntot - UP_C) + col - UP_C);
+#pragma unroll
+                            for (int k = 0; k < CHUNK / 4; ++k)
+                                o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < CHUNK; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 1);
+                            if ((h & 1) == 0) {
+#pragma unroll
+                                for (int k = 0; k < CHUNK; ++k) hold[hc + k] = v[k];
+                            } else {
+                                // each point of the pair writes half of the channels
+#pragma unroll
+                                for (int k = 0; k < CHUNK; ++k) v[k] = hold[hc + k] + v[k];
+                                const size_t at = cpix * UP_C + col + (lane & 1) * (CHUNK / 2);
+                                store_half(v, lane & 1, a.mask + at, a.y + at);
+                            }
+                        }
+                    } else {
+                        if constexpr (EPI == EP_MASK) {
+                            const uint4 *m = (const uint4 *)(a.mask + pix * ntot + n0 + c0);
+#pragma unroll
+                            for (int k = 0; k < CHUNK / 8; ++k) {
+                                const uint4 mq = __ldg(m + k);
+                                const __nv_bfloat16 *mv = (const __nv_bfloat16 *)&mq;
+#pragma unroll
+                                for (int z = 0; z < 8; ++z)
+                                    if (!(__bfloat162float(mv[z]) > 0.f)) v[8 * k + z] = 0.f;
+                            }
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < CHUNK; ++k) v[k] = fmaxf(v[k] + s_bias[c0 + k], 0.f);
+                        }
+                        uint4 *o = (uint4 *)(a.y + pix * ntot + n0 + c0);
+#pragma unroll
+                        for (int k = 0; k < CHUNK / 8; ++k) {
+                            __nv_bfloat162 o2[4];
+#pragma unroll
+                            for (int z = 0; z < 4; ++z) o2[z] = __floats2bfloat162_rn(v[8 * k + 2 * z], v[8 * k + 2 * z + 1]);
+                            o[k] = *(const uint4 *)o2;
+                        }
+                        if constexpr (EPI == EP_ACT_POOL) {
+                            // the mean is of the activations as stored
+#pragma unroll
+                            for (int k = 0; k < CHUNK; ++k) {
+                                v[k] = __bfloat162float(__float2bfloat16_rn(v[k]));
+                                v[k] += __shfl_xor_sync(0xffffffffu, v[k], 1);
+                            }
+                            if ((h & 1) == 0) {
+#pragma unroll
+                                for (int k = 0; k < CHUNK; ++k) hold[hc + k] = v[k];
+                            } else {
+#pragma unroll
+                                for (int k = 0; k < CHUNK; ++k) v[k] = 0.25f * (hold[hc + k] + v[k]);
+                                const size_t at = cpix * ntot + n0 + c0 + (lane & 1) * (CHUNK / 2);
+                                store_half(v, lane & 1, nullptr, a.yp + at);
+                            }
+                        }
                     }
                 }
-                mma_commit(smem_u32(&s_mbar[buf]));
             }
-            __syncwarp();
-            if (h > h0) {
-                // row h-1: its MMAs are done once its barrier phase completes
-                wait_acc(buf ^ 1);
-                __syncthreads();
-                if (s_bad) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                epilogue(buf ^ 1, b, h - 1, w0);
-            }
-            ready();      // row h+2 staged; accumulator buf ^ 1 free for row h+1
         }
-        if (s_bad) break;
-        // the unit's last row
-        wait_acc((h1 - 1 - h0) & 1);
-        __syncthreads();
-        if (s_bad) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        epilogue((h1 - 1 - h0) & 1, b, h1 - 1, w0);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
-    if (s_bad && threadIdx.x == 0) {
-        // a tensor-core wait ran out: flag it, and give outstanding work a
-        // bounded chance to drain before TMEM is freed
-        atomicExch(err, 1);
-        mbar_wait(smem_u32(&s_mbar[0]), par[0]);
-        mbar_wait(smem_u32(&s_mbar[1]), par[1]);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (s_bad && threadIdx.x == 0) atomicExch(err, 1);
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TCOLS)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ACCS * TCOLS)
                      : "memory");
 }
 
-// ---------------------------------------------------------------------------
-template <int CIN, int COUT, bool DGRAD>
-static size_t tc_smem()
+template <int CIN, int CS, int COUT, bool DGRAD, int EPI>
+static cudaError_t conv_tc_t(const ConvArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
 {
-    return (size_t)9 * (CIN / 8) * COUT * 16 + (size_t)tc_slots(DGRAD) * (CIN / 8) * TC_P * 16;
-}
-
-template <int CIN, int COUT, bool DGRAD>
-static cudaError_t conv_tc_t(const ConvArgs &a, int sms, int *err, cudaStream_t s)
-{
-    const size_t smem = tc_smem<CIN, COUT, DGRAD>();
+    typedef ConvShape<CIN, COUT> S;
+    const size_t smem = S::BYTES;
     int bps = 0;
-    cudaError_t e = occupancy_once<k_conv_tc<CIN, COUT, DGRAD>>(128, smem, &bps);
+    cudaError_t e = occupancy_once<k_conv_tc<CIN, CS, COUT, DGRAD, EPI>>(S::THREADS, smem, &bps);
     if (e != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
-    // TMEM: 512 columns per SM shared by the resident blocks
-    const int per = 2 * tmem_cols(COUT);
-    if (bps * per > 512) bps = 512 / per;
-    const long nunits = (long)a.B * (a.W / TC_TW) * ((a.H + TC_STRIP - 1) / TC_STRIP);
-    long grid = (long)bps * sms;
-    if (grid > nunits) grid = nunits;
-    k_conv_tc<CIN, COUT, DGRAD><<<(int)grid, 128, smem, s>>>(a, err);
+    // (the occupancy query answers 1 for every kernel that allocates TMEM)
+    bps = S::MINB;
+    static_assert(S::MINB * ACCS * S::TCOLS <= 512, "");
+    // strips of 8 rows (10 input rows each), shorter while blocks would be idle
+    const long cap = (long)bps * sms / nsplit > 0 ? (long)bps * sms / nsplit : 1;
+    int strip = 8;
+    auto units = [&](int st) { return (long)a.B * (a.W / TC_TW) * ((a.H + st - 1) / st); };
+    while (strip > 2 && units(strip) < cap) strip /= 2;
+    const long n = units(strip);
+    k_conv_tc<CIN, CS, COUT, DGRAD, EPI><<<dim3((unsigned)(n < cap ? n : cap), nsplit), S::THREADS, smem, s>>>(a, strip, err);
     return cudaGetLastError();
 }
 
-// true when the tcgen05 kernel takes this convolution: rows of a multiple of
-// 128 points, operands within shared memory, and a layer where it measured
-// faster than the mma.sync kernel (the forward layers with 32 or more input
-// channels; with few MMAs per row, or a per-point FP32 store of many
-// channels, the fixed cost per row dominates)
-bool conv_tc_supported(int cin, int cout, bool dgrad, int W)
+cudaError_t launch_conv_tc(ConvStep step, const ConvArgs &a, int sms, int *err, cudaStream_t s)
 {
-    if (W % TC_TW || dgrad || cin < 32 || cout < 32) return false;
-    const size_t smem = (size_t)9 * (cin / 8) * cout * 16 + (size_t)tc_slots(dgrad) * (cin / 8) * TC_P * 16;
-    if (smem > 227 * 1024) return false;
-#define NN_TC(CI, CO) if (cin == CI && cout == CO) return true;
-    NN_TC(16, 32) NN_TC(32, 64) NN_TC(96, 32) NN_TC(32, 16) NN_TC(64, 32) NN_TC(64, 128) NN_TC(32, 96)
-    NN_TC(64, 64) NN_TC(128, 64)
-#undef NN_TC
-    return false;
-}
-
-cudaError_t launch_conv_tc(int cin, int cout, bool dgrad, const ConvArgs &a, int sms, int *err, cudaStream_t s)
-{
-#define NN_TC(CI, CO)                                                                            \
-    if (cin == CI && cout == CO)                                                                 \
-        return dgrad ? conv_tc_t<CI, CO, true>(a, sms, err, s) : conv_tc_t<CI, CO, false>(a, sms, err, s);
-    NN_TC(16, 32) NN_TC(32, 64) NN_TC(96, 32) NN_TC(32, 16) NN_TC(64, 32) NN_TC(64, 128) NN_TC(32, 96)
-    NN_TC(64, 64) NN_TC(128, 64)
-#undef NN_TC
+    switch (step) {
+    case CONV_C1: return conv_tc_t<16, 0, 32, false, EP_ACT_POOL>(a, 1, sms, err, s);
+    case CONV_C2: return conv_tc_t<32, 0, 64, false, EP_ACT_POOL>(a, 1, sms, err, s);
+    case CONV_C3: return conv_tc_t<64, 0, 64, false, EP_ACT>(a, 1, sms, err, s);
+    // 128 input channels: 147 KB of weights for 64 outputs, so 32 a block
+    case CONV_C4: return conv_tc_t<128, 64, 32, false, EP_ACT>(a, 2, sms, err, s);
+    case CONV_C5: return conv_tc_t<96, 64, 32, false, EP_ACT>(a, 1, sms, err, s);
+    case CONV_C6: return conv_tc_t<32, 0, 16, false, EP_Y>(a, 1, sms, err, s);
+    case CONV_D6: return conv_tc_t<16, 0, 32, true, EP_MASK>(a, 1, sms, err, s);
+    case CONV_D5: return conv_tc_t<32, 0, 96, true, EP_UP>(a, 1, sms, err, s);
+    case CONV_D4: return conv_tc_t<64, 0, 64, true, EP_UP>(a, 2, sms, err, s);
+    case CONV_D3: return conv_tc_t<64, 0, 64, true, EP_F32>(a, 1, sms, err, s);
+    case CONV_D2: return conv_tc_t<64, 0, 32, true, EP_F32>(a, 1, sms, err, s);
+    }
     return cudaErrorInvalidValue;
 }
 
@@ -396,7 +637,7 @@ struct WgShape {
     static constexpr unsigned NCOL = 3 * KYS * COUT;
 };
 
-template <int CIN, int COUT, int KYS>
+template <int CIN, int CS, int COUT, int KYS>
 __global__ void __launch_bounds__(128) k_wgrad_tc(WgradArgs a, int *err)
 {
     typedef WgShape<CIN, COUT, KYS> S;
@@ -448,7 +689,10 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(WgradArgs a, int *err)
             const int c = q % S::KC, pt = q / S::KC;
             int ws = (w0 - 1 + pt + shift) % W;
             if (ws < 0) ws += W;
-            cp16(xs + ((size_t)c * TC_P + pt) * 16, a.x + (((size_t)b * H + hs) * W + ws) * CIN + c * 8);
+            const size_t px = ((size_t)b * H + hs) * W + ws;
+            const size_t pc = ((size_t)b * (H / 2) + hs / 2) * (W / 2) + ws / 2;
+            cp16(xs + ((size_t)c * TC_P + pt) * 16,
+                 c < CS / 8 ? a.xc + pc * CS + c * 8 : a.x + px * (CIN - CS) + (c - CS / 8) * 8);
         }
     };
     auto stage_g = [&](int b, int w0, int h) {
@@ -570,25 +814,26 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(WgradArgs a, int *err)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
 }
 
-template <int CIN, int COUT, int KYS>
+template <int CIN, int CS, int COUT, int KYS>
 static cudaError_t wgrad_tc_t(const WgradArgs &a, int sms, int *err, cudaStream_t s)
 {
     typedef WgShape<CIN, COUT, KYS> S;
     const size_t smem = S::BYTES;
-    cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<CIN, COUT, KYS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<CIN, CS, COUT, KYS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
     constexpr int NKG = 3 / KYS;
     const long nunits = (long)a.B * (a.W / TC_TW) * ((a.H + WG_STRIP - 1) / WG_STRIP);
     long nsplit = sms / NKG > 0 ? sms / NKG : 1;   // about one block per SM
     if (nsplit > nunits) nsplit = nunits;
-    k_wgrad_tc<CIN, COUT, KYS><<<(int)(NKG * nsplit), 128, smem, s>>>(a, err);
+    k_wgrad_tc<CIN, CS, COUT, KYS><<<(int)(NKG * nsplit), 128, smem, s>>>(a, err);
     return cudaGetLastError();
 }
 
 // the layers whose weight gradient takes tcgen05: c5 (96 -> 32, all nine taps
 // in one block, 288 TMEM columns) and c4 (128 -> 64, a kernel row per block,
-// 192 columns), rows of a multiple of 128 points
+// 192 columns), rows of a multiple of 128 points; both read their input from
+// the coarser level and the skip connection, like the forward pass
 bool wgrad_tc_supported(int cin, int cout, int W)
 {
     return W % TC_TW == 0 && ((cin == 96 && cout == 32) || (cin == 128 && cout == 64));
@@ -596,8 +841,8 @@ bool wgrad_tc_supported(int cin, int cout, int W)
 
 cudaError_t launch_wgrad_tc(int cin, int cout, const WgradArgs &a, int sms, int *err, cudaStream_t s)
 {
-    if (cin == 96 && cout == 32) return wgrad_tc_t<96, 32, 3>(a, sms, err, s);
-    if (cin == 128 && cout == 64) return wgrad_tc_t<128, 64, 1>(a, sms, err, s);
+    if (cin == 96 && cout == 32) return wgrad_tc_t<96, 64, 32, 3>(a, sms, err, s);
+    if (cin == 128 && cout == 64) return wgrad_tc_t<128, 64, 64, 1>(a, sms, err, s);
     return cudaErrorInvalidValue;
 }
 
