@@ -83,13 +83,11 @@ enum ConvStep : int {
 inline bool conv_tc_rows(int W) { return W % 128 == 0; }
 cudaError_t launch_conv_tc(ConvStep step, const ConvArgs &a, int sms, int *err, cudaStream_t s);
 cudaError_t launch_wgrad(int cin, int cout, const WgradArgs &a, int sms, cudaStream_t s);
-// the weight gradient on tcgen05 (nn_tc.cu) for the layers it takes
-bool wgrad_tc_supported(int cin, int cout, int W);
+// the weight gradient on tcgen05 (nn_tc.cu), rows of a multiple of 128 points
 cudaError_t launch_wgrad_tc(int cin, int cout, const WgradArgs &a, int sms, int *err, cudaStream_t s);
 inline cudaError_t launch_wgrad_auto(int cin, int cout, const WgradArgs &a, int sms, int *err, cudaStream_t s)
 {
-    return wgrad_tc_supported(cin, cout, a.W) ? launch_wgrad_tc(cin, cout, a, sms, err, s)
-                                              : launch_wgrad(cin, cout, a, sms, s);
+    return conv_tc_rows(a.W) ? launch_wgrad_tc(cin, cout, a, sms, err, s) : launch_wgrad(cin, cout, a, sms, s);
 }
 
 // elementwise and small kernels (nn_ops.cu); shapes are of the fine level

@@ -61,17 +61,7 @@ __host__ __device__ constexpr unsigned idesc_bf16(int M, int N)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(unsigned dtmem, unsigned long long a, unsigned long long b, unsigned id,
-                                         unsigned accumulate)
-{
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-        "l"(a), "l"(b), "r"(id), "r"(accumulate)
-        : "memory");
-}
-
-// the same, issued by the lane with one != 0 of a warp that runs together: the
+// one MMA, issued by the lane with one != 0 of a warp that runs together: the
 // descriptors are then warp-uniform values
 __device__ __forceinline__ void mma_bf16_one(unsigned dtmem, unsigned long long a, unsigned long long b, unsigned id,
                                              unsigned accumulate, unsigned one)
@@ -98,12 +88,6 @@ __device__ __forceinline__ unsigned elect_one()
     unsigned one;
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(one));
     return one;
-}
-
-__device__ __forceinline__ void mma_commit(unsigned mbar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-                 : "memory");
 }
 
 // wait for the mbarrier phase of the given parity; false after TC_WAIT_NS
@@ -183,7 +167,7 @@ __device__ __forceinline__ void store_half(const float (&v)[N], int hi, const __
     }
 }
 
-__host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : 256)); }
+__host__ __device__ constexpr int tmem_cols(int n) { return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : (n <= 256 ? 256 : 512))); }
 
 } // namespace
 
@@ -600,68 +584,81 @@ cudaError_t launch_conv_tc(ConvStep step, const ConvArgs &a, int sms, int *err, 
 }
 
 // ---------------------------------------------------------------------------
-// weight gradient on tcgen05
+// weight gradient
 // ---------------------------------------------------------------------------
-// dW[ky][kx][co][ci] = sum over points p of x[row h + ky - 1][p + kx - 1][ci]
-// g[row h][p][co], with the forward convolution's sphere halo.  As a GEMM
-// D[m][n] = sum_k A[m][k] B[n][k]: m = ci (M = 128), n = co (N = COUT) for
-// each tap, k = points.  The operands sit in shared memory in the layout the
-// forward kernel stages (one plane per 8 channels, a 16-byte row per point),
-// which for this GEMM is the MN-major no-swizzle layout (8 consecutive MN
-// elements per 16-byte row, 8 rows per K core matrix): both are read with
-// the transpose bits of the instruction descriptor set, and a longitude tap
-// shift is a 16-byte start offset.  With fewer than 128 input channels the A
-// operand's upper rows read the next ring slot: those rows of D are never
-// read out.
+// dW[ky][kx][co][ci] = sum over points p of x[row h + ky - 1][p] g[row h][p - kx + 1][co]
+// with the forward convolution's sphere halo on x (beyond a pole the pole row
+// shifted by half a circle; periodic in longitude).  As a GEMM D[m][n] = sum_k
+// A[m][k] B[n][k]: m = input channels of one or more consecutive input rows
+// (M = 128), n = co (N = COUT) for each kx, k = points.  Both operands sit in
+// shared memory one plane per 8 channels, a 16-byte row per point: the MN-major
+// no-swizzle layout (8 consecutive MN elements per 16-byte row, 8 rows per K
+// core matrix), read with the transpose bits of the instruction descriptor.
+// The longitude shift of a tap is a 16-byte start offset, and it is on g, the
+// smaller operand: an A read that does not start on a core matrix costs twice.
 //
-// A block works down a strip of WG_STRIP output rows of one 128-point column
-// and accumulates KYS kernel rows (3 KYS taps, 3 KYS COUT TMEM columns) over
-// all of its strips; only at the end are the accumulators read out of TMEM
-// and added to dW.  Input rows sit in a ring (each staged once per strip) and
-// gradient rows in a second one, WG_AHEAD rows ahead of the MMAs; every row's
-// MMAs are committed to one of three mbarriers, and a ring slot is restaged
-// only after the MMAs of the last row that reads it are complete.  Every wait
-// is bounded.
-constexpr int WG_STRIP = 8;     // output rows of one work unit
-constexpr int WG_AHEAD = 2;     // rows staged ahead of the MMAs
-
-template <int CIN, int COUT, int KYS>
+// Input rows sit in a ring of slots that follow one another in memory, so that
+// with fewer than 128 input channels one A operand spans the rows of several
+// ky: all three with 16 or 32 channels, two with 64 (the rows of D beyond the
+// third are never read out).  The first slots are kept twice, behind the last
+// one, for rows that wrap.
+//
+// What bounds it: one set of 128 threads that staged, issued and waited in turn
+// took 4.8 us per 128-point row of c5 (its 72 MMAs need about 2), and mma.sync
+// with nothing in flight 180 us for the padded c6.  The jobs run in warps of
+// their own, as in k_conv_tc: producers stage a step (an input row and a
+// gradient row) at a time, several in flight; one warp issues a step's MMAs into
+// the 3 COUT columns of each group of rows, accumulated over all of the block's
+// steps; the four warps that read the result out at the end add up the bias
+// gradient meanwhile.  us at 32 samples of 256 x 128, before and now:
+// c1 143, 59; c2 56, 29; c4 178, 112; c5 260, 123; c6 180, 50.
+template <int CIN, int COUT>
 struct WgShape {
     static constexpr int KC = CIN / 8, GC = COUT / 8;
-    static constexpr int XR = WG_AHEAD + KYS + 1;                  // input-row ring slots
-    static constexpr int GR = WG_AHEAD + 2;                        // gradient-row ring slots
-    static constexpr size_t XSLOT = (size_t)KC * TC_P * 16;
-    static constexpr size_t XPAD = (size_t)(16 - KC) * TC_P * 16;  // the last slot's 16-plane read
-    static constexpr size_t GSLOT = (size_t)GC * TC_TW * 16;
-    static constexpr size_t BYTES = XR * XSLOT + XPAD + GR * GSLOT;
-    static constexpr unsigned NCOL = 3 * KYS * COUT;
+    static constexpr int RPG = 128 / CIN > 3 ? 3 : 128 / CIN;      // kernel rows of one A operand
+    static constexpr int NG = (3 + RPG - 1) / RPG;                 // A operands per step
+    static constexpr int MIR = RPG - 1;                            // slots kept twice
+    static constexpr size_t XSLOT = (size_t)KC * TC_TW * 16;
+    static constexpr size_t GSLOT = (size_t)GC * TC_P * 16;
+    static constexpr int GR = 5;                                   // gradient-row slots
+    // the last slot's A operand reads 16 planes
+    static constexpr size_t PAD = (size_t)(16 - KC) * TC_TW * 16;
+    static constexpr int FIT = (int)((222 * 1024 - GR * GSLOT - PAD) / XSLOT) - MIR;
+    static constexpr int XR = FIT > 8 ? 8 : FIT;                   // input-row slots
+    static constexpr size_t XBYTES = (XR + MIR) * XSLOT + PAD;
+    static constexpr size_t BYTES = XBYTES + GR * GSLOT;
+    static constexpr int DEPTH = 2;                                // steps in flight behind the newest one
+    static constexpr int NCOL = NG * 3 * COUT;
 };
 
-template <int CIN, int CS, int COUT, int KYS>
-__global__ void __launch_bounds__(128) k_wgrad_tc(WgradArgs a, int *err)
+template <int CIN, int CS, int COUT>
+__global__ void __launch_bounds__(288) k_wgrad_tc(WgradArgs a, int strip, int *err)
 {
-    typedef WgShape<CIN, COUT, KYS> S;
+    typedef WgShape<CIN, COUT> S;
+    constexpr int KC = S::KC, GC = S::GC, XR = S::XR, GR = S::GR, DEPTH = S::DEPTH;
+    static_assert(XR >= 4 && S::NCOL <= 512 && DEPTH < GR, "");
     constexpr unsigned TCOLS = tmem_cols(S::NCOL);
     // BF16 A and B, both MN-major (transpose bits 15 and 16), FP32 accumulator
     constexpr unsigned ID = idesc_bf16(TC_TW, COUT) | (1u << 15) | (1u << 16);
-    constexpr int NKG = 3 / KYS;                       // groups of kernel rows
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char *Xs = smem, *Gs = smem + S::XR * S::XSLOT + S::XPAD;
-    __shared__ __align__(8) unsigned long long s_mbar[3];
+    unsigned char *Xs = smem, *Gs = smem + S::XBYTES;
+    __shared__ __align__(8) unsigned long long s_full[GR], s_empty[GR], s_done;
     __shared__ unsigned s_tmem;
     __shared__ int s_bad;
     const int H = a.H, W = a.W;
-    const int nseg = W / TC_TW, nstrip = (H + WG_STRIP - 1) / WG_STRIP;
+    const int nseg = W / TC_TW, nstrip = (H + strip - 1) / strip;
     const long nunits = (long)a.B * nseg * nstrip;
-    const int ky0 = (blockIdx.x % NKG) * KYS;
-    const int split = blockIdx.x / NKG, nsplit = gridDim.x / NKG;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool do_bias = a.db && ky0 == 0;
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+    const int n0 = blockIdx.y * COUT, ntot = gridDim.y * COUT;
 
     if (threadIdx.x == 0) {
         s_bad = 0;
-        for (int q = 0; q < 3; ++q)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[q])) : "memory");
+        for (int q = 0; q < GR; ++q) {
+            mbar_init(&s_full[q], 128);
+            mbar_init(&s_empty[q], 5);      // the step's MMAs, and the four bias warps
+        }
+        mbar_init(&s_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
@@ -673,140 +670,190 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(WgradArgs a, int *err)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = s_tmem;
-    unsigned par[3] = {0, 0, 0};
-    bool pend[3] = {false, false, false};
+    volatile int *bad = &s_bad;
+    struct Unit { int b, w0, h0, h1; };
+    auto unit_of = [&](long u) {
+        Unit q;
+        q.w0 = (int)(u % nseg) * TC_TW;
+        q.h0 = (int)((u / nseg) % nstrip) * strip;
+        q.b = (int)(u / nseg / nstrip);
+        q.h1 = min(q.h0 + strip, H);
+        return q;
+    };
+    // step n of the block is one gradient row; input rows h0 - 1 .. h1 of a unit
+    // are entries of their ring, numbered on over the units, entry i of a unit
+    // last read by its step min(i, h1 - h0 - 1)
 
-    auto xslot = [&](int xr) { return Xs + (size_t)((xr + 2 * S::XR) % S::XR) * S::XSLOT; };
-    auto gslot = [&](int h) { return Gs + (size_t)(h % S::GR) * S::GSLOT; };
-    // input row xr (-1 .. H) with the sphere halo: beyond a pole, the pole row
-    // shifted by half a circle
-    auto stage_x = [&](int b, int w0, int xr) {
-        int hs = xr, shift = 0;
-        if (hs < 0) { hs = 0; shift = W / 2; }
-        else if (hs >= H) { hs = H - 1; shift = W / 2; }
-        unsigned char *xs = xslot(xr);
-        for (int q = threadIdx.x; q < TC_P * S::KC; q += blockDim.x) {
-            const int c = q % S::KC, pt = q / S::KC;
-            int ws = (w0 - 1 + pt + shift) % W;
-            if (ws < 0) ws += W;
-            const size_t px = ((size_t)b * H + hs) * W + ws;
-            const size_t pc = ((size_t)b * (H / 2) + hs / 2) * (W / 2) + ws / 2;
-            cp16(xs + ((size_t)c * TC_P + pt) * 16,
-                 c < CS / 8 ? a.xc + pc * CS + c * 8 : a.x + px * (CIN - CS) + (c - CS / 8) * 8);
-        }
-    };
-    auto stage_g = [&](int b, int w0, int h) {
-        unsigned char *gs = gslot(h);
-        for (int q = threadIdx.x; q < TC_TW * S::GC; q += blockDim.x) {
-            const int c = q % S::GC, pt = q / S::GC;
-            cp16(gs + ((size_t)c * TC_TW + pt) * 16, a.g + (((size_t)b * H + h) * W + w0 + pt) * COUT + c * 8);
-        }
-    };
-    // the MMAs committed to mbarrier q are complete
-    auto wait_row = [&](int q) {
-        if (!pend[q]) return;
-        const bool okw = mbar_wait(smem_u32(&s_mbar[q]), par[q]);
-        par[q] ^= 1;
-        pend[q] = false;
-        if (!okw && lane == 0) atomicExch(&s_bad, 1);
-    };
-
-    float bsum = 0.f;
-    unsigned acc = 0;
-    for (long u = split; u < nunits && !s_bad; u += nsplit) {
-        const int seg = (int)(u % nseg);
-        const int strip = (int)((u / nseg) % nstrip);
-        const int b = (int)(u / nseg / nstrip);
-        const int w0 = seg * TC_TW;
-        const int h0 = strip * WG_STRIP, h1 = min(h0 + WG_STRIP, H);
-        // the previous unit's MMAs read the slots about to be restaged
-        for (int q = 0; q < 3; ++q) wait_row(q);
-        __syncthreads();
-        // prologue: the input and gradient rows of the first WG_AHEAD output rows
-        const int hp = min(h0 + WG_AHEAD, h1);
-        for (int xr = h0 + ky0 - 1; xr <= hp - 1 + ky0 + KYS - 2; ++xr) stage_x(b, w0, xr);
-        for (int h = h0; h < hp; ++h) stage_g(b, w0, h);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        for (int h = h0; h < h1; ++h) {
-            // rows for output row h + WG_AHEAD: its newest input row and its
-            // gradient row, into the slots that output row h - 2 read last
-            const int hn = h + WG_AHEAD;
-            if (hn < h1) {
-                if (h - 2 >= h0) wait_row((h - 2) % 3);
-                __syncthreads();
-                stage_x(b, w0, hn + ky0 + KYS - 2);
-                stage_g(b, w0, hn);
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            // row h's copies were committed WG_AHEAD groups ago (or in the prologue)
-            asm volatile("cp.async.wait_group %0;" ::"n"(WG_AHEAD) : "memory");
+    if (warp >= 4 && warp < 8) {
+        // ---- producers ----
+        const int p = threadIdx.x - 128;
+        constexpr int NX = KC, NGP = (TC_P * GC + 127) / 128;      // pieces per thread of a row
+        int n = 0, told = 0, done = 0;           // steps staged, handed over, known to be complete
+        auto hand_over = [&](int upto) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (s_bad) break;
-            wait_row(h % 3);                       // row h - 3 left this mbarrier's phase
-            if (threadIdx.x == 0) {
-                const unsigned ga = smem_u32(gslot(h));
+            for (; told < upto; ++told) mbar_arrive(&s_full[told % GR]);
+        };
+        auto wait_step = [&](int step) {         // step `step` is complete
+            if (step >= told) {                  // it may wait for copies in flight
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                hand_over(n);
+            }
+            for (; done <= step; ++done)
+                if (!mbar_wait(smem_u32(&s_empty[done % GR]), (done / GR) & 1)) return false;
+            return true;
+        };
+        // a thread's pieces (16 bytes, channel chunk c of point pt) are the same
+        // in every row: their offsets in a row are kept
+        int src[NX], gsrc[NGP], cur_w0 = -1, cur_shift = -1;
+        int e = 0, last[XR];                     // next entry; last step that reads each slot's row
 #pragma unroll
-                for (int kyl = 0; kyl < KYS; ++kyl) {
-                    const unsigned xa = smem_u32(xslot(h + ky0 + kyl - 1));
+        for (int q = 0; q < XR; ++q) last[q] = -1;
+        for (long u = blockIdx.x; u < nunits && !*bad; u += gridDim.x) {
+            const Unit q = unit_of(u);
+            const int rows = q.h1 - q.h0, n_first = n;
+            bool ok = true;
+            for (int i = 0; i < rows && ok; ++i) {
+                if (n >= GR) ok = ok && wait_step(n - GR);
+                for (int r = i == 0 ? 0 : i + 2; r <= i + 2; ++r, ++e) {
+                    const int slot = e % XR;
+                    int before = -1;
 #pragma unroll
-                    for (int kx = 0; kx < 3; ++kx) {
-#pragma unroll
-                        for (int ks = 0; ks < TC_TW / 16; ++ks) {
-                            const unsigned aa = xa + (unsigned)(ks * 16 + kx) * 16;
-                            const unsigned ba = ga + (unsigned)(ks * 16) * 16;
-                            // MN-major: the leading offset steps along K (8 points,
-                            // 128 bytes), the stride offset along MN (one plane)
-                            mma_bf16(tmem + (unsigned)((kyl * 3 + kx) * COUT), sdesc(aa, 128, TC_P * 16),
-                                     sdesc(ba, 128, TC_TW * 16), ID, acc | (unsigned)ks);
+                    for (int k = 0; k < XR; ++k)
+                        if (k == slot) {
+                            before = last[k];
+                            last[k] = n_first + min(r, rows - 1);
                         }
+                    ok = ok && (before < 0 || wait_step(before));
+                    int hr = q.h0 - 1 + r, shift = 0;
+                    if (hr < 0 || hr >= H) {
+                        hr = hr < 0 ? 0 : H - 1;
+                        shift = W / 2;
+                    }
+                    const __nv_bfloat16 *row = a.x + ((size_t)q.b * H + hr) * W * (CIN - CS);
+                    const __nv_bfloat16 *crow =
+                        CS > 0 ? a.xc + ((size_t)q.b * (H / 2) + hr / 2) * (W / 2) * CS : nullptr;
+                    unsigned char *base = Xs + (size_t)slot * S::XSLOT;
+                    if (q.w0 != cur_w0 || shift != cur_shift) {
+#pragma unroll
+                        for (int k = 0; k < NX; ++k) {
+                            const int z = p + 128 * k, c = z % KC;
+                            int ws = q.w0 + z / KC + shift;
+                            if (ws >= W) ws -= W;
+                            src[k] = CS > 0 && c < CS / 8 ? (ws >> 1) * CS + c * 8 : ws * (CIN - CS) + (c - CS / 8) * 8;
+                        }
+#pragma unroll
+                        for (int k = 0; k < NGP; ++k) {
+                            const int z = p + 128 * k;
+                            int ws = q.w0 - 1 + z / GC;
+                            if (ws < 0) ws += W;
+                            else if (ws >= W) ws -= W;
+                            gsrc[k] = ws * ntot + z % GC * 8;
+                        }
+                        cur_w0 = q.w0;
+                        cur_shift = shift;
+                    }
+#pragma unroll
+                    for (int k = 0; k < NX; ++k) {
+                        const int z = p + 128 * k, c = z % KC;
+                        const __nv_bfloat16 *sp = (CS > 0 && c < CS / 8 ? crow : row) + src[k];
+                        unsigned char *dst = base + (c * TC_TW + z / KC) * 16;
+                        cp16(dst, sp);
+                        if (slot < S::MIR) cp16(dst + XR * S::XSLOT, sp);
                     }
                 }
-                mma_commit(smem_u32(&s_mbar[h % 3]));
+                const __nv_bfloat16 *grow = a.g + ((size_t)q.b * H + q.h0 + i) * W * ntot + n0;
+                unsigned char *gb = Gs + (size_t)(n % GR) * S::GSLOT;
+#pragma unroll
+                for (int k = 0; k < NGP; ++k) {
+                    const int z = p + 128 * k;
+                    if (z >= TC_P * GC) break;
+                    cp16(gb + (z % GC * TC_P + z / GC) * 16, grow + gsrc[k]);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                ++n;
+                asm volatile("cp.async.wait_group %0;" ::"n"(DEPTH) : "memory");
+                if (n - DEPTH > told) hand_over(n - DEPTH);
             }
-            __syncwarp();
-            acc = 1;
-            pend[h % 3] = true;
-            if (do_bias) {
-                // bias gradient: thread t adds channel t % COUT over every
-                // (128 / COUT)-th point of the row, all threads at once
-                constexpr int NPART = 128 / COUT;
-                const unsigned char *gs = gslot(h);
-                const int co = threadIdx.x % COUT, c = co / 8, e = co % 8;
+            if (!ok) *bad = 1;
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        hand_over(n);
+    } else if (warp == 8) {
+        // ---- MMAs: the whole warp runs the role, one lane issues ----
+        const unsigned one = elect_one();
+        // the leading offset steps along K (8 points, 128 bytes), the stride
+        // offset along MN (one plane)
+        const unsigned long long A0 = sdesc(smem_u32(Xs), 128, TC_TW * 16), B0 = sdesc(smem_u32(Gs), 128, TC_P * 16);
+        int n = 0, e0 = 0;
+        unsigned acc = 0;
+        for (long u = blockIdx.x; u < nunits && !*bad; u += gridDim.x) {
+            const Unit q = unit_of(u);
+            for (int i = 0; i < q.h1 - q.h0; ++i, ++n) {
+                if (!mbar_wait(smem_u32(&s_full[n % GR]), (n / GR) & 1)) { *bad = 1; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const unsigned long long gd = B0 + (unsigned)(n % GR) * (unsigned)(S::GSLOT / 16);
+#pragma unroll
+                for (int gq = 0; gq < S::NG; ++gq) {
+                    const int slot = (e0 + i + gq * S::RPG) % XR;
+                    const unsigned long long xd = A0 + (unsigned)slot * (unsigned)(S::XSLOT / 16);
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+                        for (int ks = 0; ks < TC_TW / 16; ++ks)
+                            mma_bf16_one(tmem + (unsigned)((gq * 3 + kx) * COUT), xd + ks * 16, gd + (ks * 16 + 2 - kx),
+                                         ID, acc | (unsigned)ks, one);
+                }
+                mma_commit_one(smem_u32(&s_empty[n % GR]), one);
+                acc = 1;
+            }
+            e0 += q.h1 - q.h0 + 2;
+        }
+        mma_commit_one(smem_u32(&s_done), one);
+        if (!mbar_wait(smem_u32(&s_done), 0)) *bad = 1;
+    } else {
+        // ---- bias gradient: thread t adds channel t % COUT over every
+        // (128 / COUT)-th point of the step's row ----
+        constexpr int NPART = 128 / COUT;
+        const int co = threadIdx.x % COUT, p0 = threadIdx.x / COUT;
+        float bsum = 0.f;
+        int n = 0;
+        for (long u = blockIdx.x; u < nunits && !*bad; u += gridDim.x) {
+            const Unit q = unit_of(u);
+            for (int i = 0; i < q.h1 - q.h0; ++i, ++n) {
+                if (!mbar_wait(smem_u32(&s_full[n % GR]), (n / GR) & 1)) *bad = 1;
+                if (__any_sync(0xffffffffu, *bad)) break;
+                const __nv_bfloat16 *gs =
+                    (const __nv_bfloat16 *)(Gs + (size_t)(n % GR) * S::GSLOT + (size_t)(co / 8 * TC_P + 1) * 16) + co % 8;
 #pragma unroll 8
-                for (int p = threadIdx.x / COUT; p < TC_TW; p += NPART)
-                    bsum += __bfloat162float(((const __nv_bfloat16 *)(gs + ((size_t)c * TC_TW + p) * 16))[e]);
+                for (int k = p0; k < TC_TW; k += NPART) bsum += __bfloat162float(gs[k * 8]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&s_empty[n % GR]);
             }
         }
+        if (a.db && !*bad) atomicAdd(a.db + n0 + co, bsum);
     }
-    for (int q = 0; q < 3; ++q) wait_row(q);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!s_bad && acc) {
-        // lanes = input channels (warp w: 32 w .. 32 w + 31), columns = (ky, kx, co)
-        const int ci = warp * 32 + lane;
+    if (!s_bad && warp < 4) {
+        // lanes = (kernel row of the group, input channel), columns = (group, kx, co)
+        const int m = warp * 32 + lane, kr = m / CIN, ci = m % CIN;
         const unsigned trow = tmem + ((unsigned)(warp * 32) << 16);
-#pragma unroll 4
-        for (int c0 = 0; c0 < (int)S::NCOL; c0 += 8) {
-            float v[8];
-            tmem_ld8(trow + c0, v);
+#pragma unroll 2
+        for (int c0 = 0; c0 < S::NCOL; c0 += 16) {
+            float v[16];
+            tmem_ld16(trow + c0, v);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (ci < CIN) {
+            const int grp = c0 / (3 * COUT), kx = c0 / COUT % 3, co = n0 + c0 % COUT;
+            const int ky = grp * S::RPG + kr;
+            if (kr < S::RPG && ky < 3) {
+                float *dw = a.dw + ((size_t)(ky * 3 + kx) * ntot + co) * CIN + ci;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int col = c0 + q, tap = col / COUT, co = col % COUT;
-                    atomicAdd(a.dw + ((size_t)(ky0 * 3 + tap) * COUT + co) * CIN + ci, v[q]);
-                }
+                for (int k = 0; k < 16; ++k) atomicAdd(dw + (size_t)k * CIN, v[k]);
             }
         }
     }
-    if (do_bias && acc) atomicAdd(a.db + threadIdx.x % COUT, bsum);
     if (s_bad && threadIdx.x == 0) atomicExch(err, 1);
-    asm volatile("cp.async.wait_all;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -814,35 +861,33 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(WgradArgs a, int *err)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
 }
 
-template <int CIN, int CS, int COUT, int KYS>
-static cudaError_t wgrad_tc_t(const WgradArgs &a, int sms, int *err, cudaStream_t s)
+template <int CIN, int CS, int COUT>
+static cudaError_t wgrad_tc_t(const WgradArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
 {
-    typedef WgShape<CIN, COUT, KYS> S;
-    const size_t smem = S::BYTES;
-    cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<CIN, CS, COUT, KYS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const size_t smem = WgShape<CIN, COUT>::BYTES;
+    int bps = 0;
+    cudaError_t e = occupancy_once<k_wgrad_tc<CIN, CS, COUT>>(288, smem, &bps);
     if (e != cudaSuccess) return e;
-    constexpr int NKG = 3 / KYS;
-    const long nunits = (long)a.B * (a.W / TC_TW) * ((a.H + WG_STRIP - 1) / WG_STRIP);
-    long nsplit = sms / NKG > 0 ? sms / NKG : 1;   // about one block per SM
-    if (nsplit > nunits) nsplit = nunits;
-    k_wgrad_tc<CIN, CS, COUT, KYS><<<(int)(NKG * nsplit), 128, smem, s>>>(a, err);
+    if (bps < 1) return cudaErrorInvalidConfiguration;
+    // one block per SM; strips of 8 rows, shorter while blocks would be idle
+    const long cap = sms / nsplit > 0 ? sms / nsplit : 1;
+    int strip = 8;
+    auto units = [&](int st) { return (long)a.B * (a.W / TC_TW) * ((a.H + st - 1) / st); };
+    while (strip > 2 && units(strip) < cap) strip /= 2;
+    const long n = units(strip);
+    k_wgrad_tc<CIN, CS, COUT><<<dim3((unsigned)(n < cap ? n : cap), nsplit), 288, smem, s>>>(a, strip, err);
     return cudaGetLastError();
-}
-
-// the layers whose weight gradient takes tcgen05: c5 (96 -> 32, all nine taps
-// in one block, 288 TMEM columns) and c4 (128 -> 64, a kernel row per block,
-// 192 columns), rows of a multiple of 128 points; both read their input from
-// the coarser level and the skip connection, like the forward pass
-bool wgrad_tc_supported(int cin, int cout, int W)
-{
-    return W % TC_TW == 0 && ((cin == 96 && cout == 32) || (cin == 128 && cout == 64));
 }
 
 cudaError_t launch_wgrad_tc(int cin, int cout, const WgradArgs &a, int sms, int *err, cudaStream_t s)
 {
-    if (cin == 96 && cout == 32) return wgrad_tc_t<96, 64, 32, 3>(a, sms, err, s);
-    if (cin == 128 && cout == 64) return wgrad_tc_t<128, 64, 64, 1>(a, sms, err, s);
+    if (cin == 16 && cout == 32) return wgrad_tc_t<16, 0, 32>(a, 1, sms, err, s);
+    if (cin == 32 && cout == 64) return wgrad_tc_t<32, 0, 64>(a, 1, sms, err, s);
+    if (cin == 64 && cout == 64) return wgrad_tc_t<64, 0, 64>(a, 1, sms, err, s);
+    // 9 x 64 accumulator columns are more than TMEM has: 32 outputs a block
+    if (cin == 128 && cout == 64) return wgrad_tc_t<128, 64, 32>(a, 2, sms, err, s);
+    if (cin == 96 && cout == 32) return wgrad_tc_t<96, 64, 32>(a, 1, sms, err, s);
+    if (cin == 32 && cout == 16) return wgrad_tc_t<32, 0, 16>(a, 1, sms, err, s);
     return cudaErrorInvalidValue;
 }
 
