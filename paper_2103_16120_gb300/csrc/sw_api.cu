@@ -525,31 +525,25 @@ extern "C" sw_status sw_precond_apply(sw_grid g, const sw_solve_opts *o, const v
         if ((st = refactor(g, s))) return st;
     }
     if ((st = ensure_ws(g, o->prec, o->k))) return st;
-    alignas(16) unsigned char hbuf[sizeof(SolverBlock::dev)];
-    int nst = o->pc >= 2 ? o->n_richardson : 1;
+    const int nst = o->pc >= 2 ? o->n_richardson : 1, threads = row_threads(g->nx, o->threads_per_row);
     if (o->prec == SW_PREC_FP64) {
         if ((st = ensure_f64(g, s))) return st;
         MemberDev<PolFP64> M;
         fill_member<PolFP64>(g, o, nullptr, nullptr, M);
         M.r = (double *)r;                    // the stages read r from the member's r
         M.e = (double *)q;                    // FP64: the last stage writes q directly
-        std::memcpy(hbuf, &M, sizeof(M));
+        CK(launch_precond(o->prec, &M, g->nx, g->ny, nst, q, threads, s));
     } else if (o->prec == SW_PREC_MIXED_FP16) {
         MemberDev<PolF16> M;
         fill_member<PolF16>(g, o, nullptr, nullptr, M);
         M.r = (float *)r;
-        std::memcpy(hbuf, &M, sizeof(M));
+        CK(launch_precond(o->prec, &M, g->nx, g->ny, nst, q, threads, s));
     } else {
         MemberDev<PolBF16> M;
         fill_member<PolBF16>(g, o, nullptr, nullptr, M);
         M.r = (float *)r;
-        std::memcpy(hbuf, &M, sizeof(M));
+        CK(launch_precond(o->prec, &M, g->nx, g->ny, nst, q, threads, s));
     }
-    CK(cudaMemcpyAsync(g->blk->dev, hbuf, member_dev_bytes(o->prec), cudaMemcpyHostToDevice, s));
-    CK(launch_precond(o->prec, g->blk->dev, g->nx, g->ny, nst, o->prec == SW_PREC_FP64 ? nullptr : q,
-                      row_threads(g->nx, o->threads_per_row), s));
-    // the host staging buffer must outlive the asynchronous copy
-    CK(cudaStreamSynchronize(s));
     return SW_OK;
 }
 

@@ -122,20 +122,34 @@ __global__ void __launch_bounds__(128) k_operator4(OpArgs<CT> a, const T *__rest
     st4(y + row + i0, out);
 }
 
-// one preconditioner stage of every row (stage 0 from the residual r)
-template <class Pol>
-__global__ void __launch_bounds__(MAX_THREADS) k_precond(const MemberDev<Pol> *Mp, int mu)
+// one preconditioner stage of every row (stage 0 from the residual r), one
+// block per row.  The member descriptor is a kernel parameter: copied to the
+// device first, it cost the call a copy and a wait for the stream (the host
+// copy had to outlive it).  qout (mixed policies, last stage): receives the
+// output's values as stored, which a pass of its own read back before.
+// Bound by the row's chain of loads, scans and stores (mixed) and by FP64 issue
+// (FP64), so the registers are held down for more blocks per SM: two stages
+// with 1 / 2 / 3 (FP64) and 2 / 3 / 4 (FP16) blocks per SM, us: 2048 x 1024 235
+// / 199 / 191 and 83 / 74 / 84, 1440 x 721 149 / 136 / 110 and 55 / 45 / 51, 1024
+// x 512 (128 threads) 68 / 55 / 60 and 23 / 25 / 28.  Before (descriptor copy,
+// unpacking pass) 254 and 83 at 2048 x 1024 and 1440 x 721.
+template <class Pol, int MINB>
+__global__ void __launch_bounds__(MAX_THREADS, MINB) k_precond(const __grid_constant__ MemberDev<Pol> Mp, int mu,
+                                                               typename Pol::comp *qout)
 {
     typedef typename Pol::comp comp;
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ MemberDev<Pol> s_M;
-    copy_in(&s_M, Mp);
+    static_assert(sizeof(MemberDev<Pol>) % 4 == 0, "descriptor copied as 32-bit words");
+    for (int k = threadIdx.x; k < (int)(sizeof(s_M) / 4); k += blockDim.x)
+        reinterpret_cast<int *>(&s_M)[k] = reinterpret_cast<const int *>(&Mp)[k];
     __syncthreads();
     const MemberDev<Pol> &M = s_M;
     const int j = blockIdx.x;
     RowView<Pol> v;
     view_const_global(M, j, v);
     view_state_global(M, j, v);
+    if (qout) v.el = qout + (size_t)j * M.nx;
     const comp eta = (comp)(*M.etap);
     if (mu == 0) {
         comp *sb = (comp *)(dsm + sb_offset<Pol>(M.nx));
@@ -161,16 +175,6 @@ __global__ void __launch_bounds__(MAX_THREADS) k_store_e(const MemberDev<Pol> *M
     for (int i = threadIdx.x; i < nx; i += blockDim.x) sb[pidx(i)] = (comp)ef[(size_t)j * nx + i];
     __syncthreads();
     q_store_row(M, M.e, M.e32, M.e_s, j, sb, (comp *)nullptr, scratch);
-}
-
-// dequantise the preconditioner output e into q (mixed policies)
-template <class Pol>
-__global__ void k_unpack_e(const MemberDev<Pol> *Mp, float *q)
-{
-    const MemberDev<Pol> &M = *Mp;
-    const int j = blockIdx.x;
-    const float sc = q_scale(M, M.e_s, j);
-    for (int i = threadIdx.x; i < M.nx; i += blockDim.x) q[(size_t)j * M.nx + i] = (float)q_load(M, M.e, M.e32, sc, j, i);
 }
 
 // ---------------------------------------------------------------------------
@@ -357,26 +361,28 @@ cudaError_t launch_operator_f32(const OpArgs<float> &a, const float *x, float *y
     return cudaGetLastError();
 }
 
-template <class Pol>
-static cudaError_t launch_precond_t(const void *Mdev, int nx, int ny, int nstages, float *qout, int threads,
+template <class Pol, int MINB>
+static cudaError_t launch_precond_t(const void *M, int nx, int ny, int nstages, void *qout, int threads,
                                     cudaStream_t s)
 {
-    const MemberDev<Pol> *M = (const MemberDev<Pol> *)Mdev;
-    size_t smem = work_bytes<Pol>(nx);
-    cudaError_t e = cudaFuncSetAttribute(k_precond<Pol>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = work_bytes<Pol>(nx);
+    cudaError_t e = raise_smem_limit((const void *)k_precond<Pol, MINB>, smem);
     if (e != cudaSuccess) return e;
-    for (int mu = 0; mu < nstages; ++mu) k_precond<Pol><<<ny, threads, smem, s>>>(M, mu);
-    if (qout) k_unpack_e<Pol><<<ny, 128, 0, s>>>(M, qout);
+    for (int mu = 0; mu < nstages; ++mu)
+        k_precond<Pol, MINB><<<ny, threads, smem, s>>>(
+            *(const MemberDev<Pol> *)M, mu, Pol::kMixed && mu == nstages - 1 ? (typename Pol::comp *)qout : nullptr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_precond(int prec, const void *Mdev, int nx, int ny, int nstages, void *qout, int threads,
+// M: the member descriptor, host memory (read before the call returns)
+cudaError_t launch_precond(int prec, const void *M, int nx, int ny, int nstages, void *qout, int threads,
                            cudaStream_t s)
 {
     switch (prec) {
-    case 0: return launch_precond_t<PolFP64>(Mdev, nx, ny, nstages, nullptr, threads, s);
-    case 1: return launch_precond_t<PolF16>(Mdev, nx, ny, nstages, (float *)qout, threads, s);
-    case 2: return launch_precond_t<PolBF16>(Mdev, nx, ny, nstages, (float *)qout, threads, s);
+    case 0: return threads > 128 ? launch_precond_t<PolFP64, 3>(M, nx, ny, nstages, qout, threads, s)
+                                 : launch_precond_t<PolFP64, 2>(M, nx, ny, nstages, qout, threads, s);
+    case 1: return launch_precond_t<PolF16, 3>(M, nx, ny, nstages, qout, threads, s);
+    case 2: return launch_precond_t<PolBF16, 3>(M, nx, ny, nstages, qout, threads, s);
     default: return cudaErrorInvalidValue;
     }
 }
