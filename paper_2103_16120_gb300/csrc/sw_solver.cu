@@ -122,6 +122,72 @@ __global__ void __launch_bounds__(128) k_operator4(OpArgs<CT> a, const T *__rest
     st4(y + row + i0, out);
 }
 
+// The FP64 operator, bound by FP64 issue (64 cycles per warp instruction): a
+// thread takes 4 columns down R rows, so that a meridional face's flux is formed
+// once for its two rows and a zonal one once for its two points, with the sums
+// that faces share: about 20 FP64 operations a point (26 with R = 1) instead of
+// k_operator4's 35.  A face's expression is the same wherever it is formed, so
+// the results do not depend on R.  us: 2048 x 1024 (R = 4) 121, now 90; 1440 x 721
+// (4) 70, 54; 1024 x 512 (2) 35, 31; 512 x 256 (1) 12.4, 10.3.
+template <int R>
+__global__ void __launch_bounds__(128) k_operator_rows(OpArgs<double> a, const double *__restrict__ x,
+                                                       double *__restrict__ y)
+{
+    const int nx = a.nx, ny = a.ny, j0 = blockIdx.y * R;
+    const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (i0 >= nx) return;
+    const int iw = i0 == 0 ? nx - 1 : i0 - 1;
+    double xs[6], xc[6], xn[6];
+    auto load_row = [&](int j, double (&v)[6]) {
+        int src, sh;
+        ghost_row(j, nx, ny, src, sh);
+        ld6(x + (size_t)src * nx, i0, sh, nx, v);
+    };
+    // flux through the faces between the rows of two windows, the lower one row j
+    auto face = [&](int j, const double (&lo)[6], const double (&hi)[6], double (&F)[4]) {
+        double ay[4], cy[4], by[4], v[6];
+        const size_t at = (size_t)j * nx + i0;
+        ld4(a.ay + at, ay); ld4(a.cy + at, cy); ld4(a.by + at, by);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = lo[k] + hi[k];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            F[u] = fma(by[u], v[u + 1], fma(cy[u], v[u + 2] - v[u], ay[u] * (hi[u + 1] - lo[u + 1])));
+    };
+    load_row(j0 - 1, xs);
+    load_row(j0, xc);
+    double FS[4] = {}, FN[4];
+    if (j0 > 0) face(j0 - 1, xs, xc, FS);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int j = j0 + r;
+        if (j >= ny) break;
+        load_row(j + 1, xn);
+        const size_t row = (size_t)j * nx;
+        double ax[5], cx[5], bx[5], cc[4], q[4], F[5], d[6];
+        ax[0] = __ldg(a.ax + row + iw); cx[0] = __ldg(a.cx + row + iw); bx[0] = __ldg(a.bx + row + iw);
+        ld4(a.ax + row + i0, q); for (int k = 0; k < 4; ++k) ax[k + 1] = q[k];
+        ld4(a.cx + row + i0, q); for (int k = 0; k < 4; ++k) cx[k + 1] = q[k];
+        ld4(a.bx + row + i0, q); for (int k = 0; k < 4; ++k) bx[k + 1] = q[k];
+        ld4(a.C + row + i0, cc);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) d[k] = xn[k] - xs[k];
+#pragma unroll
+        for (int m = 0; m < 5; ++m)
+            F[m] = fma(cx[m], d[m] + d[m + 1], fma(bx[m], xc[m] + xc[m + 1], ax[m] * (xc[m + 1] - xc[m])));
+        if (j < ny - 1) face(j, xc, xn, FN);
+        else FN[0] = FN[1] = FN[2] = FN[3] = 0.0;
+        double out[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) out[u] = fma(-cc[u], xc[u + 1], (F[u + 1] - F[u]) + (FN[u] - FS[u]));
+        st4(y + row + i0, out);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) { xs[k] = xc[k]; xc[k] = xn[k]; }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) FS[u] = FN[u];
+    }
+}
+
 // one preconditioner stage of every row (stage 0 from the residual r), one
 // block per row.  The member descriptor is a kernel parameter: copied to the
 // device first, it cost the call a copy and a wait for the stream (the host
@@ -338,7 +404,12 @@ static bool op4_ok(const OpArgs<T> &a, const T *x, const T *y)
 cudaError_t launch_operator_f64(const OpArgs<double> &a, const double *x, double *y, int threads, cudaStream_t s)
 {
     if (op4_ok(a, x, y)) {
-        k_operator4<double, double><<<dim3((a.nx / 4 + 127) / 128, a.ny), 128, 0, s>>>(a, x, y);
+        // four rows a thread while that leaves three blocks for every SM
+        const unsigned bx = (a.nx / 4 + 127) / 128;
+        const long want = 3 * 152;
+        if ((long)bx * ((a.ny + 3) / 4) >= want) k_operator_rows<4><<<dim3(bx, (a.ny + 3) / 4), 128, 0, s>>>(a, x, y);
+        else if ((long)bx * ((a.ny + 1) / 2) >= want) k_operator_rows<2><<<dim3(bx, (a.ny + 1) / 2), 128, 0, s>>>(a, x, y);
+        else k_operator_rows<1><<<dim3(bx, a.ny), 128, 0, s>>>(a, x, y);
         return cudaGetLastError();
     }
     size_t smem = 3 * (size_t)a.nx * sizeof(double);
