@@ -112,8 +112,8 @@ static int row_threads(int nx, int requested = 0)
     return t;
 }
 
-// threads of the set-up kernels' blocks, one row each: about four points a
-// thread (the pivots' chunks set the rounding of the FP32 factors)
+// threads of the FP32 factorisation's blocks, one row each: about four points
+// a thread (the pivots' chunks set the rounding of the FP32 factors)
 static int setup_threads(int nx)
 {
     int t = ((nx / 4 + 31) / 32) * 32;
@@ -323,7 +323,7 @@ static FactorArgs factor_args(const sw_grid_s *g)
 {
     FactorArgs f;
     f.nx = g->nx; f.ny = g->ny; f.eta_explicit = g->eta_explicit;
-    f.ax = g->ax; f.C = g->C; f.rowmax = g->rowmax;
+    f.ax = g->ax; f.C = g->C; f.rowmax = g->rowmax; f.wax = g->wax; f.wC = g->wC;
     f.lf = g->lf; f.invD = g->invD; f.zz = g->zz; f.gam = g->gam; f.ec = g->ec; f.eta_out = g->eta;
     f.lf32 = g->lf32; f.invD32 = g->invD32; f.zz32 = g->zz32; f.gam32 = g->gam32; f.ec32 = g->ec32;
     f.lfT = g->lfT; f.invDT = g->invDT; f.zzT = g->zzT;
@@ -349,7 +349,7 @@ static sw_status ensure_f64(sw_grid g, cudaStream_t s)
     CK(cudaStreamIsCapturing(s, &cap));
     const bool recorded = (cap != cudaStreamCaptureStatusNone);
     if (g->f64_valid && !recorded) return SW_OK;
-    CK(launch_factor(factor_args(g), true, setup_threads(g->nx), s));
+    CK(launch_factor(factor_args(g), true, row_threads(g->nx), s));
     CK(launch_weights(WeightArgs{g->nx, g->ny, g->ax, g->cx, g->bx, g->ay, g->cy, g->by, g->C, g->wgt}, s));
     if (!recorded) g->f64_valid = true;
     return SW_OK;
@@ -364,12 +364,14 @@ extern "C" sw_status sw_elliptic_set_coeffs(sw_grid g, const double *A11, const 
         return fail(SW_ERR_INVALID_ARG, "sw_elliptic_set_coeffs: NULL coefficient pointer");
     cudaStream_t s = (cudaStream_t)stream;
     FaceArgs a;
-    a.nx = g->nx; a.ny = g->ny; a.dlam = g->dlam; a.dphi = g->dphi;
+    a.nx = g->nx; a.ny = g->ny;
+    a.idl2 = 0.5 / (g->dlam * g->dlam); a.idp2 = 0.5 / (g->dphi * g->dphi); a.i4 = 0.5 / (4.0 * g->dlam * g->dphi);
+    a.i2l = 0.5 / (2.0 * g->dlam); a.i2p = 0.5 / (2.0 * g->dphi);
     a.A11 = A11; a.A12 = A12; a.A21 = A21; a.A22 = A22; a.B1 = B1; a.B2 = B2; a.C = C;
     a.ax = g->ax; a.cx = g->cx; a.bx = g->bx; a.ay = g->ay; a.cy = g->cy; a.by = g->by; a.C64 = g->C; a.diag = g->diag;
     a.wax = g->wax; a.wcx = g->wcx; a.wbx = g->wbx; a.way = g->way; a.wcy = g->wcy; a.wby = g->wby; a.wC = g->wC;
     a.wdiag = g->wdiag; a.rowmax = g->rowmax;
-    CK(launch_faces(a, setup_threads(g->nx), s));
+    CK(launch_faces(a, std::min(MAX_THREADS, (g->nx + 31) / 32 * 32), s));
     sw_status st = refactor(g, s);
     if (st) return st;
     g->has_coeffs = true;

@@ -13,56 +13,91 @@
 
 namespace sw {
 
+// x rounded to FP32 (nearest, ties to even) with integer instructions: the
+// conversion runs at the FP64 rate, 64 cycles per warp instruction, and every
+// point makes eight of them.  Results outside FP32's normal range (and NaN)
+// take the conversion.
+__device__ __forceinline__ float to_f32(double x)
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const unsigned hi = (unsigned)(u >> 32);
+    const unsigned ex = (hi >> 20) & 0x7ff;                    // biased by 1023
+    if (ex - 897u < 254u) {                                    // 2^-126 .. 2^127
+        const unsigned long long m = (u & 0x7fffffffffffffffull) - ((unsigned long long)896 << 52);
+        const unsigned r = (unsigned)((m + 0x0fffffffull + ((m >> 29) & 1)) >> 29);
+        return __uint_as_float(r | (hi & 0x80000000u));
+    }
+    if ((u << 1) == 0) return __uint_as_float(hi);             // +-0
+    return (float)x;
+}
+
+// One block per row, bound by FP64 issue.  A point's west face is its
+// neighbour's east one, read back from shared memory instead of formed twice;
+// the FP32 copies and the row's maximum take integer instructions: about 24
+// FP64 operations a point.  With 46 (west faces formed again, conversions) and
+// about four points a thread, and five divisions in
+// every thread for the face scales, us: 2048 x 1024 178, now 111; 512 x 256 20.3,
+// 10.9; 128 x 64 16.5, 4.5.
 __global__ void __launch_bounds__(MAX_THREADS) k_faces(FaceArgs a)
 {
-    __shared__ double red[MAX_THREADS / 32];
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ unsigned long long red[MAX_THREADS / 32];
     const int nx = a.nx, ny = a.ny, j = blockIdx.x;
-    // the face scales, each with the 1/2 of the face mean folded in (a power
-    // of two: the products round exactly as (a + b)/2 times the scale)
-    const double idl2 = 0.5 / (a.dlam * a.dlam), idp2 = 0.5 / (a.dphi * a.dphi);
-    const double i4 = 0.5 / (4.0 * a.dlam * a.dphi), i2l = 0.5 / (2.0 * a.dlam), i2p = 0.5 / (2.0 * a.dphi);
+    double *sax = (double *)dsm, *sbx = sax + nx;              // the row's ax and bx
+    const double idl2 = a.idl2, idp2 = a.idp2, i4 = a.i4, i2l = a.i2l, i2p = a.i2p;
     const size_t row = (size_t)j * nx;
-    double m = 0.0;
     for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-        const int ip = (i + 1 == nx) ? 0 : i + 1, im = (i == 0) ? nx - 1 : i - 1;
+        const int ip = (i + 1 == nx) ? 0 : i + 1;
         const size_t id = row + i;
-        // x faces i+1/2 and i-1/2 of row j
-        double ax = (a.A11[id] + a.A11[row + ip]) * idl2;
-        double cx = (a.A12[id] + a.A12[row + ip]) * i4;
-        double bx = (a.B1[id] + a.B1[row + ip]) * i2l;
-        double axm = (a.A11[row + im] + a.A11[id]) * idl2;
-        double bxm = (a.B1[row + im] + a.B1[id]) * i2l;
+        // x faces i+1/2 of row j
+        const double ax = (a.A11[id] + a.A11[row + ip]) * idl2;
+        const double cx = (a.A12[id] + a.A12[row + ip]) * i4;
+        const double bx = (a.B1[id] + a.B1[row + ip]) * i2l;
+        sax[i] = ax; sbx[i] = bx;
+        a.ax[id] = ax; a.cx[id] = cx; a.bx[id] = bx;
+        a.wax[id] = to_f32(ax); a.wcx[id] = to_f32(cx); a.wbx[id] = to_f32(bx);
+    }
+    __syncthreads();
+    unsigned long long m = 0;                                  // bits of the largest |diag(P^M)|
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+        const int im = (i == 0) ? nx - 1 : i - 1;
+        const size_t id = row + i;
+        const double ax = sax[i], axm = sax[im], bx = sbx[i], bxm = sbx[im];
         // y faces j+1/2 and j-1/2 (zero through the pole faces)
         double ay = 0.0, cy = 0.0, by = 0.0, ays = 0.0, bys = 0.0;
+        const double a22 = a.A22[id], b2 = a.B2[id];
         if (j < ny - 1) {
-            ay = (a.A22[id] + a.A22[id + nx]) * idp2;
+            ay = (a22 + a.A22[id + nx]) * idp2;
             cy = (a.A21[id] + a.A21[id + nx]) * i4;
-            by = (a.B2[id] + a.B2[id + nx]) * i2p;
+            by = (b2 + a.B2[id + nx]) * i2p;
         }
         if (j > 0) {
-            ays = (a.A22[id - nx] + a.A22[id]) * idp2;
-            bys = (a.B2[id - nx] + a.B2[id]) * i2p;
+            ays = (a.A22[id - nx] + a22) * idp2;
+            bys = (a.B2[id - nx] + b2) * i2p;
         }
         const double c = a.C[id];
         // diagonal of P^M = L - P^Z + P^H, and of L
         const double dpm = (bx - bxm) - (ay + ays) + (by - bys);
         const double dl = -(ax + axm) + dpm - c;
-        a.ax[id] = ax; a.cx[id] = cx; a.bx[id] = bx;
         a.ay[id] = ay; a.cy[id] = cy; a.by[id] = by;
         a.C64[id] = c; a.diag[id] = dl;
-        a.wax[id] = (float)ax; a.wcx[id] = (float)cx; a.wbx[id] = (float)bx;
-        a.way[id] = (float)ay; a.wcy[id] = (float)cy; a.wby[id] = (float)by;
-        a.wC[id] = (float)c; a.wdiag[id] = (float)dl;
-        m = fmax(m, fabs(dpm));
+        a.way[id] = to_f32(ay); a.wcy[id] = to_f32(cy); a.wby[id] = to_f32(by);
+        a.wC[id] = to_f32(c); a.wdiag[id] = to_f32(dl);
+        // magnitudes compare as their bits do; a NaN takes no part, as in fmax
+        const unsigned long long b = (unsigned long long)__double_as_longlong(dpm) & 0x7fffffffffffffffull;
+        if (b <= 0x7ff0000000000000ull && b > m) m = b;
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long q = __shfl_xor_sync(0xffffffffu, m, o);
+        m = q > m ? q : m;
+    }
     if (lane == 0) red[w] = m;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double mm = 0.0;
-        for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) mm = fmax(mm, red[ww]);
-        a.rowmax[j] = mm;
+        unsigned long long mm = 0;
+        for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) mm = red[ww] > mm ? red[ww] : mm;
+        a.rowmax[j] = __longlong_as_double((long long)mm);
     }
 }
 
@@ -114,16 +149,35 @@ __device__ __forceinline__ M2<T> mul(const M2<T> &A, const M2<T> &B)   // A B
             A.m10 * B.m00 + A.m11 * B.m10, A.m10 * B.m01 + A.m11 * B.m11};
 }
 
-// scale by a power of two so that the largest entry is O(1) (ratios unchanged)
+// scale by a power of two so that the largest entry is O(1) (ratios
+// unchanged).  FP64: on the exponent fields, where an entry that falls below
+// the normal range becomes zero (fmax, frexp and ldexp on the FP64 pipe were
+// most of k_factor<double>)
 template <class T>
 __device__ __forceinline__ void renorm(M2<T> &A)
 {
-    T m = fmax(fmax(fabs(A.m00), fabs(A.m01)), fmax(fabs(A.m10), fabs(A.m11)));
-    if (m > T(0) && isfinite(m)) {
-        int e;
-        frexp(m, &e);
-        A.m00 = ldexp(A.m00, -e); A.m01 = ldexp(A.m01, -e);
-        A.m10 = ldexp(A.m10, -e); A.m11 = ldexp(A.m11, -e);
+    if constexpr (sizeof(T) == 8) {
+        double *v = &A.m00;
+        int ex[4], m = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            ex[k] = (__double2hiint(v[k]) >> 20) & 0x7ff;
+            m = max(m, ex[k]);
+        }
+        if (m == 0 || m == 0x7ff) return;                      // all zero, or not finite
+        const int sh = 1022 - m;                               // the largest magnitude into [0.5, 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            v[k] = ex[k] + sh > 0 && ex[k] > 0 ? __hiloint2double(__double2hiint(v[k]) + sh * (1 << 20), __double2loint(v[k]))
+                                               : 0.0;
+    } else {
+        T m = fmax(fmax(fabs(A.m00), fabs(A.m01)), fmax(fabs(A.m10), fabs(A.m11)));
+        if (m > T(0) && isfinite(m)) {
+            int e;
+            frexp(m, &e);
+            A.m00 = ldexp(A.m00, -e); A.m01 = ldexp(A.m01, -e);
+            A.m10 = ldexp(A.m10, -e); A.m11 = ldexp(A.m11, -e);
+        }
     }
 }
 
@@ -197,7 +251,11 @@ __global__ void __launch_bounds__(MAX_THREADS) k_factor(FactorArgs a)
 
     // row of T: diag_i = 1 + eta (ax_i + ax_{i-1} + C_i); coupling of i and
     // i+1: o_i = -eta ax_i (o_{nx-1} couples the last point to the first)
-    const double *ax = a.ax + row, *C = a.C + row;
+    // (the FP32 copies are the FP64 faces rounded, as reading those would, but
+    // a conversion costs an FP64 instruction: eight a point)
+    const T *ax, *C;
+    if constexpr (f64) { ax = a.ax + row; C = a.C + row; }
+    else { ax = a.wax + row; C = a.wC + row; }
     auto diagT = [&](int i) {
         int im = (i == 0) ? nx - 1 : i - 1;
         return T(1) + eta * ((T)ax[i] + (T)ax[im] + (T)C[i]);
@@ -269,7 +327,12 @@ __global__ void __launch_bounds__(MAX_THREADS) k_factor(FactorArgs a)
 
 cudaError_t launch_faces(const FaceArgs &a, int threads, cudaStream_t s)
 {
-    k_faces<<<a.ny, threads, 0, s>>>(a);
+    const size_t smem = 2 * (size_t)a.nx * sizeof(double);
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_faces, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_faces<<<a.ny, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
