@@ -565,6 +565,36 @@ struct Plan {
     std::vector<int> nb;
 };
 
+// Share cap blocks of `lanes` warps, one row each, out to the members of an
+// ensemble.  A member's time is its iterations (about nx) times its phases, and
+// a phase lasts as long as the warp with most rows: rounds = ceil(ny / (lanes
+// nb)) of about nx + 64 points each, and the barrier (about two hundred points'
+// worth).  So blocks go to the slowest member whose next round still fits, as
+// many at a time as take a round off it.  In proportion to the work instead,
+// the 8 members of 512 x 256 in the 64-member ensemble got 26 blocks of 8 warps
+// for their 256 rows, and every phase lasted two rows: the
+// ensemble took 5.33 ms, 4.92 with this in blocks of 4 warps.
+static int share_blocks(int n, const sw_grid *grids, int cap, int lanes, std::vector<int> &nb)
+{
+    auto rounds = [&](int m) { return (grids[m]->ny + lanes * nb[m] - 1) / (lanes * nb[m]); };
+    auto cost = [&](int m) { return grids[m]->nx * (rounds(m) * (grids[m]->nx + 64.0) + 200.0); };
+    std::vector<char> full(n, 0);
+    int used = n;
+    for (int m = 0; m < n; ++m) nb[m] = 1;
+    for (;;) {
+        int slow = -1;
+        for (int m = 0; m < n; ++m)
+            if (!full[m] && (slow < 0 || cost(m) > cost(slow))) slow = m;
+        if (slow < 0) return used;
+        // the fewest blocks that do it in one round less
+        const int r = rounds(slow), per = lanes * (r - 1);
+        const int want = r > 1 ? (grids[slow]->ny + per - 1) / per : 0;
+        if (r == 1 || used + want - nb[slow] > cap) { full[slow] = 1; continue; }
+        used += want - nb[slow];
+        nb[slow] = want;
+    }
+}
+
 static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o, int max_nx, Plan &P)
 {
     const int sms = grids[0]->sms;
@@ -604,8 +634,9 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     if (!P.grid && warp_possible && (o->row_mode == 2 || (o->row_mode == 0 && warp_auto))) {
         // more rows than resident blocks, rows of a power of two of at least
         // 128 points: one warp per row (every SM works on as many rows at once
-        // as it holds warps), on every SM
-        P.threads = MAX_THREADS;
+        // as it holds warps), on every SM; ensembles in blocks of four warps,
+        // so that members share the blocks out more evenly
+        P.threads = n == 1 ? MAX_THREADS : 128;
         P.cc = P.cs = 0;
         // the rows' zonal factors staged in shared memory where they fit
         int bps = 0, bps2 = 0;
@@ -622,9 +653,13 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
         long need = 0;                                          // blocks that give every row its own warp
         for (int m = 0; m < n; ++m) need += (grids[m]->ny + warps - 1) / warps;
         // the register budget of one block per SM unless that leaves rows
-        // without a warp and two blocks fit
+        // without a warp and two blocks fit.  Ensembles with rows of more than
+        // 128 points keep it all the same: their passes spill a quarter of
+        // their registers with half the budget (64 members of 128 x 64 to 512 x
+        // 256 4.93 against 4.41 ms, 40 of 256 x 128 2.09 against 1.89; 64 of 128
+        // x 64 0.65 against 0.71)
         P.minb = 1;
-        if ((long)bps * sms < need && bps2 > bps) { bps = bps2; P.minb = 2; }
+        if ((long)bps * sms < need && bps2 > bps && (n == 1 || max_nx <= 128)) { bps = bps2; P.minb = 2; }
         if (bps >= 1 && n <= bps * sms) {
             if (n == 1) {
                 // the same number of blocks on every SM, as few as give every
@@ -634,25 +669,7 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
                 P.grid = std::min(per_sm * sms, grids[0]->ny);
                 P.nb[0] = P.grid;
             } else {
-                // members share the resident blocks in proportion to their work
-                // (rows per warp x row length x iterations, which grow with nx),
-                // each at most the blocks that give all of its rows a warp
-                const int cap = bps * sms;
-                int used = n;
-                while (used < cap) {
-                    int best = -1;
-                    double bw = 0.0;
-                    for (int m = 0; m < n; ++m) {
-                        const int mcap = std::min(grids[m]->ny, (grids[m]->ny + warps - 1) / warps);
-                        if (P.nb[m] >= mcap) continue;
-                        const double wgt = (double)grids[m]->ny * grids[m]->nx * grids[m]->nx / P.nb[m];
-                        if (wgt > bw) { bw = wgt; best = m; }
-                    }
-                    if (best < 0) break;
-                    ++P.nb[best];
-                    ++used;
-                }
-                P.grid = used;
+                P.grid = share_blocks(n, grids, bps * sms, warps, P.nb);
             }
             P.warp = 1;
             // every member with rows of 1024 or 2048 points (and GCR k <= 4,
