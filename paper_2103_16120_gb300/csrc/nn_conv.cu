@@ -1,5 +1,5 @@
 // nn_conv.cu -- 3x3 convolutions of the learned preconditioner, for the rows that
-// nn_tc.cu does not take (no multiple of 128 points), on the tensor
+// nn_tc.cu does not take (16 or 32 points), on the tensor
 // cores (BF16 operands, FP32 accumulation, mma.sync m16n8k16), as implicit
 // GEMMs over NHWC activations [B][H][W][C]:
 //

@@ -68,7 +68,7 @@ struct WgradArgs {
 
 cudaError_t launch_conv(int cin, int cout, bool dgrad, const ConvArgs &a, int sms, cudaStream_t s);
 // the network's convolutions and input gradients on tcgen05 (nn_tc.cu), with
-// what follows them fused, for rows of a multiple of 128 points (the others
+// what follows them fused, for rows of a multiple of 64 points (the others
 // take launch_conv and the kernels of nn_ops.cu); err (device) is set if a
 // tensor-core wait ran out
 enum ConvStep : int {
@@ -80,10 +80,10 @@ enum ConvStep : int {
     CONV_D5, CONV_D4,   // x -> the adjoint of [up, skip]: coarse part (mask: coarse activation) -> y, skip part -> yf
     CONV_D3, CONV_D2    // x -> yf
 };
-inline bool conv_tc_rows(int W) { return W % 128 == 0; }
+inline bool conv_tc_rows(int W) { return W % 64 == 0; }
 cudaError_t launch_conv_tc(ConvStep step, const ConvArgs &a, int sms, int *err, cudaStream_t s);
 cudaError_t launch_wgrad(int cin, int cout, const WgradArgs &a, int sms, cudaStream_t s);
-// the weight gradient on tcgen05 (nn_tc.cu), rows of a multiple of 128 points
+// the weight gradient on tcgen05 (nn_tc.cu), rows of a multiple of 64 points
 cudaError_t launch_wgrad_tc(int cin, int cout, const WgradArgs &a, int sms, int *err, cudaStream_t s);
 inline cudaError_t launch_wgrad_auto(int cin, int cout, const WgradArgs &a, int sms, int *err, cudaStream_t s)
 {

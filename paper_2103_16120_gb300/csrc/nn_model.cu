@@ -47,7 +47,8 @@ struct sw_model_s {
     void *pmem = nullptr;
     float *master, *m, *v, *gflat;
     bf16 *wf[NLAYERS], *wd[NLAYERS];
-    float *bias[NLAYERS], *dw[NLAYERS], *db[NLAYERS];
+    float *bias[NLAYERS], *dw[NLAYERS], *db[NLAYERS];   // the gradients in one run of grad_bytes
+    size_t grad_bytes = 0;
     int *err;                    // device: a tensor-core wait ran out
     int t = 0;
     Acts A;
@@ -181,10 +182,7 @@ sw_status backward(sw_model_s *M, int B, int H, int W, const float *target, cuda
 {
     Acts &A = M->A;
     const int H1 = H / 2, W1 = W / 2, H2 = H / 4, W2 = W / 4;
-    for (int l = 0; l < NLAYERS; ++l) {
-        NCK(cudaMemsetAsync(M->dw[l], 0, (size_t)9 * LAYER[l].cout_pad * LAYER[l].cin_pad * 4, s));
-        NCK(cudaMemsetAsync(M->db[l], 0, (size_t)LAYER[l].cout_pad * 4, s));
-    }
+    NCK(cudaMemsetAsync(M->dw[0], 0, M->grad_bytes, s));        // every dw and db
     NCK(cudaMemsetAsync(A.scal + 1, 0, sizeof(double), s));
     NCK(launch_loss(A.y, target, A.gy16, A.scal + 1, B, H, W, s));
     auto wg = [&](int l, const bf16 *g, const bf16 *x, int h_, int w_, const bf16 *coarse = nullptr,
@@ -399,10 +397,13 @@ extern "C" sw_status sw_model_create(sw_model *out)
         const size_t nw = (size_t)9 * LAYER[l].cout_pad * LAYER[l].cin_pad;
         M->wf[l] = (bf16 *)p; p += al256(nw * 2);
         M->wd[l] = (bf16 *)p; p += al256(nw * 2);
-        M->dw[l] = (float *)p; p += al256(nw * 4);
         M->bias[l] = (float *)p; p += al256((size_t)LAYER[l].cout_pad * 4);
+    }
+    for (int l = 0; l < NLAYERS; ++l) {
+        M->dw[l] = (float *)p; p += al256((size_t)9 * LAYER[l].cout_pad * LAYER[l].cin_pad * 4);
         M->db[l] = (float *)p; p += al256((size_t)LAYER[l].cout_pad * 4);
     }
+    M->grad_bytes = (size_t)(p - (char *)M->dw[0]);
     *out = M;
     return SW_OK;
 }

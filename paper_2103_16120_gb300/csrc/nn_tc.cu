@@ -1,9 +1,9 @@
 // nn_tc.cu -- the 3x3 convolutions and weight gradients of nn_conv.cu on the
-// fifth-generation tensor cores (tcgen05), for rows of a multiple of 128
+// fifth-generation tensor cores (tcgen05), for rows of a multiple of 64
 // points: BF16 operands from shared memory, FP32 accumulator in tensor memory
 // (TMEM), one thread issuing the MMAs.
 //
-// Tile: 128 consecutive output points of one latitude row (M = 128) x all
+// Tile: 128 (or 64) consecutive output points of one latitude row (M) x the
 // output channels (N = COUT).  Operands use the no-swizzle K-major layout:
 // 16-byte rows (8 channels) of consecutive points (or output channels), one
 // plane per 8 input channels.  In this layout a longitude tap shift is a
@@ -12,7 +12,7 @@
 // 16 ks + 15, A starts at row ky, plane 2 ks, point kx, and one
 // tcgen05.mma of K = 16 accumulates it.
 //
-// A block works down strips of up to 8 rows of one 128-point column.  Input
+// A block works down strips of up to 8 rows of one tile's column.  Input
 // rows sit in a ring of shared-memory slots (the shifted pole rows of the
 // input gradient among them), so every input row of a strip is staged once.
 // Every mbarrier wait is bounded.
@@ -25,8 +25,6 @@ namespace nn {
 
 namespace {
 
-constexpr int TC_TW = 128;                  // points per tile (MMA M)
-constexpr int TC_P = TC_TW + 2;             // staged points per row (halo)
 constexpr unsigned long long TC_WAIT_NS = 200000000ull;   // longest wait: 0.2 s
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -188,8 +186,9 @@ enum Epi : int {
 constexpr int UP_C = 64;                    // channels of the coarse level in both concatenations
 
 // ring slots of input rows, as many as fit beside the weights, at most 8
-template <int CIN, int COUT>
+template <int TW, int CIN, int COUT>
 struct ConvShape {
+    static constexpr int TC_P = TW + 2;                           // staged points of a row (halo)
     static constexpr int KC = CIN / 8;                            // 16-byte channel chunks of a point
     static constexpr size_t WB = (size_t)9 * KC * COUT * 16;      // weights
     static constexpr size_t SLOT = (size_t)KC * TC_P * 16;        // one staged row
@@ -229,15 +228,15 @@ constexpr int ACCS = 4;                     // accumulators: three rows in progr
 // 42; c2 59, 31; c4 354, 86; c5 298, 111; c6 84, 38; d6 96, 47; d5 481, 96; d4
 // 285, 85; d2 87, 35.  An N = 32 MMA takes 38 ns in c5, about twice its operands'
 // shared-memory time: the MMAs bound c4, c5 and d4, the bytes c1, c6 and d6.
-template <int CIN, int CS, int COUT, bool DGRAD, int EPI>
-__global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, COUT>::MINB) k_conv_tc(ConvArgs a, int strip, int *err)
+template <int TW, int CIN, int CS, int COUT, bool DGRAD, int EPI>
+__global__ void __launch_bounds__(ConvShape<TW, CIN, COUT>::THREADS, ConvShape<TW, CIN, COUT>::MINB) k_conv_tc(ConvArgs a, int strip, int *err)
 {
-    typedef ConvShape<CIN, COUT> S;
-    constexpr int KC = S::KC, RING = S::RING, DEPTH = S::DEPTH, SLOT = (int)S::SLOT;
+    typedef ConvShape<TW, CIN, COUT> S;
+    constexpr int KC = S::KC, RING = S::RING, DEPTH = S::DEPTH, SLOT = (int)S::SLOT, TC_P = S::TC_P;
     static_assert(RING >= DEPTH + 2, "a slot is freed once its row, handed over, is done");
     static_assert(COUT % 16 == 0 && ACCS * S::TCOLS <= 512, "");
     constexpr unsigned TCOLS = S::TCOLS;
-    constexpr unsigned ID = idesc_bf16(TC_TW, COUT);
+    constexpr unsigned ID = idesc_bf16(TW, COUT);
     constexpr int EG = S::EG;
     constexpr int CHUNK = EG > 1 || COUT < 32 ? 16 : 32;    // columns read out at once
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -248,7 +247,7 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
     __shared__ int s_bad;
     __shared__ float s_bias[COUT];
     const int H = a.H, W = a.W;
-    const int nseg = W / TC_TW;
+    const int nseg = W / TW;
     const int nstrip = (H + strip - 1) / strip;
     const long nunits = (long)a.B * nseg * nstrip;
     const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
@@ -293,7 +292,7 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
     struct Unit { int b, w0, h0, h1, r0, south, north, nent; };
     auto unit_of = [&](long u) {
         Unit q;
-        q.w0 = (int)(u % nseg) * TC_TW;
+        q.w0 = (int)(u % nseg) * TW;
         q.h0 = (int)((u / nseg) % nstrip) * strip;
         q.b = (int)(u / nseg / nstrip);
         q.h1 = min(q.h0 + strip, H);
@@ -431,13 +430,15 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
     } else {
         // ---- epilogue: thread = output point, warp w reads TMEM lanes 32 (w % 4)
         // .. + 31, group w / 4 every EG-th chunk of columns ----
+        // (M = 64: output point 16 w + l in lane 32 w + l, l < 16)
         const int eg = warp / 4;
+        const bool on = lane < TW / 4;
         int t = 0;
         // pair sums of the even row
         float hold[EPI == EP_ACT_POOL || EPI == EP_UP ? (EPI == EP_UP && COUT > UP_C ? UP_C : COUT) / EG : 1];
         for (long u = blockIdx.x; u < nunits && !*bad; u += gridDim.x) {
             const Unit q = unit_of(u);
-            const int w = q.w0 + (warp & 3) * 32 + lane;
+            const int w = q.w0 + (warp & 3) * (TW / 4) + lane % (TW / 4);
             for (int h = q.h0; h < q.h1; ++h, ++t) {
                 const int buf = t % ACCS;
                 if (!mbar_wait(smem_u32(&s_accf[buf]), (t / ACCS) & 1)) *bad = 1;
@@ -461,19 +462,19 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
                         mbar_arrive(&s_acce[buf]);
                     }
                     if constexpr (EPI == EP_Y) {
-                        a.yf[pix] = v[0] + s_bias[0];
+                        if (on) a.yf[pix] = v[0] + s_bias[0];
                     } else if constexpr (EPI == EP_F32) {
                         float4 *o = (float4 *)(a.yf + pix * ntot + n0 + c0);
 #pragma unroll
                         for (int k = 0; k < CHUNK / 4; ++k)
-                            o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                            if (on) o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
                     } else if constexpr (EPI == EP_UP) {
                         const int col = n0 + c0;
                         if (ci * CHUNK >= UP_C || col >= UP_C) {
                             float4 *o = (float4 *)(a.yf + pix * (ntot - UP_C) + col - UP_C);
 #pragma unroll
                             for (int k = 0; k < CHUNK / 4; ++k)
-                                o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                                if (on) o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
                         } else {
 #pragma unroll
                             for (int k = 0; k < CHUNK; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 1);
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
 #pragma unroll
                                 for (int k = 0; k < CHUNK; ++k) v[k] = hold[hc + k] + v[k];
                                 const size_t at = cpix * UP_C + col + (lane & 1) * (CHUNK / 2);
-                                store_half(v, lane & 1, a.mask + at, a.y + at);
+                                if (on) store_half(v, lane & 1, a.mask + at, a.y + at);
                             }
                         }
                     } else {
@@ -493,7 +494,7 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
                             const uint4 *m = (const uint4 *)(a.mask + pix * ntot + n0 + c0);
 #pragma unroll
                             for (int k = 0; k < CHUNK / 8; ++k) {
-                                const uint4 mq = __ldg(m + k);
+                                const uint4 mq = on ? __ldg(m + k) : make_uint4(0, 0, 0, 0);
                                 const __nv_bfloat16 *mv = (const __nv_bfloat16 *)&mq;
 #pragma unroll
                                 for (int z = 0; z < 8; ++z)
@@ -509,7 +510,7 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
                             __nv_bfloat162 o2[4];
 #pragma unroll
                             for (int z = 0; z < 4; ++z) o2[z] = __floats2bfloat162_rn(v[8 * k + 2 * z], v[8 * k + 2 * z + 1]);
-                            o[k] = *(const uint4 *)o2;
+                            if (on) o[k] = *(const uint4 *)o2;
                         }
                         if constexpr (EPI == EP_ACT_POOL) {
                             // the mean is of the activations as stored
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
 #pragma unroll
                                 for (int k = 0; k < CHUNK; ++k) v[k] = 0.25f * (hold[hc + k] + v[k]);
                                 const size_t at = cpix * ntot + n0 + c0 + (lane & 1) * (CHUNK / 2);
-                                store_half(v, lane & 1, nullptr, a.yp + at);
+                                if (on) store_half(v, lane & 1, nullptr, a.yp + at);
                             }
                         }
                     }
@@ -542,13 +543,13 @@ __global__ void __launch_bounds__(ConvShape<CIN, COUT>::THREADS, ConvShape<CIN, 
                      : "memory");
 }
 
-template <int CIN, int CS, int COUT, bool DGRAD, int EPI>
-static cudaError_t conv_tc_t(const ConvArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
+template <int TW, int CIN, int CS, int COUT, bool DGRAD, int EPI>
+static cudaError_t conv_tw_t(const ConvArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
 {
-    typedef ConvShape<CIN, COUT> S;
+    typedef ConvShape<TW, CIN, COUT> S;
     const size_t smem = S::BYTES;
     int bps = 0;
-    cudaError_t e = occupancy_once<k_conv_tc<CIN, CS, COUT, DGRAD, EPI>>(S::THREADS, smem, &bps);
+    cudaError_t e = occupancy_once<k_conv_tc<TW, CIN, CS, COUT, DGRAD, EPI>>(S::THREADS, smem, &bps);
     if (e != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
     // (the occupancy query answers 1 for every kernel that allocates TMEM)
@@ -557,11 +558,18 @@ static cudaError_t conv_tc_t(const ConvArgs &a, int nsplit, int sms, int *err, c
     // strips of 8 rows (10 input rows each), shorter while blocks would be idle
     const long cap = (long)bps * sms / nsplit > 0 ? (long)bps * sms / nsplit : 1;
     int strip = 8;
-    auto units = [&](int st) { return (long)a.B * (a.W / TC_TW) * ((a.H + st - 1) / st); };
+    auto units = [&](int st) { return (long)a.B * (a.W / TW) * ((a.H + st - 1) / st); };
     while (strip > 2 && units(strip) < cap) strip /= 2;
     const long n = units(strip);
-    k_conv_tc<CIN, CS, COUT, DGRAD, EPI><<<dim3((unsigned)(n < cap ? n : cap), nsplit), S::THREADS, smem, s>>>(a, strip, err);
+    k_conv_tc<TW, CIN, CS, COUT, DGRAD, EPI><<<dim3((unsigned)(n < cap ? n : cap), nsplit), S::THREADS, smem, s>>>(a, strip, err);
     return cudaGetLastError();
+}
+
+template <int CIN, int CS, int COUT, bool DGRAD, int EPI>
+static cudaError_t conv_tc_t(const ConvArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
+{
+    return a.W % 128 == 0 ? conv_tw_t<128, CIN, CS, COUT, DGRAD, EPI>(a, nsplit, sms, err, s)
+                          : conv_tw_t<64, CIN, CS, COUT, DGRAD, EPI>(a, nsplit, sms, err, s);
 }
 
 cudaError_t launch_conv_tc(ConvStep step, const ConvArgs &a, int sms, int *err, cudaStream_t s)
@@ -612,8 +620,9 @@ cudaError_t launch_conv_tc(ConvStep step, const ConvArgs &a, int sms, int *err, 
 // steps; the four warps that read the result out at the end add up the bias
 // gradient meanwhile.  us at 32 samples of 256 x 128, before and now:
 // c1 143, 59; c2 56, 29; c4 178, 112; c5 260, 123; c6 180, 50.
-template <int CIN, int COUT>
+template <int TW, int CIN, int COUT>
 struct WgShape {
+    static constexpr int TC_TW = TW, TC_P = TW + 2;                // points of an input row, of a gradient row (halo)
     static constexpr int KC = CIN / 8, GC = COUT / 8;
     static constexpr int RPG = 128 / CIN > 3 ? 3 : 128 / CIN;      // kernel rows of one A operand
     static constexpr int NG = (3 + RPG - 1) / RPG;                 // A operands per step
@@ -631,15 +640,15 @@ struct WgShape {
     static constexpr int NCOL = NG * 3 * COUT;
 };
 
-template <int CIN, int CS, int COUT>
+template <int TW, int CIN, int CS, int COUT>
 __global__ void __launch_bounds__(288) k_wgrad_tc(WgradArgs a, int strip, int *err)
 {
-    typedef WgShape<CIN, COUT> S;
-    constexpr int KC = S::KC, GC = S::GC, XR = S::XR, GR = S::GR, DEPTH = S::DEPTH;
+    typedef WgShape<TW, CIN, COUT> S;
+    constexpr int KC = S::KC, GC = S::GC, XR = S::XR, GR = S::GR, DEPTH = S::DEPTH, TC_TW = TW, TC_P = S::TC_P;
     static_assert(XR >= 4 && S::NCOL <= 512 && DEPTH < GR, "");
     constexpr unsigned TCOLS = tmem_cols(S::NCOL);
     // BF16 A and B, both MN-major (transpose bits 15 and 16), FP32 accumulator
-    constexpr unsigned ID = idesc_bf16(TC_TW, COUT) | (1u << 15) | (1u << 16);
+    constexpr unsigned ID = idesc_bf16(128, COUT) | (1u << 15) | (1u << 16);
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *Xs = smem, *Gs = smem + S::XBYTES;
     __shared__ __align__(8) unsigned long long s_full[GR], s_empty[GR], s_done;
@@ -674,7 +683,7 @@ __global__ void __launch_bounds__(288) k_wgrad_tc(WgradArgs a, int strip, int *e
     struct Unit { int b, w0, h0, h1; };
     auto unit_of = [&](long u) {
         Unit q;
-        q.w0 = (int)(u % nseg) * TC_TW;
+        q.w0 = (int)(u % nseg) * TW;
         q.h0 = (int)((u / nseg) % nstrip) * strip;
         q.b = (int)(u / nseg / nstrip);
         q.h1 = min(q.h0 + strip, H);
@@ -687,7 +696,7 @@ __global__ void __launch_bounds__(288) k_wgrad_tc(WgradArgs a, int strip, int *e
     if (warp >= 4 && warp < 8) {
         // ---- producers ----
         const int p = threadIdx.x - 128;
-        constexpr int NX = KC, NGP = (TC_P * GC + 127) / 128;      // pieces per thread of a row
+        constexpr int NX = TW * KC / 128, NGP = (TC_P * GC + 127) / 128;      // pieces per thread of a row
         int n = 0, told = 0, done = 0;           // steps staged, handed over, known to be complete
         auto hand_over = [&](int upto) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -861,22 +870,29 @@ __global__ void __launch_bounds__(288) k_wgrad_tc(WgradArgs a, int strip, int *e
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");
 }
 
-template <int CIN, int CS, int COUT>
-static cudaError_t wgrad_tc_t(const WgradArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
+template <int TW, int CIN, int CS, int COUT>
+static cudaError_t wgrad_tw_t(const WgradArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
 {
-    const size_t smem = WgShape<CIN, COUT>::BYTES;
+    const size_t smem = WgShape<TW, CIN, COUT>::BYTES;
     int bps = 0;
-    cudaError_t e = occupancy_once<k_wgrad_tc<CIN, CS, COUT>>(288, smem, &bps);
+    cudaError_t e = occupancy_once<k_wgrad_tc<TW, CIN, CS, COUT>>(288, smem, &bps);
     if (e != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
     // one block per SM; strips of 8 rows, shorter while blocks would be idle
     const long cap = sms / nsplit > 0 ? sms / nsplit : 1;
     int strip = 8;
-    auto units = [&](int st) { return (long)a.B * (a.W / TC_TW) * ((a.H + st - 1) / st); };
+    auto units = [&](int st) { return (long)a.B * (a.W / TW) * ((a.H + st - 1) / st); };
     while (strip > 2 && units(strip) < cap) strip /= 2;
     const long n = units(strip);
-    k_wgrad_tc<CIN, CS, COUT><<<dim3((unsigned)(n < cap ? n : cap), nsplit), 288, smem, s>>>(a, strip, err);
+    k_wgrad_tc<TW, CIN, CS, COUT><<<dim3((unsigned)(n < cap ? n : cap), nsplit), 288, smem, s>>>(a, strip, err);
     return cudaGetLastError();
+}
+
+template <int CIN, int CS, int COUT>
+static cudaError_t wgrad_tc_t(const WgradArgs &a, int nsplit, int sms, int *err, cudaStream_t s)
+{
+    return a.W % 128 == 0 ? wgrad_tw_t<128, CIN, CS, COUT>(a, nsplit, sms, err, s)
+                          : wgrad_tw_t<64, CIN, CS, COUT>(a, nsplit, sms, err, s);
 }
 
 cudaError_t launch_wgrad_tc(int cin, int cout, const WgradArgs &a, int sms, int *err, cudaStream_t s)

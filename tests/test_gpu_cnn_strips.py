@@ -14,12 +14,13 @@ import paper_2103_16120_gb300 as sw  # noqa: E402
 from test_gpu_cnn import dev, inputs, model_with, params, rel  # noqa: E402
 
 
-@pytest.mark.parametrize("B,H,W", [(1, 8, 512), (1, 20, 512), (2, 12, 256), (1, 36, 128), (12, 64, 256)])
+@pytest.mark.parametrize("B,H,W", [(1, 8, 512), (1, 20, 512), (2, 12, 256), (1, 36, 128), (12, 64, 256), (4, 24, 64),
+                                   (1, 12, 768)])
 def test_forward_and_gradients(B, H, W):
     P = params(70 + H)
     m = model_with(P)
     x0 = cnn.round_bf16(inputs(80 + H, B, H, W))
-    if B > 2:                        # samples alternate, so that the oracle runs two
+    if B > 2:                        # (even) samples alternate, so that the oracle runs two
         x0 = np.ascontiguousarray(x0[np.arange(B) % 2])
     target = np.random.default_rng(90 + H).standard_normal((B, H, W))[np.arange(B) % 2 if B > 2 else slice(None)]
     y = torch.empty((B, H, W), dtype=torch.float32, device="cuda")
