@@ -617,7 +617,7 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     const int shapes[2] = {P.threads, narrow};
     for (int sh = 0; sh < (narrow < P.threads ? 2 : 1) && !P.grid && o->row_mode != 2; ++sh) {
         for (int lv = (o->pc == SW_PC_LEARNED ? 1 : 0); lv < 3 && !P.grid; ++lv) {
-            const size_t sm_l = gcr_smem_bytes(o->prec, max_nx, o->k, levels[lv][0], levels[lv][1]);
+            const size_t sm_l = gcr_smem_bytes(o->prec, max_nx, o->k, levels[lv][0], levels[lv][1], shapes[sh]);
             int bps = 0;
             CK(gcr_occupancy(o->prec, o->k, 1, 0, shapes[sh], sm_l, &bps));
             if (bps > 0 && rows_total <= (long)bps * sms) {
@@ -693,9 +693,9 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     if (!P.grid) {
         // blocks own several rows: take the register budget that fits more
         // resident blocks
-        P.smem = gcr_smem_bytes(o->prec, max_nx, o->k, 0, 0);
-        P.cc = P.cs = 0;
         if (n > 1) P.threads = narrow;
+        P.smem = gcr_smem_bytes(o->prec, max_nx, o->k, 0, 0, P.threads);
+        P.cc = P.cs = 0;
         int bps = 0, bps2 = 0;
         CK(gcr_occupancy(o->prec, o->k, 1, 0, P.threads, P.smem, &bps));
         CK(gcr_occupancy(o->prec, o->k, 2, 0, P.threads, P.smem, &bps2));

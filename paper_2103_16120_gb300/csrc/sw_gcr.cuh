@@ -754,6 +754,15 @@ __global__ void __launch_bounds__(MAX_THREADS, MINB) k_gcr(const EnsDesc *__rest
         if (D->cache_state && single) view_state_cache(M, sslot, vc); else view_state_global(M, j0, vc);
     }
     __syncthreads();
+    if constexpr (!Pol::kMixed && !wmode) {
+        // the data-independent half of the row's zonal scans, once per solve
+        if (single && j0 < ny && M.pc >= 3) {
+            double *tab = (double *)(sslot + (D->cache_state ? state_bytes<Pol>(max_nx, M.k) : 0));
+            if (vc.fpad) tri_table<true>(nx, vc.lf, tab);
+            else tri_table<false>(nx, vc.lf, tab);
+            vc.tab = tab;
+        }
+    }
     const comp eta = (comp)(*M.etap);
     GlobalCtl *G = &B->g;
     double *partg = M.part;

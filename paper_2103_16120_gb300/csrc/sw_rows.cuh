@@ -21,6 +21,7 @@ __host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~(size_t)15
 //   red   reduction / scan scratch
 //   const 11 coefficient rows (FP64: 12 weight rows and the diagonal) + 3
 //         padded factor rows of the owned row (optional)
+//   (FP64, after the optional parts) the row's tri_table
 //   state r, L e, e copy, (k+1) p rows, (k+1) L p rows of the owned row (optional)
 // ---------------------------------------------------------------------------
 template <class Pol>
@@ -81,6 +82,7 @@ struct RowView {
     const FT *lf, *invD, *zz;
     bool fpad;
     double gam, ec;
+    const double *tab;              // FP64: tri_table of the row in shared memory, or null
     // owner-only vectors of the row
     typename Pol::res *r;
     VT *Le;
@@ -113,6 +115,7 @@ __device__ __forceinline__ void view_const_global(const MemberDev<Pol> &M, int j
     v.lf = M.lf + row; v.invD = M.invD + row; v.zz = M.zz + row;
     v.fpad = false;
     v.gam = M.gam[j]; v.ec = M.ec[j];
+    v.tab = nullptr;
 }
 
 // copy row j's constants into the block's cache and point the view there
@@ -146,6 +149,7 @@ __device__ void view_const_cache(const MemberDev<Pol> &M, int j, unsigned char *
     v.lf = f; v.invD = f + pl; v.zz = f + 2 * pl;
     v.fpad = true;
     v.gam = g.gam; v.ec = g.ec;
+    v.tab = nullptr;
 }
 
 template <class Pol>
@@ -518,6 +522,13 @@ __device__ __forceinline__ void trisolve_view(typename Pol::comp *sb, int nx, co
                                               typename Pol::comp *sm)
 {
     typedef typename Pol::comp comp;
+    if constexpr (!Pol::kMixed) {
+        if (v.tab) {
+            if (v.fpad) trisolve_tab<true>(sb, nx, v.lf, v.invD, v.zz, v.gam, v.ec, sm, v.tab);
+            else trisolve_tab<false>(sb, nx, v.lf, v.invD, v.zz, v.gam, v.ec, sm, v.tab);
+            return;
+        }
+    }
     if (v.fpad) trisolve_block<comp, typename Pol::fac, true>(sb, nx, v.lf, v.invD, v.zz, (comp)v.gam, (comp)v.ec, sm);
     else trisolve_block<comp, typename Pol::fac, false>(sb, nx, v.lf, v.invD, v.zz, (comp)v.gam, (comp)v.ec, sm);
 }

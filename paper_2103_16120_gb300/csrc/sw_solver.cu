@@ -308,10 +308,10 @@ __global__ void k_fill(double *p, size_t n, double v)
 // host-side launchers (declared in sw_internal.h)
 // ---------------------------------------------------------------------------
 template <class Pol>
-static size_t smem_t(int max_nx, int k, int cache_const, int cache_state)
+static size_t smem_t(int max_nx, int k, int cache_const, int cache_state, int threads)
 {
     return work_bytes<Pol>(max_nx) + (cache_const ? const_bytes<Pol>(max_nx) : 0) +
-           (cache_state ? state_bytes<Pol>(max_nx, k) : 0);
+           (cache_state ? state_bytes<Pol>(max_nx, k) : 0) + (Pol::kMixed ? 0 : (size_t)TRI_TAB * threads * sizeof(double));
 }
 
 template <class Pol>
@@ -326,12 +326,12 @@ size_t gcr_warp_smem_bytes(int prec, int nx, int threads, int stage)
     return prec == 0 ? warp_smem_t<PolFP64>(nx, threads, stage) : warp_smem_t<PolF16>(nx, threads, stage);
 }
 
-size_t gcr_smem_bytes(int prec, int max_nx, int k, int cache_const, int cache_state)
+size_t gcr_smem_bytes(int prec, int max_nx, int k, int cache_const, int cache_state, int threads)
 {
     switch (prec) {
-    case 0: return smem_t<PolFP64>(max_nx, k, cache_const, cache_state);
-    case 1: return smem_t<PolF16>(max_nx, k, cache_const, cache_state);
-    default: return smem_t<PolBF16>(max_nx, k, cache_const, cache_state);
+    case 0: return smem_t<PolFP64>(max_nx, k, cache_const, cache_state, threads);
+    case 1: return smem_t<PolF16>(max_nx, k, cache_const, cache_state, threads);
+    default: return smem_t<PolBF16>(max_nx, k, cache_const, cache_state, threads);
     }
 }
 
