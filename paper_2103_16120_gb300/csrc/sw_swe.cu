@@ -32,6 +32,9 @@ struct Geom {
     int nx, ny;
     double a, dt, grav, omega;
     double inv2dlam, inv2dphi, invdlam, invdphi;   // 1/(2 dlam), 1/(2 dphi), 1/dlam, 1/dphi
+    // uniform factors, formed on the host (as quotients in every thread they were
+    // a quarter of the forcing kernel's FP64 instructions)
+    double delta, inva, ga, hga, hdg;   // dt/2, 1/a, g/a, g/(2a), dt/4 g
     const double *cosr, *sinr, *tanr;   // per latitude row
     const double *invcos;               // 1 / cos(phi_j)
     const double *Crow;                 // C of Eq. 10: a^2 cos(phi_j) / (dt/2)
@@ -74,7 +77,7 @@ __global__ void __launch_bounds__(SWE_THREADS) k_swe_forcing(ForcingArgs A)
     const int nx = A.G.nx, ny = A.G.ny;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nx) return;
-    const double a = A.G.a, delta = 0.5 * A.G.dt, ga = A.G.grav / a, inva = 1.0 / a;
+    const double a = A.G.a, delta = A.G.delta, ga = A.G.ga, inva = A.G.inva;
     for (int j = blockIdx.y; j < ny; j += gridDim.y) {
         const Nbr q = neighbours(i, j, nx, ny);
         const double cj = A.G.cosr[j], sj = A.G.sinr[j], tja = A.G.tanr[j] * inva;
@@ -171,8 +174,7 @@ __global__ void __launch_bounds__(SWE_THREADS) k_swe_coeffs(CoeffArgs A)
     const int nx = A.G.nx, ny = A.G.ny;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nx) return;
-    const double a = A.G.a, g = A.G.grav, delta = 0.5 * A.G.dt;
-    const double hdg = 0.5 * delta * g, hga = 0.5 * g / a;
+    const double a = A.G.a, delta = A.G.delta, hdg = A.G.hdg, hga = A.G.hga;
     for (int j = blockIdx.y; j < ny; j += gridDim.y) {
         const Nbr q = neighbours(i, j, nx, ny);
         const double cj = A.G.cosr[j], ic = A.G.invcos[j];
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(SWE_THREADS) k_swe_recover(RecoverArgs A)
     const int nx = A.G.nx, ny = A.G.ny;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nx) return;
-    const double delta = 0.5 * A.G.dt, hga = 0.5 * A.G.grav / A.G.a;
+    const double delta = A.G.delta, hga = A.G.hga;
     for (int j = blockIdx.y; j < ny; j += gridDim.y) {
         const Nbr q = neighbours(i, j, nx, ny);
         const double p1c = A.phi[q.c] + A.dphi[q.c];
@@ -339,6 +341,8 @@ Geom geom(const sw_swe_s *m)
     const double dlam = 2.0 * M_PI / m->nx, dphi = M_PI / m->ny;
     G.nx = m->nx; G.ny = m->ny; G.a = m->radius;
     G.dt = m->p.dt; G.grav = m->p.gravity; G.omega = m->p.omega;
+    G.delta = 0.5 * G.dt; G.inva = 1.0 / G.a; G.ga = G.grav / G.a; G.hga = 0.5 * G.grav / G.a;
+    G.hdg = 0.5 * G.delta * G.grav;
     G.inv2dlam = 1.0 / (2.0 * dlam); G.inv2dphi = 1.0 / (2.0 * dphi);
     G.invdlam = 1.0 / dlam; G.invdphi = 1.0 / dphi;
     const double *r = m->rows;
