@@ -635,10 +635,9 @@ def _grid(sw, torch, P, dev):
 
 # kernels of one learned solve: the solver's first launch and the graph's first
 # test of the member's state, then per network turn the graph body's kernels
-# (sum of squares and features of r, input packing, 6 convolutions, 2 poolings,
-# 2 upsample + concatenations, output scaling, e stored in the member's format,
-# the resumed solver, the state test)
-LEARNED_LAUNCHES_PER_SOLVE, LEARNED_LAUNCHES_PER_TURN = 2, 17
+# (sum of squares and features of r, input packing, 6 convolutions, output
+# scaling, e stored in the member's format, the resumed solver, the state test)
+LEARNED_LAUNCHES_PER_SOLVE, LEARNED_LAUNCHES_PER_TURN = 2, 13
 
 
 def _time_solves(sw, torch, g, opts, Rs, reps, turns=None):

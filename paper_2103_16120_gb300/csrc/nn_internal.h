@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
+#include <mutex>
+
 namespace nn {
 
 // Resident blocks per SM of kernel KERN for a block size and a dynamic
@@ -22,6 +24,8 @@ inline cudaError_t occupancy_once(int threads, size_t smem, int *bps)
     static Entry seen[16];
     static int n = 0;
     static size_t limit[8] = {};
+    static std::mutex mu;                // host threads with models of their own
+    std::lock_guard<std::mutex> lock(mu);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;

@@ -2,6 +2,8 @@
 // sw_operator_apply and sw_precond_apply, the member initialisation kernels,
 // and the host-side launchers of the persistent GCR kernel, whose
 // instantiations live in sw_gcr_*.cu.
+#include <mutex>
+
 #include "sw_gcr.cuh"
 #include "sw_internal.h"
 
@@ -357,6 +359,8 @@ cudaError_t raise_smem_limit(const void *f, size_t smem)
     struct Lim { const void *f; int dev; size_t smem; };
     static Lim lim[256];
     static int n = 0;
+    static std::mutex mu;                // host threads with grids of their own
+    std::lock_guard<std::mutex> lock(mu);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
