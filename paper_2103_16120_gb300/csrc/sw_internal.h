@@ -86,8 +86,10 @@ size_t gcr_warp_smem_bytes(int prec, int nx, int threads, int stage);
 cudaError_t gcr_occupancy(int prec, int k, int minb, int warp, int threads, size_t smem, int *blocks_per_sm);
 // Raise kernel f's dynamic shared-memory limit on the current device to at
 // least smem bytes.  The limit only grows: a launch recorded in a CUDA graph
-// (the ensemble and learned-preconditioner graphs) keeps its size, so a later
-// launch must not lower the limit below it.
+// (the ensemble and learned-preconditioner graphs) keeps its size, and another
+// host thread may be about to launch f for longer rows, so a later launch must
+// not lower the limit below either.  Every launch with more than 48 KB takes
+// its limit from here.
 cudaError_t raise_smem_limit(const void *f, size_t smem);
 cudaError_t launch_gcr(int prec, int k, int minb, int warp, const EnsDesc *Ddev, int grid, int max_nx, int threads,
                        size_t smem, cudaStream_t s);

@@ -329,7 +329,7 @@ cudaError_t launch_faces(const FaceArgs &a, int threads, cudaStream_t s)
 {
     const size_t smem = 2 * (size_t)a.nx * sizeof(double);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_faces, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = raise_smem_limit((const void *)k_faces, smem);
         if (e != cudaSuccess) return e;
     }
     k_faces<<<a.ny, threads, smem, s>>>(a);
@@ -340,8 +340,7 @@ cudaError_t launch_factor(const FactorArgs &a, bool fp64, int threads, cudaStrea
 {
     const size_t smem = (size_t)a.nx * (fp64 ? sizeof(double) : sizeof(float));
     if (smem > 48 * 1024) {
-        cudaError_t e = fp64 ? cudaFuncSetAttribute(k_factor<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                             : cudaFuncSetAttribute(k_factor<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = raise_smem_limit(fp64 ? (const void *)k_factor<double> : (const void *)k_factor<float>, smem);
         if (e != cudaSuccess) return e;
     }
     if (fp64) k_factor<double><<<a.ny, threads, smem, s>>>(a);

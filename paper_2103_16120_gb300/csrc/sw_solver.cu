@@ -417,7 +417,7 @@ cudaError_t launch_operator_f64(const OpArgs<double> &a, const double *x, double
         return cudaGetLastError();
     }
     size_t smem = 3 * (size_t)a.nx * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_operator<double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit((const void *)k_operator<double, double>, smem);
     if (e != cudaSuccess) return e;
     k_operator<double, double><<<a.ny, threads, smem, s>>>(a, x, y);
     return cudaGetLastError();
@@ -430,7 +430,7 @@ cudaError_t launch_operator_f32(const OpArgs<float> &a, const float *x, float *y
         return cudaGetLastError();
     }
     size_t smem = 3 * (size_t)a.nx * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_operator<float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit((const void *)k_operator<float, float>, smem);
     if (e != cudaSuccess) return e;
     k_operator<float, float><<<a.ny, threads, smem, s>>>(a, x, y);
     return cudaGetLastError();
@@ -466,7 +466,7 @@ template <class Pol>
 static cudaError_t store_e_t(const void *Mdev, const float *ef, int nx, int ny, int threads, cudaStream_t s)
 {
     const size_t smem = work_bytes<Pol>(nx);
-    cudaError_t e = cudaFuncSetAttribute(k_store_e<Pol>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit((const void *)k_store_e<Pol>, smem);
     if (e != cudaSuccess) return e;
     k_store_e<Pol><<<ny, threads, smem, s>>>((const MemberDev<Pol> *)Mdev, ef);
     return cudaGetLastError();
