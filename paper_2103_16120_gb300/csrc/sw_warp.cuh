@@ -859,6 +859,40 @@ struct LeQuad {
     typename Pol::vec lp4[KM][4];
 };
 
+// f(integral_constant<int, ND>) for nd directions: ND = nd where a loop of its
+// own is compiled for that number, else 0, a loop that tests nd.  With no
+// directions yet (the first L(e) of a solve) that is the loop that tests, and
+// it reads none.  Where ONE, the loop for one direction runs instead, on the
+// row that direction_row gives: the code of one more loop makes the kernels
+// specialised for one row length slower (2048 x 1024 30.35 ms a solve with
+// it, 29.84 without), the generic ones not (64-member ensemble 4.54 ms; 4.57
+// with ONE).
+#pragma nv_exec_check_disable
+template <int KM, bool ONE, class F>
+__host__ __device__ __forceinline__ void with_directions(int nd, F f)
+{
+    if constexpr (KM == 4) {
+        switch (ONE && nd == 0 ? 1 : nd) {
+        case 1: f(std::integral_constant<int, 1>{}); break;
+        case 2: f(std::integral_constant<int, 2>{}); break;
+        case 3: f(std::integral_constant<int, 3>{}); break;
+        case 4: f(std::integral_constant<int, 4>{}); break;
+        default: if constexpr (!ONE) f(std::integral_constant<int, 0>{}); break;
+        }
+    } else {
+        f(std::integral_constant<int, 0>{});
+    }
+}
+
+// the L p row that a pass reads as its l-th of nd: of one that does not exist,
+// which nothing has written yet, a row that the pass reads in any case (its
+// sums are not published, phase_slots)
+template <class V>
+__host__ __device__ __forceinline__ const V *direction_row(int l, int nd, const V *Lp, const V *written)
+{
+    return l < nd ? Lp : written;
+}
+
 // L(e) of row j into the row's L e and the inner products <Le,Le>, <r,Le>,
 // <Le,Lp_l>, <r,Lp_l> (phase_le)
 template <class Pol, int KM, int SEL>
@@ -875,9 +909,13 @@ __device__ void wphase_le(const MemberDev<Pol> &M, const MemberCtl &c, const Row
                     qN = qrow(M, M.e, M.e32, M.e_s, j + 1);
     const bool has_n = j < ny - 1, has_s = j > 0;
     const RowCoef<CT> cf = coef_of(v);
+    constexpr bool ONE = SEL > 0 && KM == 4;      // one compiled loop per number of directions only
     const vec *Lpl[KM];
 #pragma unroll
-    for (int l = 0; l < KM; ++l) Lpl[l] = v.Lpb + (size_t)phys_slot(c, M.k, l < nd ? l : 0) * v.vstride;
+    for (int l = 0; l < KM; ++l) {
+        Lpl[l] = v.Lpb + (size_t)phys_slot(c, M.k, l < nd ? l : 0) * v.vstride;
+        if constexpr (ONE) Lpl[l] = direction_row<vec>(l, nd, Lpl[l], v.r);
+    }
     // PL: a plain row (rows_plain), conditions fixed at compile time; ND: the
     // number of directions, so that no load waits behind a test of it (0: nd).
     // 2048 x 1024 32.2 -> 31.7 ms a solve, the 64-member ensemble 4.48 -> 4.40;
@@ -933,16 +971,7 @@ __device__ void wphase_le(const MemberDev<Pol> &M, const MemberCtl &c, const Row
             pass(std::false_type{}, nd_t);
         }
     };
-    if constexpr (KM == 4) {
-        switch (nd) {
-        case 1: row_pass(std::integral_constant<int, 1>{}); break;
-        case 2: row_pass(std::integral_constant<int, 2>{}); break;
-        case 3: row_pass(std::integral_constant<int, 3>{}); break;
-        default: row_pass(std::integral_constant<int, 4>{}); break;
-        }
-    } else {
-        row_pass(std::integral_constant<int, 0>{});
-    }
+    with_directions<KM, ONE>(nd, row_pass);
     SW_TRACE(111);
 }
 
