@@ -560,7 +560,7 @@ extern "C" sw_status sw_precond_apply(sw_grid g, const sw_solve_opts *o, const v
 // linearly with the resolution) and cycle over several rows each, with
 // everything in global memory.
 struct Plan {
-    int grid = 0, cc = 0, cs = 0, threads = 0, minb = 1, warp = 0, stage = 0;
+    int grid = 0, cc = 0, cs = 0, tab = 0, threads = 0, minb = 1, warp = 0, stage = 0;
     size_t smem = 0;
     std::vector<int> nb;
 };
@@ -600,7 +600,14 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     const int sms = grids[0]->sms;
     P.threads = row_threads(max_nx, o->threads_per_row);
     P.nb.assign(n, 1);
-    const int levels[3][2] = {{1, 1}, {1, 0}, {0, 0}};
+    // what a block that owns one row keeps in shared memory (the row's
+    // constants, its owner-only vectors, the products of its scans in FP64 with
+    // a zonal solve), by preference.  The products come first: us per FP64
+    // iteration with constants and products, constants and vectors, products
+    // alone, nothing: 400 x 200 42.1, 45.2, 42.6, 45.5; 520 x 260 49.3, 52.9, 49.1,
+    // 52.3 (the second with one block per SM, which is all that then fits)
+    const bool scans = o->prec == SW_PREC_FP64 && o->pc >= 3;
+    const int levels[6][3] = {{1, 1, 1}, {1, 0, 1}, {0, 0, 1}, {1, 1, 0}, {1, 0, 0}, {0, 0, 0}};
     long rows_total = 0;
     for (int m = 0; m < n; ++m) rows_total += grids[m]->ny;
     // the learned preconditioner ends a launch before every application of
@@ -616,14 +623,15 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     const int narrow = o->threads_per_row > 0 ? P.threads : setup_threads(max_nx);
     const int shapes[2] = {P.threads, narrow};
     for (int sh = 0; sh < (narrow < P.threads ? 2 : 1) && !P.grid && o->row_mode != 2; ++sh) {
-        for (int lv = (o->pc == SW_PC_LEARNED ? 1 : 0); lv < 3 && !P.grid; ++lv) {
-            const size_t sm_l = gcr_smem_bytes(o->prec, max_nx, o->k, levels[lv][0], levels[lv][1], shapes[sh]);
+        for (const int(&lv)[3] : levels) {
+            if (P.grid || (lv[1] && o->pc == SW_PC_LEARNED) || (lv[2] && !scans)) continue;
+            const size_t sm_l = gcr_smem_bytes(o->prec, max_nx, o->k, lv[0], lv[1], lv[2] ? shapes[sh] : 0);
             int bps = 0;
             CK(gcr_occupancy(o->prec, o->k, 1, 0, shapes[sh], sm_l, &bps));
             if (bps > 0 && rows_total <= (long)bps * sms) {
                 for (int m = 0; m < n; ++m) P.nb[m] = grids[m]->ny;
                 P.threads = shapes[sh];
-                P.grid = (int)rows_total; P.cc = levels[lv][0]; P.cs = levels[lv][1]; P.smem = sm_l;
+                P.grid = (int)rows_total; P.cc = lv[0]; P.cs = lv[1]; P.tab = lv[2]; P.smem = sm_l;
             }
         }
     }
@@ -694,12 +702,20 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
         // blocks own several rows: take the register budget that fits more
         // resident blocks
         if (n > 1) P.threads = narrow;
-        P.smem = gcr_smem_bytes(o->prec, max_nx, o->k, 0, 0, P.threads);
+        P.smem = gcr_smem_bytes(o->prec, max_nx, o->k, 0, 0, 0);
         P.cc = P.cs = 0;
         int bps = 0, bps2 = 0;
         CK(gcr_occupancy(o->prec, o->k, 1, 0, P.threads, P.smem, &bps));
         CK(gcr_occupancy(o->prec, o->k, 2, 0, P.threads, P.smem, &bps2));
-        if (bps2 > bps) { bps = bps2; P.minb = 2; }
+        // FP64: two blocks on an SM take 1.6 times (rows of 3000 points and more
+        // 1.9 times) one block's time for a round of rows, so the last round
+        // decides, one against two, us per iteration: 2048 x 1024 437, 392; 2600 x
+        // 1300 766, 691; 2600 x 400 271, 292; 3400 x 1700 1181, 1134; 3400 x 650 506,
+        // 571
+        auto rounds = [&](int b) { return (grids[0]->ny + b * sms - 1) / (b * sms); };
+        const bool one = o->prec == SW_PREC_FP64 && n == 1 && bps > 0 && bps2 > bps &&
+                         rounds(bps) < (max_nx > 2800 ? 1.9 : 1.6) * rounds(bps2);
+        if (bps2 > bps && !one) { bps = bps2; P.minb = 2; }
         if (bps < 1) return fail(SW_ERR_INVALID_ARG, "grid rows too long for the solver kernel");
         const int cap = bps * sms;
         if (n > cap) return fail(SW_ERR_INVALID_ARG, "too many members for one launch on this device");
@@ -717,6 +733,16 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
             ++used;
         }
         P.grid = used;
+        // members that end up with a block for every row (1024 x 512 does, at
+        // four blocks per SM) keep their rows' scan products, where those leave
+        // room for as many blocks
+        bool rows_own = false;
+        for (int m = 0; m < n; ++m) rows_own = rows_own || P.nb[m] >= grids[m]->ny;
+        if (scans && rows_own) {
+            const size_t with = gcr_smem_bytes(o->prec, max_nx, o->k, 0, 0, P.threads);
+            CK(gcr_occupancy(o->prec, o->k, P.minb, 0, P.threads, with, &bps));
+            if (used <= bps * sms) { P.tab = 1; P.smem = with; }
+        }
     }
     return SW_OK;
 }
@@ -728,6 +754,7 @@ static void fill_desc(EnsDesc &D, int n, const sw_grid *grids, const Plan &P, sw
     D.grid = P.grid;
     D.cache_const = P.cc;
     D.cache_state = P.cs;
+    D.scan_table = P.tab;
     D.warp_rows = P.warp != 0;
     D.warp_stage = P.stage;
     D.cta_begin[0] = 0;
@@ -798,6 +825,7 @@ static sw_status solve_one_async(sw_grid g, const sw_solve_opts *o, const double
     a.nb0 = P.nb[0];
     a.cache_const = P.cc;
     a.cache_state = P.cs;
+    a.scan_table = P.tab;
     a.warp_rows = P.warp != 0;
     a.warp_stage = P.stage;
     CK(launch_init_one(a, s));

@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(MAX_THREADS, MINB) k_gcr(const EnsDesc *__rest
     __syncthreads();
     if constexpr (!Pol::kMixed && !wmode) {
         // the data-independent half of the row's zonal scans, once per solve
-        if (single && j0 < ny && M.pc >= 3) {
+        if (D->scan_table && single && j0 < ny) {
             double *tab = (double *)(sslot + (D->cache_state ? state_bytes<Pol>(max_nx, M.k) : 0));
             if (vc.fpad) tri_table<true>(nx, vc.lf, tab);
             else tri_table<false>(nx, vc.lf, tab);

@@ -80,7 +80,9 @@ cudaError_t launch_split_residual(const SplitResidualArgs &a, cudaStream_t s);
 cudaError_t launch_faces(const FaceArgs &a, int threads, cudaStream_t s);
 cudaError_t launch_weights(const WeightArgs &a, cudaStream_t s);
 cudaError_t launch_factor(const FactorArgs &a, bool fp64, int threads, cudaStream_t s);
-size_t gcr_smem_bytes(int prec, int max_nx, int k, int cache_const, int cache_state, int threads);
+// shared memory of the block-per-row mode; scan_table (FP64): with the tables of
+// that many threads' scans (tri_table)
+size_t gcr_smem_bytes(int prec, int max_nx, int k, int cache_const, int cache_state, int scan_table);
 // shared memory of the warp-per-row mode (0 when nx does not allow it)
 size_t gcr_warp_smem_bytes(int prec, int nx, int threads, int stage);
 cudaError_t gcr_occupancy(int prec, int k, int minb, int warp, int threads, size_t smem, int *blocks_per_sm);

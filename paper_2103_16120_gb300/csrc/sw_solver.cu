@@ -310,10 +310,10 @@ __global__ void k_fill(double *p, size_t n, double v)
 // host-side launchers (declared in sw_internal.h)
 // ---------------------------------------------------------------------------
 template <class Pol>
-static size_t smem_t(int max_nx, int k, int cache_const, int cache_state, int threads)
+static size_t smem_t(int max_nx, int k, int cache_const, int cache_state, int scan_table)
 {
     return work_bytes<Pol>(max_nx) + (cache_const ? const_bytes<Pol>(max_nx) : 0) +
-           (cache_state ? state_bytes<Pol>(max_nx, k) : 0) + (Pol::kMixed ? 0 : (size_t)TRI_TAB * threads * sizeof(double));
+           (cache_state ? state_bytes<Pol>(max_nx, k) : 0) + (Pol::kMixed ? 0 : (size_t)TRI_TAB * scan_table * sizeof(double));
 }
 
 template <class Pol>
@@ -328,12 +328,12 @@ size_t gcr_warp_smem_bytes(int prec, int nx, int threads, int stage)
     return prec == 0 ? warp_smem_t<PolFP64>(nx, threads, stage) : warp_smem_t<PolF16>(nx, threads, stage);
 }
 
-size_t gcr_smem_bytes(int prec, int max_nx, int k, int cache_const, int cache_state, int threads)
+size_t gcr_smem_bytes(int prec, int max_nx, int k, int cache_const, int cache_state, int scan_table)
 {
     switch (prec) {
-    case 0: return smem_t<PolFP64>(max_nx, k, cache_const, cache_state, threads);
-    case 1: return smem_t<PolF16>(max_nx, k, cache_const, cache_state, threads);
-    default: return smem_t<PolBF16>(max_nx, k, cache_const, cache_state, threads);
+    case 0: return smem_t<PolFP64>(max_nx, k, cache_const, cache_state, scan_table);
+    case 1: return smem_t<PolF16>(max_nx, k, cache_const, cache_state, scan_table);
+    default: return smem_t<PolBF16>(max_nx, k, cache_const, cache_state, scan_table);
     }
 }
 
@@ -516,6 +516,7 @@ __global__ void k_init_one(const __grid_constant__ InitOneArgs a)
         D->grid = a.grid;
         D->cache_const = a.cache_const;
         D->cache_state = a.cache_state;
+        D->scan_table = a.scan_table;
         D->warp_rows = a.warp_rows;
         D->warp_stage = a.warp_stage;
         D->stats = a.stats;

@@ -1,0 +1,70 @@
+"""The launch shape that the solver picks, read from a CUDA graph that the call
+is recorded in (nothing runs)."""
+import ctypes as C
+
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2103_16120_gb300 as sw  # noqa: E402
+
+
+class KernelNodeParams(C.Structure):
+    _fields_ = [("func", C.c_void_p), ("grid", C.c_uint * 3), ("block", C.c_uint * 3), ("smem", C.c_uint),
+                ("params", C.c_void_p), ("extra", C.c_void_p)]
+
+
+def solver_launch(nx, ny, **opts):
+    """(blocks, threads, dynamic shared memory) of the solver kernel for a grid:
+    of the recorded kernels the one with most shared memory"""
+    P = synth.problem(nx, ny, 7)
+    g = sw.sw_grid_create(nx, ny)
+    sw.sw_elliptic_set_coeffs(g, *[torch.as_tensor(P[k], device="cuda") for k in sw.COEFF_KEYS])
+    R = torch.as_tensor(P["R"], device="cuda")
+    phi = torch.zeros_like(R)
+    o = sw.sw_solve_opts_default(max_iters=1, **opts)
+    sw.sw_gcr_solve(g, o, R, phi)                      # the workspace exists from here on
+    torch.cuda.synchronize()
+    rt, s = C.CDLL("libcudart.so.13"), torch.cuda.Stream()
+    graph, n, p = C.c_void_p(), C.c_size_t(), KernelNodeParams()
+    st = C.c_void_p(s.cuda_stream)
+    assert rt.cudaStreamBeginCapture(st, 2) == 0       # relaxed
+    try:
+        sw.sw_ensemble_solve_async([g], o, [R], [phi], stream=s)
+    finally:
+        assert rt.cudaStreamEndCapture(st, C.byref(graph)) == 0
+    assert rt.cudaGraphGetNodes(graph, None, C.byref(n)) == 0
+    nodes = (C.c_void_p * n.value)()
+    assert rt.cudaGraphGetNodes(graph, nodes, C.byref(n)) == 0
+    found = []
+    for q in nodes:
+        kind = C.c_int()
+        assert rt.cudaGraphNodeGetType(C.c_void_p(q), C.byref(kind)) == 0
+        if kind.value == 0 and rt.cudaGraphKernelNodeGetParams(C.c_void_p(q), C.byref(p)) == 0:
+            found.append((p.smem, p.grid[0], p.block[0]))
+    assert rt.cudaGraphDestroy(graph) == 0
+    smem, blocks, threads = max(found)
+    return blocks, threads, smem
+
+
+# rows of 2600 to 3400 points: two blocks fit an SM unless the launch counts the
+# scan products, which blocks of several rows do not keep; fewer rows than a
+# second block per SM pays for (three rounds of rows against two) stay with one
+@pytest.mark.parametrize("nx,ny,per_sm", [(2048, 1024, 2), (2600, 1300, 2), (3400, 800, 2), (2600, 400, 1),
+                                          (3400, 400, 1)])
+def test_fp64_blocks_per_sm_of_several_rows_each(nx, ny, per_sm):
+    blocks, threads, _ = solver_launch(nx, ny, prec=sw.SW_PREC_FP64)
+    assert threads == 256
+    assert blocks == per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def test_scan_products_are_kept_where_they_are_used():
+    """One row per block, with two blocks an SM at most and with four: 14 doubles
+    a thread for the zonal solve of option 3, none for option 1."""
+    for ny in (64, 512):
+        blocks, threads, smem3 = solver_launch(1024, ny, prec=sw.SW_PREC_FP64)
+        assert blocks == ny
+        assert smem3 - solver_launch(1024, ny, prec=sw.SW_PREC_FP64, pc=sw.SW_PC_DIAG)[2] == 14 * 8 * threads
