@@ -46,6 +46,7 @@ struct sw_grid_s {
     double *gam32, *ec32;          // per row, of the FP32 zonal factors
     double *wgt;                   // nine-point weights of the FP64 policy (NWGT fields)
     bool f64_valid;                // the FP64 zonal factors and weights match the coefficients and eta
+    bool recorded;                 // a graph holds a call that sets them: f64_valid says nothing any more
     float *wax, *wcx, *wbx, *way, *wcy, *wby, *wC, *wdiag, *lf32, *invD32, *zz32;
     // the zonal factors transposed per row for the warp-per-row solver (rows
     // of a power of two of at least 128 points; null otherwise)
@@ -331,10 +332,23 @@ static FactorArgs factor_args(const sw_grid_s *g)
     return f;
 }
 
+static sw_status is_recording(cudaStream_t s, bool &recording)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(s, &cap));
+    recording = cap != cudaStreamCaptureStatusNone;
+    return SW_OK;
+}
+
 // new coefficients or eta: the FP32 zonal factors (mixed solvers) now; the
-// FP64 ones and the nine-point weights when an FP64 solve or preconditioner needs them (ensure_f64)
+// FP64 ones and the nine-point weights when an FP64 solve or preconditioner
+// needs them (ensure_f64).  Recorded in a CUDA graph, the change comes with
+// every replay, which the host does not see.
 static sw_status refactor(sw_grid g, cudaStream_t s)
 {
+    bool recording = false;
+    if (sw_status st = is_recording(s, recording)) return st;
+    g->recorded = g->recorded || recording;
     CK(launch_factor(factor_args(g), false, setup_threads(g->nx), s));
     g->f64_valid = false;
     return SW_OK;
@@ -342,16 +356,18 @@ static sw_status refactor(sw_grid g, cudaStream_t s)
 
 // the FP64 zonal factors and weights, stream-ordered before the FP64 work that follows on
 // s.  Inside a CUDA graph capture they are always recorded: a replay cannot
-// know whether the coefficients changed since.
+// know whether the coefficients changed since.  For the same reason a grid
+// whose coefficients or eta a graph sets forms them at every call: a solve
+// with the weights of the coefficients before a replay would solve another
+// problem.
 static sw_status ensure_f64(sw_grid g, cudaStream_t s)
 {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(s, &cap));
-    const bool recorded = (cap != cudaStreamCaptureStatusNone);
-    if (g->f64_valid && !recorded) return SW_OK;
+    bool recording = false;
+    if (sw_status st = is_recording(s, recording)) return st;
+    if (g->f64_valid && !recording && !g->recorded) return SW_OK;
     CK(launch_factor(factor_args(g), true, row_threads(g->nx), s));
     CK(launch_weights(WeightArgs{g->nx, g->ny, g->ax, g->cx, g->bx, g->ay, g->cy, g->by, g->C, g->wgt}, s));
-    if (!recorded) g->f64_valid = true;
+    if (!recording) g->f64_valid = true;
     return SW_OK;
 }
 
