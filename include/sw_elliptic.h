@@ -164,7 +164,11 @@ void sw_solve_opts_default(sw_solve_opts *o);
 
 /* Create a grid of nx x ny points on a sphere of the given radius (m).
  * nx even, 4 <= nx <= 4096, 2 <= ny <= 65536.  The grid takes the current
- * CUDA device.  Allocates the coefficient storage. */
+ * CUDA device.  Allocates the coefficient storage: 132 bytes per point, 168
+ * where nx is a power of two of at least 128.  FP64 solves and preconditioners
+ * take L from weights of 96 bytes per point more: up to 1 MiB of them are
+ * allocated here, larger ones by the grid's first FP64 call (SW_ERR_OOM if that
+ * fails), which may be one that is being captured. */
 sw_status sw_grid_create(int nx, int ny, double radius, sw_grid *out);
 sw_status sw_grid_destroy(sw_grid g);
 
@@ -250,8 +254,9 @@ sw_status sw_ensemble_solve(int n, const sw_grid *grids, const sw_solve_opts *o,
  * too: each grid stages the descriptors of a call in one of four pinned host
  * slots, and a call waits on the host only while the stream is four calls
  * behind.  Nothing is allocated once each grid's workspace exists, i.e.
- * after one solve with the same precision and k (or an attached workspace),
- * so the call can then be recorded in a CUDA graph and replayed.  With one
+ * after one solve with the same precision and k (or an attached workspace;
+ * FP64 then still allocates its weights, see sw_grid_create), so the call can
+ * then be recorded in a CUDA graph and replayed.  With one
  * member (n = 1) the descriptors travel as kernel parameters, with no host
  * staging and no copies, and a recorded call keeps them for the graph's
  * lifetime.  With more, a recorded call stages into a slot of its own, which
@@ -324,6 +329,8 @@ sw_status sw_model_target(sw_model m, sw_grid g, const float *r, const float *e,
  * vectors live.  They are not in the grid's workspace, and nothing is
  * allocated for them.  They go in one fixed array of SW_NOALLOC_SCRATCH_BYTES
  * per device, built into the library and shared by every grid on that device.
+ * (FP64 solves of a grid that has no weights yet, see sw_grid_create, form
+ * them in a second such array, at every call.)
  * The call makes no device or pinned-host allocation of any kind.  On a
  * failing call, the error message text may use the host heap.
  *  - Size limit: sw_grid_workspace_bytes(g, o) must not exceed

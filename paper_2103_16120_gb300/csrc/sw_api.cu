@@ -44,9 +44,15 @@ struct sw_grid_s {
     void *cmem;
     double *ax, *cx, *bx, *ay, *cy, *by, *C, *diag, *lf, *invD, *zz, *gam, *ec, *rowmax, *eta;
     double *gam32, *ec32;          // per row, of the FP32 zonal factors
-    double *wgt;                   // nine-point weights of the FP64 policy (NWGT fields)
-    bool f64_valid;                // the FP64 zonal factors and weights match the coefficients and eta
-    bool recorded;                 // a graph holds a call that sets them: f64_valid says nothing any more
+    bool f64_valid;                // the FP64 zonal factors match the coefficients and eta
+    // nine-point weights of the FP64 policy (NWGT fields): with the coefficients
+    // (small grids), else, from the first FP64 call on, behind the grid's own
+    // workspace (wgt_in_ws) or in wmem
+    double *wgt;
+    void *wmem;
+    bool wgt_in_ws;
+    bool wgt_valid;                // wgt matches the coefficients
+    bool recorded;                 // a graph holds a call that sets them: the two say nothing any more
     float *wax, *wcx, *wbx, *way, *wcy, *wby, *wC, *wdiag, *lf32, *invD32, *zz32;
     // the zonal factors transposed per row for the warp-per-row solver (rows
     // of a power of two of at least 128 points; null otherwise)
@@ -127,6 +133,8 @@ static int setup_threads(int nx)
 
 static size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
+static size_t weight_bytes(const sw_grid_s *g) { return (size_t)NWGT * g->N * sizeof(double); }
+
 extern "C" void sw_solve_opts_default(sw_solve_opts *o)
 {
     if (!o) return;
@@ -163,8 +171,12 @@ extern "C" sw_status sw_grid_create(int nx, int ny, double radius, sw_grid *out)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device);
     size_t N = g->N;
     const bool wt = warp_rows_ok(nx);
+    // the weights of a small grid come with it: at most 1 MiB, and where they had
+    // to be allocated later the first FP64 solve of a 128 x 64 grid took 245 us, 152
+    // so
+    const bool small = weight_bytes(g) <= (1u << 20);
     size_t bytes = 11 * al(N * 8) + 5 * al((size_t)ny * 8) + al(8) + 11 * al(N * 4) + (wt ? 3 * (al(N * 8) + al(N * 4)) : 0) +
-                   al((size_t)NWGT * N * 8);
+                   (small ? al(weight_bytes(g)) : 0);
     if (e == cudaSuccess) e = cudaMalloc(&g->cmem, bytes);
     if (e == cudaSuccess) e = cudaMalloc((void **)&g->blk, sizeof(SolverBlock));
     if (e == cudaSuccess) e = cudaMalloc((void **)&g->desc, sizeof(EnsDesc));
@@ -203,7 +215,7 @@ extern "C" sw_status sw_grid_create(int nx, int ny, double radius, sw_grid *out)
         for (auto q : {&g->lfT, &g->invDT, &g->zzT}) { *q = (double *)p; p += al(N * 8); }
         for (auto q : {&g->lf32T, &g->invD32T, &g->zz32T}) { *q = (float *)p; p += al(N * 4); }
     }
-    g->wgt = (double *)p;
+    if (small) g->wgt = (double *)p;
     *out = g;
     return SW_OK;
 }
@@ -213,6 +225,7 @@ extern "C" sw_status sw_grid_destroy(sw_grid g)
     if (!g) return fail(SW_ERR_INVALID_ARG, "sw_grid_destroy: NULL grid");
     cudaFree(g->cmem);
     if (g->split_mem) cudaFree(g->split_mem);
+    if (g->wmem) cudaFree(g->wmem);
     cudaFree(g->blk);
     cudaFree(g->desc);
     cudaFreeHost(g->h_desc);
@@ -293,11 +306,20 @@ extern "C" sw_status sw_grid_workspace_bytes(sw_grid g, const sw_solve_opts *o, 
     return SW_OK;
 }
 
+// free the grid's own workspace, and the weights with it if they lie there
+static void drop_ws(sw_grid g)
+{
+    if (g->ws_owned && g->ws) cudaFree(g->ws);
+    g->ws = nullptr;
+    g->ws_bytes = 0;
+    if (g->wgt_in_ws) { g->wgt = nullptr; g->wgt_in_ws = g->wgt_valid = false; }
+}
+
 extern "C" sw_status sw_grid_attach_workspace(sw_grid g, void *dev_ptr, size_t bytes)
 {
     if (!g) return fail(SW_ERR_INVALID_ARG, "sw_grid_attach_workspace: NULL grid");
     if (dev_ptr && ((uintptr_t)dev_ptr & 255)) return fail(SW_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
-    if (g->ws_owned && g->ws) cudaFree(g->ws);
+    drop_ws(g);
     g->ws = dev_ptr;
     g->ws_bytes = dev_ptr ? bytes : 0;
     g->ws_owned = false;
@@ -310,10 +332,13 @@ static sw_status ensure_ws(sw_grid g, int prec, int k)
     if (g->ws && g->ws_bytes >= need) return SW_OK;
     if (g->ws && !g->ws_owned)
         return fail(SW_ERR_INVALID_ARG, "attached workspace is smaller than sw_grid_workspace_bytes");
-    if (g->ws) { cudaFree(g->ws); g->ws = nullptr; g->ws_bytes = 0; }
-    CK(cudaMalloc(&g->ws, need));
+    // FP64: the weights of L in the same allocation
+    const bool with_wgt = g->wgt_in_ws || (prec == SW_PREC_FP64 && !g->wgt);
+    drop_ws(g);
+    CK(cudaMalloc(&g->ws, need + (with_wgt ? weight_bytes(g) : 0)));
     g->ws_bytes = need;
     g->ws_owned = true;
+    if (with_wgt) { g->wgt = (double *)((char *)g->ws + need); g->wgt_in_ws = true; }
     return SW_OK;
 }
 
@@ -359,15 +384,37 @@ static sw_status refactor(sw_grid g, cudaStream_t s)
 // know whether the coefficients changed since.  For the same reason a grid
 // whose coefficients or eta a graph sets forms them at every call: a solve
 // with the weights of the coefficients before a replay would solve another
-// problem.
-static sw_status ensure_f64(sw_grid g, cudaStream_t s)
+// problem.  lent: device memory for the weights, which are then formed there
+// at every call; otherwise they lie with the grid's own data: 96 bytes a point
+// that grids above 1 MiB of them without FP64 calls do not pay for.
+static sw_status ensure_f64(sw_grid g, cudaStream_t s, double *lent = nullptr)
 {
     bool recording = false;
     if (sw_status st = is_recording(s, recording)) return st;
-    if (g->f64_valid && !recording && !g->recorded) return SW_OK;
-    CK(launch_factor(factor_args(g), true, row_threads(g->nx), s));
-    CK(launch_weights(WeightArgs{g->nx, g->ny, g->ax, g->cx, g->bx, g->ay, g->cy, g->by, g->C, g->wgt}, s));
-    if (!recording) g->f64_valid = true;
+    if (!lent && !g->wgt) {
+        // an allocation is no work of the stream, and may be made while s (or
+        // another thread's stream) is being captured
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        cudaError_t e = cudaMalloc(&g->wmem, weight_bytes(g));
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            g->wmem = nullptr;
+            return cuda_fail(e, "operator weights of an FP64 call");
+        }
+        g->wgt = (double *)g->wmem;
+    }
+    const bool anew = recording || g->recorded;
+    if (!g->f64_valid || anew) {
+        CK(launch_factor(factor_args(g), true, row_threads(g->nx), s));
+        if (!recording) g->f64_valid = true;
+    }
+    if (lent || !g->wgt_valid || anew) {
+        double *w = lent ? lent : g->wgt;
+        CK(launch_weights(WeightArgs{g->nx, g->ny, g->ax, g->cx, g->bx, g->ay, g->cy, g->by, g->C, w}, s));
+        if (!lent && !recording) g->wgt_valid = true;
+    }
     return SW_OK;
 }
 
@@ -388,6 +435,7 @@ extern "C" sw_status sw_elliptic_set_coeffs(sw_grid g, const double *A11, const 
     a.wax = g->wax; a.wcx = g->wcx; a.wbx = g->wbx; a.way = g->way; a.wcy = g->wcy; a.wby = g->wby; a.wC = g->wC;
     a.wdiag = g->wdiag; a.rowmax = g->rowmax;
     CK(launch_faces(a, std::min(MAX_THREADS, (g->nx + 31) / 32 * 32), s));
+    g->wgt_valid = false;
     sw_status st = refactor(g, s);
     if (st) return st;
     g->has_coeffs = true;
@@ -1112,11 +1160,12 @@ extern "C" sw_status sw_ensemble_solve(int n, const sw_grid *grids, const sw_sol
 // kernel and launch shape as sw_gcr_solve, with no allocation
 // ---------------------------------------------------------------------------
 template <class Pol>
-static void fill_member_noalloc(const sw_grid_s *g, void *scratch, const sw_solve_opts *o, const double *R,
-                                double *phi, void *out)
+static void fill_member_noalloc(const sw_grid_s *g, void *scratch, double *weights, const sw_solve_opts *o,
+                                const double *R, double *phi, void *out)
 {
     sw_grid_s view = *g;          // a copy of the handle that points at the scratch
     view.ws = scratch;
+    view.wgt = weights;
     MemberDev<Pol> M;
     fill_member<Pol>(&view, o, R, phi, M);
     std::memcpy(out, &M, sizeof(M));
@@ -1144,18 +1193,20 @@ extern "C" sw_status sw_gcr_solve_noalloc(sw_grid g, const sw_solve_opts *o, con
         return fail(SW_ERR_INVALID_ARG, msg);
     }
     void *scratch = nullptr;
-    size_t cap = 0;
-    CK(noalloc_scratch(&scratch, &cap));
+    // FP64: the grid's own weights if an earlier call has allocated them
+    double *lent = nullptr;
+    CK(noalloc_scratch(&scratch, o->prec == SW_PREC_FP64 && !g->wgt ? &lent : nullptr));
     cudaStream_t s = (cudaStream_t)stream;
     if (o->eta > 0.0 && o->eta != g->eta_explicit) {
         g->eta_explicit = o->eta;
         if ((st = refactor(g, s))) return st;
     }
     alignas(16) unsigned char hbuf[sizeof(SolverBlock::dev)];
-    if (o->prec == SW_PREC_FP64 && (st = ensure_f64(g, s))) return st;
-    if (o->prec == SW_PREC_FP64) fill_member_noalloc<PolFP64>(g, scratch, o, R, phi, hbuf);
-    else if (o->prec == SW_PREC_MIXED_FP16) fill_member_noalloc<PolF16>(g, scratch, o, R, phi, hbuf);
-    else fill_member_noalloc<PolBF16>(g, scratch, o, R, phi, hbuf);
+    if (o->prec == SW_PREC_FP64 && (st = ensure_f64(g, s, lent))) return st;
+    double *w = lent ? lent : g->wgt;
+    if (o->prec == SW_PREC_FP64) fill_member_noalloc<PolFP64>(g, scratch, w, o, R, phi, hbuf);
+    else if (o->prec == SW_PREC_MIXED_FP16) fill_member_noalloc<PolF16>(g, scratch, w, o, R, phi, hbuf);
+    else fill_member_noalloc<PolBF16>(g, scratch, w, o, R, phi, hbuf);
     CK(cudaMemcpyAsync(g->blk->dev, hbuf, member_dev_bytes(o->prec), cudaMemcpyHostToDevice, s));
     MemberCtl c;
     std::memset(&c, 0, sizeof(c));

@@ -150,7 +150,8 @@ struct GridView {
 };
 GridView grid_view(const ::sw_grid_s *g);
 
-// the fixed scratch of sw_gcr_solve_noalloc on the current device (sw_static.cu)
-cudaError_t noalloc_scratch(void **ptr, size_t *bytes);
+// the fixed scratch of sw_gcr_solve_noalloc on the current device and (weights
+// not null) the fixed array for an FP64 solve's weights (sw_static.cu)
+cudaError_t noalloc_scratch(void **ptr, double **weights);
 
 } // namespace sw
