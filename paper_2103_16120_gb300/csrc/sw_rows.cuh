@@ -338,9 +338,13 @@ __device__ __forceinline__ bool stencil4_ok(const RowCoef<CT> &c, int nx)
 // the flux form above takes 30 (P^M) and 33 (L) per point, the weights 9 and
 // 17.  One FP64 iteration measured 398 against 577 us at 2048 x 1024,
 // 132 against 179 at 1024 x 512, 46 against 58 at 512 x 256 (the weights are 96
-// bytes a point more to hold, 16 more to read in a stage and in L).  L is written with the differences to the centre, which keeps the
-// cancellation of the flux form (a constant field gives W_SUM times it, the
-// fluxes' own b and C terms); P^M only enters multiplied by eta = 1 /
+// bytes a point more to hold, 16 more to read in a stage and in L).  L is written
+// with the differences to the centre, which keeps the cancellation of the flux
+// form (a constant field gives W_SUM times it, the fluxes' own b and C terms).
+// That term is most of L x and is added last, as C x is in the flux form:
+// added first, each of the eight sums after it was rounded at its size, and L
+// of a smooth field was off by 1.3e-16 of its norm, 0.56e-16 now (the fluxes
+// 0.41e-16).  P^M only enters multiplied by eta = 1 /
 // max|diag(P^M)| and added to the field it acts on, where the plain sum's
 // rounding is that of the field.  The weights of a point are loaded before
 // its sums start.  Wt[9]: the N, S, NE, NW, SE, SW weights, then E, W and the
@@ -362,10 +366,10 @@ __device__ __forceinline__ double stencil9(const double *S, const double *X, con
     const int ie = (i + 1 == nx) ? 0 : i + 1, iw = (i == 0) ? nx - 1 : i - 1;
     const double xc = X[i], o = FULL ? xc : 0.0;
     const double x[8] = {N[i], S[i], N[ie], N[iw], S[ie], S[iw], X[ie], X[iw]};
-    double s = Wt[8] * xc;
+    double s = FULL ? 0.0 : Wt[8] * xc;
 #pragma unroll
     for (int a = 0; a < 8; ++a) s = fma(Wt[a], FULL ? x[a] - o : x[a], s);
-    return s;
+    return FULL ? fma(Wt[8], xc, s) : s;
 }
 
 template <class Pol>
