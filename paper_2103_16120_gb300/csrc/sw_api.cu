@@ -700,8 +700,8 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
         }
     }
     // the automatic choice takes one warp per row for the mixed precisions;
-    // the FP64 solver, bound by FP64 instruction issue, measured no faster
-    // with it (582 against 572 us per iteration at 2048 x 1024)
+    // the FP64 solver, bound by FP64 instruction issue, is slower with it (455
+    // against 394 us per iteration at 2048 x 1024, 145 against 113 at 1024 x 512)
     const bool warp_auto = o->prec != SW_PREC_FP64;
     if (!P.grid && warp_possible && (o->row_mode == 2 || (o->row_mode == 0 && warp_auto))) {
         // more rows than resident blocks, rows of a power of two of at least

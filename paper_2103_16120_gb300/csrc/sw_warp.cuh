@@ -217,6 +217,42 @@ __device__ __forceinline__ void apply4(const Coef4<CT> &k, const T (&xc)[6], con
     }
 }
 
+// The nine-point form of the stencils for the FP64 policy (stencil9, the same
+// sums in the same order) at points i0 .. i0 + 3.  With the faces' fluxes
+// (apply4) an iteration took 565 us at 2048 x 1024, 455 now; at 512 x 256 83, 68.
+struct Wgt4 {
+    double w[9][4];
+};
+
+template <bool FULL, class RV>
+__device__ __forceinline__ void weights4(const RV &v, int i0, Wgt4 &k)
+{
+#pragma unroll
+    for (int a = 0; a < 6; ++a) ldg4(v.w + a * v.wstride + i0, k.w[a]);
+    ldg4(v.w + (FULL ? W_E : W_ME) * v.wstride + i0, k.w[6]);
+    ldg4(v.w + (FULL ? W_W : W_MW) * v.wstride + i0, k.w[7]);
+    ldg4(v.w + (FULL ? W_SUM : W_MC) * v.wstride + i0, k.w[8]);
+}
+
+template <bool FULL>
+__device__ __forceinline__ void apply9(const Wgt4 &k, const double (&xc)[6], const double (&xn)[6],
+                                       const double (&xs)[6], double (&y)[4])
+{
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int q = u + 1;
+        const double x[8] = {xn[q], xs[q], xn[q + 1], xn[q - 1], xs[q + 1], xs[q - 1], xc[q + 1], xc[q - 1]};
+        double s = FULL ? 0.0 : k.w[8][u] * xc[q];
+#pragma unroll
+        for (int a = 0; a < 8; ++a) s = fma(k.w[a][u], FULL ? x[a] - xc[q] : x[a], s);
+        y[u] = FULL ? fma(k.w[8][u], xc[q], s) : s;
+    }
+}
+
+// what a pass loads of the stencil
+template <class Pol>
+using Stencil4 = std::conditional_t<Pol::kMixed, Coef4<typename Pol::coef>, Wgt4>;
+
 // ---------------------------------------------------------------------------
 // staging of a row's zonal factors into shared memory
 // ---------------------------------------------------------------------------
@@ -631,6 +667,7 @@ __device__ void wphase_true(const MemberDev<Pol> &M, const RowView<Pol> &v, type
     const size_t row = (size_t)j * nx, rs = j > 0 ? row - nx : row;
     const bool staged = f.lf && M.pc >= 3;
     if (staged) wfac_issue(f, j, M.lfT + row, M.invDT + row, nx);
+    // mixed policies: the FP64 faces
     const RowCoef<double> c = {M.ax + row, M.cx + row, M.bx + row, M.ay + row, M.cy + row, M.by + row,
                                M.ay + rs, M.cy + rs, M.by + rs, M.C + row};
     int srcS, shS, srcN, shN;
@@ -646,12 +683,14 @@ __device__ void wphase_true(const MemberDev<Pol> &M, const RowView<Pol> &v, type
         cg6(pN, a, nx, xn);
         a = i0 + shS; if (a >= nx) a -= nx;
         cg6(pS, a, nx, xs);
-        Coef4<double> k;
-        coef4(c, i0, nx, true, has_n, has_s, k);
+        std::conditional_t<Pol::kMixed, Coef4<double>, Wgt4> k;
+        if constexpr (Pol::kMixed) coef4(c, i0, nx, true, has_n, has_s, k);
+        else weights4<true>(v, i0, k);
         double Rv[4];
         ldg4(M.R + row + i0, Rv);
         double lphi[4];
-        apply4(k, xc, xn, xs, has_n, has_s, lphi);
+        if constexpr (Pol::kMixed) apply4(k, xc, xn, xs, has_n, has_s, lphi);
+        else apply9<true>(k, xc, xn, xs, lphi);
         const int p0 = tpos4(w, i0);
         typename Pol::res r4[4];
 #pragma unroll
@@ -772,7 +811,7 @@ __device__ void wphase_ub(const MemberDev<Pol> &M, const MemberCtl &c, const Row
 template <class Pol>
 struct StQuad {
     typename Pol::comp xc[6], xn[6], xs[6], rv[4], dg[4];
-    Coef4<typename Pol::coef> k;
+    Stencil4<Pol> k;
 };
 
 // Richardson stage mu >= 1 (precond_stage): reads q_mu on rows j - 1 .. j + 1,
@@ -811,7 +850,9 @@ __device__ void wprecond_stage(const MemberDev<Pol> &M, const RowView<Pol> &v, t
                 q6(qN, i0, nx, d.xn);
                 q6(qS, i0, nx, d.xs);
             }
-            coef4(c, i0, nx, !o3, hn, hs, d.k);
+            if constexpr (Pol::kMixed) coef4(c, i0, nx, !o3, hn, hs, d.k);
+            else if (o3) weights4<false>(v, i0, d.k);
+            else weights4<true>(v, i0, d.k);
             ldv4(v.r + i0, d.rv);
 #pragma unroll
             for (int u = 0; u < 4; ++u) d.dg[u] = comp(1);
@@ -824,7 +865,9 @@ __device__ void wprecond_stage(const MemberDev<Pol> &M, const RowView<Pol> &v, t
         };
         auto compute = [&](int i0, StQuad<Pol> &d) {
             comp y[4];
-            apply4(d.k, d.xc, d.xn, d.xs, hn, hs, y);
+            if constexpr (Pol::kMixed) apply4(d.k, d.xc, d.xn, d.xs, hn, hs, y);
+            else if (o3) apply9<false>(d.k, d.xc, d.xn, d.xs, y);
+            else apply9<true>(d.k, d.xc, d.xn, d.xs, y);
             const int p0 = tpos4(w, i0);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -854,7 +897,7 @@ __device__ void wprecond_stage(const MemberDev<Pol> &M, const RowView<Pol> &v, t
 template <class Pol, int KM>
 struct LeQuad {
     typename Pol::comp xc[6], xn[6], xs[6];
-    Coef4<typename Pol::coef> k;
+    Stencil4<Pol> k;
     typename Pol::res r4[4];
     typename Pol::vec lp4[KM][4];
 };
@@ -934,7 +977,8 @@ __device__ void wphase_le(const MemberDev<Pol> &M, const MemberCtl &c, const Row
                 q6(qN, i0, nx, d.xn);
                 q6(qS, i0, nx, d.xs);
             }
-            coef4(cf, i0, nx, true, hn, hs, d.k);
+            if constexpr (Pol::kMixed) coef4(cf, i0, nx, true, hn, hs, d.k);
+            else weights4<true>(v, i0, d.k);
             ldv4(v.r + i0, d.r4);
 #pragma unroll
             for (int l = 0; l < KM; ++l)
@@ -942,7 +986,8 @@ __device__ void wphase_le(const MemberDev<Pol> &M, const MemberCtl &c, const Row
         };
         auto compute = [&](int i0, LeQuad<Pol, KM> &d) {
             comp y[4];
-            apply4(d.k, d.xc, d.xn, d.xs, hn, hs, y);
+            if constexpr (Pol::kMixed) apply4(d.k, d.xc, d.xn, d.xs, hn, hs, y);
+            else apply9<true>(d.k, d.xc, d.xn, d.xs, y);
             vec le4[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) le4[u] = (vec)y[u];
