@@ -109,41 +109,50 @@ __device__ __forceinline__ int phase_slots(int phase, int nd, int *slot)
 // phases on one row j (one block).  Each thread adds its share of the phase's
 // inner products to part[slot]; the caller sums them over the block.
 // ---------------------------------------------------------------------------
+// (FP64 policy: L(Phi) from the nine-point weights)
 template <class Pol, int NP>
-__device__ void phase_true(const MemberDev<Pol> &M, const RowView<Pol> &v, typename Pol::comp eta, int j,
-                           unsigned char *ws, typename Acc<Pol>::type (&part)[NP])
+__device__ void phase_true_f64(const MemberDev<Pol> &M, const RowView<Pol> &v, typename Pol::comp eta, int j,
+                               unsigned char *ws, typename Acc<Pol>::type (&part)[NP])
 {
+    static_assert(!Pol::kMixed, "");
+    const int nx = M.nx, ny = M.ny;
+    const size_t row = (size_t)j * nx;
+    double *sb = (double *)(ws + sb_offset<Pol>(nx));
+    double *ph = (double *)ws;
+    stage3_f64(ph, M.phi, nx, ny, j);
+    constexpr int UW = 2;
+    for (int i0 = threadIdx.x; i0 < nx; i0 += UW * blockDim.x) {
+        double Wt[UW][9], Rv[UW];
+#pragma unroll
+        for (int u = 0; u < UW; ++u) {
+            const int i = min(i0 + u * (int)blockDim.x, nx - 1);
+            load_weights<true>(v, i, Wt[u]);
+            Rv[u] = __ldg(M.R + row + i);
+        }
+#pragma unroll
+        for (int u = 0; u < UW; ++u) {
+            const int i = i0 + u * blockDim.x;
+            if (i >= nx) break;
+            const double rv = stencil9<true>(ph, ph + nx, ph + 2 * nx, i, nx, Wt[u]) - Rv[u];
+            v.r[i] = rv;
+            part[0] += rv * rv;
+            part[1] += Rv[u] * Rv[u];
+            sb[pidx(i)] = stage0_input(M, v, eta, rv, i);
+        }
+    }
+    stage0_finish(M, v, j, ws);
+}
+
+// (mixed policies: from the FP64 faces)
+template <class Pol, int NP>
+__device__ void phase_true_mixed(const MemberDev<Pol> &M, const RowView<Pol> &v, typename Pol::comp eta, int j,
+                                 unsigned char *ws, typename Acc<Pol>::type (&part)[NP])
+{
+    static_assert(Pol::kMixed, "");
     typedef typename Pol::comp comp;
     const int nx = M.nx, ny = M.ny;
     const size_t row = (size_t)j * nx;
     comp *sb = (comp *)(ws + sb_offset<Pol>(nx));
-    if constexpr (!Pol::kMixed) {
-        // FP64 policy: the nine-point weights
-        double *ph = (double *)ws;
-        stage3_f64(ph, M.phi, nx, ny, j);
-        constexpr int UW = 2;
-        for (int i0 = threadIdx.x; i0 < nx; i0 += UW * blockDim.x) {
-            double Wt[UW][9], Rv[UW];
-#pragma unroll
-            for (int u = 0; u < UW; ++u) {
-                const int i = min(i0 + u * (int)blockDim.x, nx - 1);
-                load_weights<true>(v, i, Wt[u]);
-                Rv[u] = __ldg(M.R + row + i);
-            }
-#pragma unroll
-            for (int u = 0; u < UW; ++u) {
-                const int i = i0 + u * blockDim.x;
-                if (i >= nx) break;
-                const double rv = stencil9<true>(ph, ph + nx, ph + 2 * nx, i, nx, Wt[u]) - Rv[u];
-                v.r[i] = rv;
-                part[0] += rv * rv;
-                part[1] += Rv[u] * Rv[u];
-                sb[pidx(i)] = stage0_input(M, v, eta, rv, i);
-            }
-        }
-        stage0_finish(M, v, j, ws);
-        return;
-    }
     const size_t rs = j > 0 ? row - nx : row;
     const RowCoef<double> c = {M.ax + row, M.cx + row, M.bx + row, M.ay + row, M.cy + row, M.by + row,
                                M.ay + rs, M.cy + rs, M.by + rs, M.C + row};
@@ -245,10 +254,56 @@ __device__ void phase_true(const MemberDev<Pol> &M, const RowView<Pol> &v, typen
     stage0_finish(M, v, j, ws);
 }
 
+// (FP64 policy: L e from the nine-point weights, its products in the same loop)
 template <class Pol, int KM>
-__device__ void phase_le(const MemberDev<Pol> &M, const MemberCtl &c, const RowView<Pol> &v, int j,
-                         unsigned char *ws, typename Acc<Pol>::type (&part)[2 + 2 * KM])
+__device__ void phase_le_f64(const MemberDev<Pol> &M, const MemberCtl &c, const RowView<Pol> &v, int j,
+                             unsigned char *ws, typename Acc<Pol>::type (&part)[2 + 2 * KM])
 {
+    static_assert(!Pol::kMixed, "");
+    const int nx = M.nx;
+    const int nd = c.nu + 1;
+    stage3_q(ws, M, M.e, M.e32, M.e_s, j);
+    SW_TRACE(101);
+    const double *stg = (const double *)ws;
+    constexpr int UW = 2;
+    const double *Lpl[KM];
+#pragma unroll
+    for (int l = 0; l < KM; ++l) Lpl[l] = v.Lpb + (size_t)phys_slot(c, M.k, l < nd ? l : 0) * v.vstride;
+    for (int i0 = threadIdx.x; i0 < nx; i0 += UW * blockDim.x) {
+        double Wt[UW][9], rv[UW], lp[UW][KM];
+#pragma unroll
+        for (int u = 0; u < UW; ++u) {
+            const int i = min(i0 + u * (int)blockDim.x, nx - 1);
+            load_weights<true>(v, i, Wt[u]);
+            rv[u] = v.r[i];
+#pragma unroll
+            for (int l = 0; l < KM; ++l) lp[u][l] = l < nd ? Lpl[l][i] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < UW; ++u) {
+            const int i = i0 + u * blockDim.x;
+            if (i >= nx) break;
+            const double la = stencil9<true>(stg, stg + nx, stg + 2 * nx, i, nx, Wt[u]);
+            v.Le[i] = la;
+            part[0] += la * la;
+            part[1] += rv[u] * la;
+#pragma unroll
+            for (int l = 0; l < KM; ++l) {
+                if (l < nd) {
+                    part[2 + l] += la * lp[u][l];
+                    part[2 + KM + l] += rv[u] * lp[u][l];
+                }
+            }
+        }
+    }
+    __syncthreads();           // the block's next row is staged over these
+}
+
+template <class Pol, int KM>
+__device__ void phase_le_mixed(const MemberDev<Pol> &M, const MemberCtl &c, const RowView<Pol> &v, int j,
+                               unsigned char *ws, typename Acc<Pol>::type (&part)[2 + 2 * KM])
+{
+    static_assert(Pol::kMixed, "");
     typedef typename Pol::comp comp;
     typedef typename Pol::vec vec;
     typedef typename Acc<Pol>::type acc_t;
@@ -257,42 +312,6 @@ __device__ void phase_le(const MemberDev<Pol> &M, const MemberCtl &c, const RowV
     stage3_q(ws, M, M.e, M.e32, M.e_s, j);
     SW_TRACE(101);
     const comp *stg = (const comp *)ws;
-    if constexpr (!Pol::kMixed) {
-        // FP64: L e from the nine-point weights, its products in the same loop
-        constexpr int UW = 2;
-        const double *Lpl[KM];
-#pragma unroll
-        for (int l = 0; l < KM; ++l) Lpl[l] = v.Lpb + (size_t)phys_slot(c, M.k, l < nd ? l : 0) * v.vstride;
-        for (int i0 = threadIdx.x; i0 < nx; i0 += UW * blockDim.x) {
-            double Wt[UW][9], rv[UW], lp[UW][KM];
-#pragma unroll
-            for (int u = 0; u < UW; ++u) {
-                const int i = min(i0 + u * (int)blockDim.x, nx - 1);
-                load_weights<true>(v, i, Wt[u]);
-                rv[u] = v.r[i];
-#pragma unroll
-                for (int l = 0; l < KM; ++l) lp[u][l] = l < nd ? Lpl[l][i] : 0.0;
-            }
-#pragma unroll
-            for (int u = 0; u < UW; ++u) {
-                const int i = i0 + u * blockDim.x;
-                if (i >= nx) break;
-                const double la = stencil9<true>(stg, stg + nx, stg + 2 * nx, i, nx, Wt[u]);
-                v.Le[i] = la;
-                part[0] += la * la;
-                part[1] += rv[u] * la;
-#pragma unroll
-                for (int l = 0; l < KM; ++l) {
-                    if (l < nd) {
-                        part[2 + l] += la * lp[u][l];
-                        part[2 + KM + l] += rv[u] * lp[u][l];
-                    }
-                }
-            }
-        }
-        __syncthreads();           // the block's next row is staged over these
-        return;
-    }
     // L e of the row, straight into the row's L e storage
     if (stencil4_ok(coef_of(v), nx) && ((uintptr_t)v.Le & 15) == 0)
         stencil_row4<comp, typename Pol::coef>(stg, stg + nx, stg + 2 * nx, nx, j, ny, coef_of(v), true, (comp *)v.Le,
@@ -304,8 +323,8 @@ __device__ void phase_le(const MemberDev<Pol> &M, const MemberCtl &c, const RowV
     const vec *Lpl[KM];
 #pragma unroll
     for (int l = 0; l < KM; ++l) Lpl[l] = v.Lpb + (size_t)phys_slot(c, M.k, l < nd ? l : 0) * v.vstride;
-    // mixed policies: 4 consecutive points per thread, vector reads
-    bool v4 = Pol::kMixed && (nx & 3) == 0 && al16p(v.Le) && al16p(v.r);
+    // 4 consecutive points per thread, vector reads
+    bool v4 = (nx & 3) == 0 && al16p(v.Le) && al16p(v.r);
 #pragma unroll
     for (int l = 0; l < KM; ++l) v4 = v4 && al16p(Lpl[l]);
     if (v4) {
@@ -840,12 +859,16 @@ __global__ void __launch_bounds__(MAX_THREADS, MINB) k_gcr(const EnsDesc *__rest
                             break;
                         }
                     }
-                    phase_true<Pol, NP>(M, v, eta, j, ws, part);
+                    if constexpr (Pol::kMixed) phase_true_mixed<Pol, NP>(M, v, eta, j, ws, part);
+                    else phase_true_f64<Pol, NP>(M, v, eta, j, ws, part);
                     break;
                 case PH_UB: phase_ub<Pol, KM>(M, s_c, v, eta, j, ws, part); break;
                 case PH_PREC: precond_stage<Pol>(M, v, eta, s_c.stage, j, ws); break;
                 case PH_PREC0: phase_prec0<Pol>(M, v, eta, j, ws); break;
-                case PH_LE: phase_le<Pol, KM>(M, s_c, v, j, ws, part); break;
+                case PH_LE:
+                    if constexpr (Pol::kMixed) phase_le_mixed<Pol, KM>(M, s_c, v, j, ws, part);
+                    else phase_le_f64<Pol, KM>(M, s_c, v, j, ws, part);
+                    break;
                 case PH_ZERO:
                     for (int i = threadIdx.x; i < nx; i += blockDim.x) M.phi[(size_t)j * nx + i] = 0.0;
                     break;

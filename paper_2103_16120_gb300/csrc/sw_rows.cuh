@@ -96,9 +96,11 @@ struct RowCoef {
     const CT *ax, *cx, *bx, *ay, *cy, *by, *ays, *cys, *bys, *C;
 };
 
+// (mixed policies: the FP64 policy's view has the weights instead)
 template <class Pol>
 __device__ __forceinline__ RowCoef<typename Pol::coef> coef_of(const RowView<Pol> &v)
 {
+    static_assert(Pol::kMixed, "FP64 takes the stencils from the weights");
     return {v.ax, v.cx, v.bx, v.ay, v.cy, v.by, v.ays, v.cys, v.bys, v.C};
 }
 
@@ -107,11 +109,17 @@ template <class Pol>
 __device__ __forceinline__ void view_const_global(const MemberDev<Pol> &M, int j, RowView<Pol> &v)
 {
     const size_t row = (size_t)j * M.nx, rs = j > 0 ? row - M.nx : row;
-    v.ax = M.wax + row; v.cx = M.wcx + row; v.bx = M.wbx + row;
-    v.ay = M.way + row; v.cy = M.wcy + row; v.by = M.wby + row;
-    v.ays = M.way + rs; v.cys = M.wcy + rs; v.bys = M.wby + rs;
-    v.C = M.wC + row; v.diag = M.wdiag + row;
-    if constexpr (!Pol::kMixed) { v.w = M.wgt + row; v.wstride = (size_t)M.nx * M.ny; }
+    if constexpr (Pol::kMixed) {
+        v.ax = M.wax + row; v.cx = M.wcx + row; v.bx = M.wbx + row;
+        v.ay = M.way + row; v.cy = M.wcy + row; v.by = M.wby + row;
+        v.ays = M.way + rs; v.cys = M.wcy + rs; v.bys = M.wby + rs;
+        v.C = M.wC + row;
+        v.w = nullptr; v.wstride = 0;
+    } else {
+        v.ax = v.cx = v.bx = v.ay = v.cy = v.by = v.ays = v.cys = v.bys = v.C = nullptr;
+        v.w = M.wgt + row; v.wstride = (size_t)M.nx * M.ny;
+    }
+    v.diag = M.wdiag + row;
     v.lf = M.lf + row; v.invD = M.invD + row; v.zz = M.zz + row;
     v.fpad = false;
     v.gam = M.gam[j]; v.ec = M.ec[j];
@@ -134,7 +142,9 @@ __device__ void view_const_cache(const MemberDev<Pol> &M, int j, unsigned char *
             for (int i = threadIdx.x; i < nx; i += blockDim.x) c[a * nx + i] = src[a][i];
         v.ax = c; v.cx = c + nx; v.bx = c + 2 * nx; v.ay = c + 3 * nx; v.cy = c + 4 * nx; v.by = c + 5 * nx;
         v.ays = c + 6 * nx; v.cys = c + 7 * nx; v.bys = c + 8 * nx; v.C = c + 9 * nx; v.diag = c + 10 * nx;
+        v.w = nullptr; v.wstride = 0;
     } else {
+        v.ax = v.cx = v.bx = v.ay = v.cy = v.by = v.ays = v.cys = v.bys = v.C = nullptr;
         for (int a = 0; a <= NWGT; ++a) {
             const CT *src = a < NWGT ? g.w + a * g.wstride : g.diag;
             for (int i = threadIdx.x; i < nx; i += blockDim.x) c[a * nx + i] = src[i];
@@ -430,37 +440,37 @@ __device__ __noinline__ void stage3_q(unsigned char *ws, const MemberDev<Pol> &M
     typedef typename Pol::q16 qt;
     const int nx = M.nx, ny = M.ny;
     comp *stg = (comp *)ws;
-    int src[3], sh[3];
     if constexpr (!Pol::kMixed) {
         stage3_f64(stg, h, nx, ny, j);
-        return;
-    }
-    unsigned char *raw = ws + raw_offset<Pol>(nx);
-    const size_t rs = (size_t)nx * 4;   // raw row stride
-    bool band[3];
+    } else {
+        int src[3], sh[3];
+        unsigned char *raw = ws + raw_offset<Pol>(nx);
+        const size_t rs = (size_t)nx * 4;   // raw row stride
+        bool band[3];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        ghost_row(j - 1 + r, nx, ny, src[r], sh[r]);
-        band[r] = in_band(M, src[r]);
-        const size_t off = (size_t)src[r] * nx;
-        if (band[r]) row_copy_issue(raw + r * rs, f32 + off, nx * 4);
-        else row_copy_issue(raw + r * rs, h + off, nx * (int)sizeof(qt));
-    }
-    float s[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) s[r] = q_scale(M, sc, src[r]);
-    row_copy_wait();
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const qt *rq = (const qt *)(raw + r * rs);
-        const float *rf = (const float *)(raw + r * rs);
-        for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-            int ii = i + sh[r];
-            if (ii >= nx) ii -= nx;
-            stg[r * nx + i] = band[r] ? rf[ii] : q_to_f(rq[ii]) * s[r];
+        for (int r = 0; r < 3; ++r) {
+            ghost_row(j - 1 + r, nx, ny, src[r], sh[r]);
+            band[r] = in_band(M, src[r]);
+            const size_t off = (size_t)src[r] * nx;
+            if (band[r]) row_copy_issue(raw + r * rs, f32 + off, nx * 4);
+            else row_copy_issue(raw + r * rs, h + off, nx * (int)sizeof(qt));
         }
+        float s[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) s[r] = q_scale(M, sc, src[r]);
+        row_copy_wait();
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const qt *rq = (const qt *)(raw + r * rs);
+            const float *rf = (const float *)(raw + r * rs);
+            for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+                int ii = i + sh[r];
+                if (ii >= nx) ii -= nx;
+                stg[r * nx + i] = band[r] ? rf[ii] : q_to_f(rq[ii]) * s[r];
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
 }
 
 // store row j of a preconditioner field from the padded buffer sb (16-bit
@@ -596,32 +606,27 @@ __device__ void precond_stage(const MemberDev<Pol> &M, const RowView<Pol> &v, ty
                 else sb[pidx(i)] = X[i] + M.omega * (rv[u] - stencil9<true>(S, X, N, i, nx, Wt[u])) / dg[u];
             }
         }
-        __syncthreads();
-        SW_TRACE(302);
-        if (opt3) trisolve_view(sb, nx, v, sm);
-        SW_TRACE(303);
-        q_store_row(M, oh, of32, os, j, sb, last ? v.el : (comp *)nullptr, (float *)sm);
-        return;
-    }
-    if (stencil4_ok(coef_of(v), nx))
-        stencil_row4<comp, typename Pol::coef>(S, X, N, nx, j, ny, coef_of(v), !opt3, sb, true);
-    else
-        stencil_row<comp, typename Pol::coef>(S, X, N, nx, j, ny, coef_of(v), !opt3, sb, true);
-    constexpr int U = batch_of<comp>();
-    for (int i0 = threadIdx.x; i0 < nx; i0 += U * blockDim.x) {
-        comp rv[U], dg[U];
+    } else {
+        if (stencil4_ok(coef_of(v), nx))
+            stencil_row4<comp, typename Pol::coef>(S, X, N, nx, j, ny, coef_of(v), !opt3, sb, true);
+        else
+            stencil_row<comp, typename Pol::coef>(S, X, N, nx, j, ny, coef_of(v), !opt3, sb, true);
+        constexpr int U = batch_of<comp>();
+        for (int i0 = threadIdx.x; i0 < nx; i0 += U * blockDim.x) {
+            comp rv[U], dg[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = min(i0 + u * (int)blockDim.x, nx - 1);
-            rv[u] = (comp)v.r[i];
-            dg[u] = opt3 ? comp(1) : (comp)v.diag[i];
-        }
+            for (int u = 0; u < U; ++u) {
+                const int i = min(i0 + u * (int)blockDim.x, nx - 1);
+                rv[u] = (comp)v.r[i];
+                dg[u] = opt3 ? comp(1) : (comp)v.diag[i];
+            }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * blockDim.x;
-            if (i >= nx) break;
-            const comp s = sb[pidx(i)], xv = X[i];
-            sb[pidx(i)] = opt3 ? xv + eta * (s - rv[u]) : xv + (comp)M.omega * (rv[u] - s) / dg[u];
+            for (int u = 0; u < U; ++u) {
+                const int i = i0 + u * blockDim.x;
+                if (i >= nx) break;
+                const comp s = sb[pidx(i)], xv = X[i];
+                sb[pidx(i)] = opt3 ? xv + eta * (s - rv[u]) : xv + (comp)M.omega * (rv[u] - s) / dg[u];
+            }
         }
     }
     __syncthreads();

@@ -116,7 +116,7 @@ __device__ __forceinline__ void split_quad(const SplitOp &M, const SplitState &S
 // the split initial residual of row j for the solver's first phase, by the
 // threads (tid, T) of a block or a warp: r (policy type) into the row's r,
 // ||r||^2 and ||R||^2 into part, the first preconditioner stage's input to
-// put(i, value) (phase_true with the operator of Eq. 14)
+// put(i, value) (phase_true_mixed with the operator of Eq. 14)
 template <class Pol, int NP, class PUT>
 __device__ __forceinline__ void split_true_row(const MemberDev<Pol> &M, const SplitState &S, const RowView<Pol> &v,
                                                typename Pol::comp eta, int j, int tid, int T,

@@ -655,7 +655,7 @@ __device__ __forceinline__ void quads(int nx, LD load, CP compute)
 
 // ---------------------------------------------------------------------------
 // phases on one row j (one warp); the thread adds its share of the phase's
-// inner products to part (phase_true, phase_ub, precond_stage, phase_le)
+// inner products to part (the block path's phase_true_*, phase_ub, precond_stage, phase_le_*)
 // ---------------------------------------------------------------------------
 template <class Pol, int NP, int SEL>
 __device__ void wphase_true(const MemberDev<Pol> &M, const RowView<Pol> &v, typename Pol::comp eta, int j,
@@ -835,11 +835,13 @@ __device__ void wprecond_stage(const MemberDev<Pol> &M, const RowView<Pol> &v, t
     float *of32 = last ? M.e32 : ((mu & 1) ? M.qb32 : M.qa32);
     float *os = last ? M.e_s : ((mu & 1) ? M.qb_s : M.qa_s);
     const QRow<Pol> qS = qrow(M, ih, if32, is, j - 1), qX = qrow(M, ih, if32, is, j), qN = qrow(M, ih, if32, is, j + 1);
-    const RowCoef<CT> c = coef_of(v);
+    RowCoef<CT> c = {};
+    if constexpr (Pol::kMixed) c = coef_of(v);
     // PL: option 3 on a plain row (rows_plain), conditions fixed at compile time
     auto pass = [&](auto plain_t) {
         constexpr bool PL = decltype(plain_t)::value;
-        const bool o3 = PL || opt3, hn = PL || has_n, hs = PL || has_s;
+        const bool o3 = PL || opt3;
+        [[maybe_unused]] const bool hn = PL || has_n, hs = PL || has_s;      // the weights need neither
         auto load = [&](int i0, StQuad<Pol> &d) {
             if constexpr (PL) {
                 q6i(qX, i0, nx, d.xc);
@@ -937,7 +939,7 @@ __host__ __device__ __forceinline__ const V *direction_row(int l, int nd, const 
 }
 
 // L(e) of row j into the row's L e and the inner products <Le,Le>, <r,Le>,
-// <Le,Lp_l>, <r,Lp_l> (phase_le)
+// <Le,Lp_l>, <r,Lp_l> (phase_le_mixed, phase_le_f64)
 template <class Pol, int KM, int SEL>
 __device__ void wphase_le(const MemberDev<Pol> &M, const MemberCtl &c, const RowView<Pol> &v, int j, const WRow w,
                           typename Acc<Pol>::type (&part)[2 + 2 * KM])
@@ -951,7 +953,8 @@ __device__ void wphase_le(const MemberDev<Pol> &M, const MemberCtl &c, const Row
     const QRow<Pol> qS = qrow(M, M.e, M.e32, M.e_s, j - 1), qX = qrow(M, M.e, M.e32, M.e_s, j),
                     qN = qrow(M, M.e, M.e32, M.e_s, j + 1);
     const bool has_n = j < ny - 1, has_s = j > 0;
-    const RowCoef<CT> cf = coef_of(v);
+    RowCoef<CT> cf = {};
+    if constexpr (Pol::kMixed) cf = coef_of(v);
     constexpr bool ONE = SEL > 0 && KM == 4;      // one compiled loop per number of directions only
     const vec *Lpl[KM];
 #pragma unroll
@@ -966,7 +969,7 @@ __device__ void wphase_le(const MemberDev<Pol> &M, const MemberCtl &c, const Row
     auto pass = [&](auto plain_t, auto nd_t) {
         constexpr int ND = decltype(nd_t)::value;
         constexpr bool PL = decltype(plain_t)::value;
-        const bool hn = PL || has_n, hs = PL || has_s;
+        [[maybe_unused]] const bool hn = PL || has_n, hs = PL || has_s;
         auto load = [&](int i0, LeQuad<Pol, KM> &d) {
             if constexpr (PL) {
                 q6i(qX, i0, nx, d.xc);
