@@ -27,6 +27,9 @@
  *    synchronise it;
  *  - errors are reported by the returned status only, never by exceptions or
  *    aborts; sw_last_error() gives a message for the calling thread;
+ *  - a call that does not synchronise returns before its work has run: its
+ *    operands and the grid (its workspace among them) are in use until then.
+ *    Calls on one grid from two streams are ordered by the caller (an event);
  *  - a grid handle must not be used by two host threads at once.
  */
 #ifndef SW_ELLIPTIC_H
@@ -226,7 +229,9 @@ sw_status sw_split_residual(sw_grid g, const double *phi, const double *R, float
 /* q = P^{-1}(r), the preconditioner o->pc with o->n_richardson iterations
  * (Sec. 2.3, Eq. 13).  FP64 when o->prec is SW_PREC_FP64 (r, q double),
  * otherwise r and q are float and the sweeps use o->prec's 16-bit storage.
- * r and q must not overlap. */
+ * r and q must not overlap.  Nothing synchronises, and once the workspace
+ * exists (as for sw_ensemble_solve_async) the call can be recorded in a CUDA
+ * graph and replayed. */
 sw_status sw_precond_apply(sw_grid g, const sw_solve_opts *o, const void *r, void *q,
                            void *stream);
 
