@@ -472,7 +472,7 @@ extern "C" sw_status sw_operator_apply(sw_grid g, int prec, const void *x, void 
     if (xb < yb + g->N * eb && yb < xb + g->N * eb) return fail(SW_ERR_INVALID_ARG, "sw_operator_apply: x and y overlap");
     if (prec == SW_PREC_FP64) {
         OpArgs<double> a{g->nx, g->ny, g->ax, g->cx, g->bx, g->ay, g->cy, g->by, g->C};
-        CK(launch_operator_f64(a, (const double *)x, (double *)y, row_threads(g->nx), s));
+        CK(launch_operator_f64(a, (const double *)x, (double *)y, row_threads(g->nx), g->sms, s));
     } else if (prec == SW_PREC_FP32) {
         OpArgs<float> a{g->nx, g->ny, g->wax, g->wcx, g->wbx, g->way, g->wcy, g->wby, g->wC};
         CK(launch_operator_f32(a, (const float *)x, (float *)y, row_threads(g->nx), s));

@@ -117,7 +117,8 @@ cudaError_t gcr_debug_s16(unsigned long long extra, unsigned long long limit_ns)
 cudaError_t gcr_debug_sbf16(unsigned long long extra, unsigned long long limit_ns);
 void gcr_trace_s16(unsigned long long *buf, int cap, int block);
 void gcr_trace_sbf16(unsigned long long *buf, int cap, int block);
-cudaError_t launch_operator_f64(const OpArgs<double> &a, const double *x, double *y, int threads, cudaStream_t s);
+cudaError_t launch_operator_f64(const OpArgs<double> &a, const double *x, double *y, int threads, int sms,
+                                cudaStream_t s);
 cudaError_t launch_operator_f32(const OpArgs<float> &a, const float *x, float *y, int threads, cudaStream_t s);
 // M: host copy of the member descriptor
 cudaError_t launch_precond(int prec, const void *M, int nx, int ny, int nstages, void *qout, int threads,

@@ -405,12 +405,13 @@ static bool op4_ok(const OpArgs<T> &a, const T *x, const T *y)
            al(a.cy) && al(a.by) && al(a.C);
 }
 
-cudaError_t launch_operator_f64(const OpArgs<double> &a, const double *x, double *y, int threads, cudaStream_t s)
+cudaError_t launch_operator_f64(const OpArgs<double> &a, const double *x, double *y, int threads, int sms,
+                                cudaStream_t s)
 {
     if (op4_ok(a, x, y)) {
         // four rows a thread while that leaves three blocks for every SM
         const unsigned bx = (a.nx / 4 + 127) / 128;
-        const long want = 3 * 152;
+        const long want = 3L * sms;
         if ((long)bx * ((a.ny + 3) / 4) >= want) k_operator_rows<4><<<dim3(bx, (a.ny + 3) / 4), 128, 0, s>>>(a, x, y);
         else if ((long)bx * ((a.ny + 1) / 2) >= want) k_operator_rows<2><<<dim3(bx, (a.ny + 1) / 2), 128, 0, s>>>(a, x, y);
         else k_operator_rows<1><<<dim3(bx, a.ny), 128, 0, s>>>(a, x, y);
