@@ -1,7 +1,7 @@
-// nn_conv.cu -- 3x3 convolutions of the learned preconditioner, for the rows that
-// nn_tc.cu does not take (16 or 32 points), on the tensor
-// cores (BF16 operands, FP32 accumulation, mma.sync m16n8k16), as implicit
-// GEMMs over NHWC activations [B][H][W][C]:
+// nn_conv.cu -- 3x3 convolutions of the learned preconditioner's coarser levels
+// where their rows are 16 or 32 points (nx = 64 or 128), which nn_tc.cu does not
+// take, on the tensor cores (BF16 operands, FP32 accumulation, mma.sync
+// m16n8k16), as implicit GEMMs over NHWC activations [B][H][W][C]:
 //
 //   k_conv   y[p][o] = b[o] + sum_{tap, c} w[tap][o][c] xt[p + tap][c]
 //            (forward: xt is x with the sphere halo -- periodic longitude,
@@ -11,11 +11,10 @@
 //   k_wgrad  dw[tap][o][c] += sum_p g[p][o] xt[p + tap][c]   (split over pixels)
 //
 // The tap order is ky * 3 + kx with (ky, kx) = (1, 1) the centre; the weight
-// rows are [tap][o][c] with c contiguous.  A block works on tiles of TW = 64
-// (or W, when W < 64) consecutive points of one latitude row: it stages the
-// tile's three input rows with their halo in shared memory once (cp.async)
-// and feeds the nine taps to the tensor cores with ldmatrix row addresses
-// shifted by the tap -- no im2col buffer.
+// rows are [tap][o][c] with c contiguous.  A block works on one latitude row at
+// a time: it stages the three input rows with their halo in shared memory once
+// (cp.async) and feeds the nine taps to the tensor cores with ldmatrix row
+// addresses shifted by the tap -- no im2col buffer.
 #include <cuda_bf16.h>
 #include <cstdint>
 
@@ -51,6 +50,8 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+constexpr int MAX_W = 32;                    // points of the longest row
+
 // shared-memory row pitch (elements) of a C-channel pixel: 8 extra elements
 // (16 bytes) put the eight rows an ldmatrix reads on distinct bank groups
 __host__ __device__ constexpr int pitch(int c) { return c + 8; }
@@ -66,10 +67,9 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
     constexpr int PI = pitch(CIN);
     extern __shared__ __align__(16) unsigned char smem[];
     __nv_bfloat16 *Ws = (__nv_bfloat16 *)smem;                       // [9][COUT][PI]
-    __nv_bfloat16 *Xs = Ws + 9 * COUT * PI;                          // [4][TW + 2][PI]
-    const int H = a.H, W = a.W, TW = W < 64 ? W : 64;
-    const int nseg = W / TW;
-    const long ntiles = (long)a.B * H * nseg;
+    __nv_bfloat16 *Xs = Ws + 9 * COUT * PI;                          // [4][W + 2][PI]
+    const int H = a.H, W = a.W;
+    const long nrow = (long)a.B * H;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     // weights, once per block
@@ -78,20 +78,17 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
         cp16(Ws + row * PI + ch * 8, a.w + (size_t)row * CIN + ch * 8);
     }
 
-    for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int seg = (int)(tile % nseg);
-        const long bh = tile / nseg;
+    for (long bh = blockIdx.x; bh < nrow; bh += gridDim.x) {
         const int h = (int)(bh % H), b = (int)(bh / H);
-        const int w0 = seg * TW;
         const bool pole = DGRAD && (h == 0 || h == H - 1);
         const int nrows = pole ? 4 : 3;
-        __syncthreads();                         // previous tile's reads are done
+        __syncthreads();                         // previous row's reads are done
         // stage rows h-1, h, h+1 (and, for DGRAD on a pole row, the pole row
         // shifted by half a circle) with one point of halo on each side
-        for (int q = threadIdx.x; q < nrows * (TW + 2) * (CIN / 8); q += blockDim.x) {
+        for (int q = threadIdx.x; q < nrows * (W + 2) * (CIN / 8); q += blockDim.x) {
             const int ch = q % (CIN / 8);
-            const int cpt = (q / (CIN / 8)) % (TW + 2);
-            const int r = q / (CIN / 8) / (TW + 2);
+            const int cpt = (q / (CIN / 8)) % (W + 2);
+            const int r = q / (CIN / 8) / (W + 2);
             int hs, shift = 0;
             bool zero = false;
             if (r < 3) {
@@ -103,11 +100,11 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
             } else {
                 hs = h; shift = W / 2;
             }
-            __nv_bfloat16 *dst = Xs + (r * (TW + 2) + cpt) * PI + ch * 8;
+            __nv_bfloat16 *dst = Xs + (r * (W + 2) + cpt) * PI + ch * 8;
             if (zero) {
                 *(uint4 *)dst = make_uint4(0, 0, 0, 0);
             } else {
-                int ws = w0 - 1 + cpt + shift;
+                int ws = cpt - 1 + shift;
                 ws %= W;
                 if (ws < 0) ws += W;
                 cp16(dst, a.x + (((size_t)b * H + hs) * W + ws) * CIN + ch * 8);
@@ -117,7 +114,7 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
         __syncthreads();
 
         const int p0 = warp * 16;
-        if (p0 < TW) {
+        if (p0 < W) {
             float acc[NT][4];
 #pragma unroll
             for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
@@ -132,7 +129,7 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
                 if (t < 9) { tap = t; xr = t / 3; }
                 else { tap = (h == 0 ? 6 : 0) + (t - 9); xr = 3; }
                 const int kx = tap % 3;
-                const __nv_bfloat16 *xa = Xs + (xr * (TW + 2) + arow + kx) * PI + akof;
+                const __nv_bfloat16 *xa = Xs + (xr * (W + 2) + arow + kx) * PI + akof;
                 const __nv_bfloat16 *wb = Ws + (tap * COUT + brow) * PI + bkof;
 #pragma unroll
                 for (int ks = 0; ks < KS; ++ks) {
@@ -147,9 +144,9 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
                     }
                 }
             }
-            // epilogue: bias, ReLU or mask, store of the 16 points x COUT
+            // epilogue: bias, ReLU, store of the 16 points x COUT
             const int g = lane >> 2, tg = lane & 3;
-            const size_t pix = ((size_t)b * H + h) * W + w0 + p0;      // first point of the warp
+            const size_t pix = ((size_t)b * H + h) * W + p0;           // first point of the warp
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
                 const int co = 8 * j + 2 * tg;
@@ -158,13 +155,6 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
                 if (a.relu)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) v[q] = fmaxf(v[q], 0.f);
-                if (a.mask) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const size_t idx = (pix + g + 8 * (q >> 1)) * COUT + co + (q & 1);
-                        if (!(__bfloat162float(a.mask[idx]) > 0.f)) v[q] = 0.f;
-                    }
-                }
                 if (a.yf) {
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -182,7 +172,7 @@ __global__ void __launch_bounds__(128) k_conv(ConvArgs a)
 
 // ---------------------------------------------------------------------------
 // weight gradient: block (ky, c-block, split) accumulates the three taps of
-// kernel row ky for COUT x NCI weights over its share of the tiles
+// kernel row ky for COUT x NCI weights over its share of the rows
 // ---------------------------------------------------------------------------
 template <int CIN, int COUT, int NCI>
 __global__ void __launch_bounds__(COUT * 2) k_wgrad(WgradArgs a)
@@ -190,15 +180,14 @@ __global__ void __launch_bounds__(COUT * 2) k_wgrad(WgradArgs a)
     constexpr int NTJ = NCI / 8;                 // n-tiles (input channels)
     constexpr int PG = pitch(COUT), PX = pitch(NCI);
     extern __shared__ __align__(16) unsigned char smem[];
-    const int H = a.H, W = a.W, TW = W < 64 ? W : 64;
-    __nv_bfloat16 *Gs = (__nv_bfloat16 *)smem;                       // [TW][PG]
-    __nv_bfloat16 *Xs = Gs + 64 * PG;                                // [TW + 2][PX]
+    const int H = a.H, W = a.W;
+    __nv_bfloat16 *Gs = (__nv_bfloat16 *)smem;                       // [W][PG]
+    __nv_bfloat16 *Xs = Gs + MAX_W * PG;                             // [W + 2][PX]
     const int ky = blockIdx.x % 3;
     const int cb = (blockIdx.x / 3) % (CIN / NCI);
     const int split = blockIdx.x / 3 / (CIN / NCI);
     const int nsplit = gridDim.x / 3 / (CIN / NCI);
-    const int nseg = W / TW;
-    const long ntiles = (long)a.B * H * nseg;
+    const long nrow = (long)a.B * H;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool do_bias = a.db && ky == 0 && cb == 0;
 
@@ -209,15 +198,12 @@ __global__ void __launch_bounds__(COUT * 2) k_wgrad(WgradArgs a)
         for (int j = 0; j < NTJ; ++j) acc[kx][j][0] = acc[kx][j][1] = acc[kx][j][2] = acc[kx][j][3] = 0.f;
     float bsum = 0.f;
 
-    for (long tile = split; tile < ntiles; tile += nsplit) {
-        const int seg = (int)(tile % nseg);
-        const long bh = tile / nseg;
+    for (long bh = split; bh < nrow; bh += nsplit) {
         const int h = (int)(bh % H), b = (int)(bh / H);
-        const int w0 = seg * TW;
         __syncthreads();
-        // gradient tile [TW][COUT]
-        const __nv_bfloat16 *gsrc = a.g + (((size_t)b * H + h) * W + w0) * COUT;
-        for (int q = threadIdx.x; q < TW * (COUT / 8); q += blockDim.x) {
+        // gradient row [W][COUT]
+        const __nv_bfloat16 *gsrc = a.g + ((size_t)b * H + h) * W * COUT;
+        for (int q = threadIdx.x; q < W * (COUT / 8); q += blockDim.x) {
             const int p = q / (COUT / 8), ch = q % (COUT / 8);
             cp16(Gs + p * PG + ch * 8, gsrc + (size_t)p * COUT + ch * 8);
         }
@@ -225,19 +211,19 @@ __global__ void __launch_bounds__(COUT * 2) k_wgrad(WgradArgs a)
         int hs = h - 1 + ky, shift = 0;
         if (hs < 0) { hs = 0; shift = W / 2; }
         else if (hs >= H) { hs = H - 1; shift = W / 2; }
-        for (int q = threadIdx.x; q < (TW + 2) * (NCI / 8); q += blockDim.x) {
+        for (int q = threadIdx.x; q < (W + 2) * (NCI / 8); q += blockDim.x) {
             const int cpt = q / (NCI / 8), ch = q % (NCI / 8);
-            int ws = (w0 - 1 + cpt + shift) % W;
+            int ws = (cpt - 1 + shift) % W;
             if (ws < 0) ws += W;
             cp16(Xs + cpt * PX + ch * 8, a.x + (((size_t)b * H + hs) * W + ws) * CIN + cb * NCI + ch * 8);
         }
         cp_wait();
         __syncthreads();
         if (do_bias && threadIdx.x < COUT)
-            for (int p = 0; p < TW; ++p) bsum += __bfloat162float(Gs[p * PG + threadIdx.x]);
+            for (int p = 0; p < W; ++p) bsum += __bfloat162float(Gs[p * PG + threadIdx.x]);
         // A = g^T (16 out channels of this warp x 16 points), B = xt (16 points x 8 channels)
         const int m = lane >> 3, r8 = lane & 7;
-        for (int k0 = 0; k0 < TW; k0 += 16) {
+        for (int k0 = 0; k0 < W; k0 += 16) {
             unsigned af[4];
             ldsm_x4_t(af, Gs + (k0 + 8 * (m >> 1) + r8) * PG + warp * 16 + 8 * (m & 1));
 #pragma unroll
@@ -276,15 +262,13 @@ __global__ void __launch_bounds__(COUT * 2) k_wgrad(WgradArgs a)
 template <int CIN, int COUT, bool DGRAD>
 static cudaError_t conv_t(const ConvArgs &a, int sms, cudaStream_t s)
 {
-    const int TW = a.W < 64 ? a.W : 64;
-    const size_t smem = (size_t)(9 * COUT + (DGRAD ? 4 : 3) * (TW + 2)) * pitch(CIN) * 2;
+    const size_t smem = (size_t)(9 * COUT + (DGRAD ? 4 : 3) * (a.W + 2)) * pitch(CIN) * 2;
     int bps = 0;
     cudaError_t e = occupancy_once<k_conv<CIN, COUT, DGRAD>>(128, smem, &bps);
     if (e != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
-    const long ntiles = (long)a.B * a.H * (a.W / TW);
     long grid = (long)bps * sms;
-    if (grid > ntiles) grid = ntiles;
+    if (grid > (long)a.B * a.H) grid = (long)a.B * a.H;
     k_conv<CIN, COUT, DGRAD><<<(int)grid, 128, smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -292,15 +276,11 @@ static cudaError_t conv_t(const ConvArgs &a, int sms, cudaStream_t s)
 template <int CIN, int COUT, int NCI>
 static cudaError_t wgrad_t(const WgradArgs &a, int sms, cudaStream_t s)
 {
-    const size_t smem = (size_t)(64 * pitch(COUT) + 66 * pitch(NCI)) * 2;
-    cudaError_t e = cudaFuncSetAttribute(k_wgrad<CIN, COUT, NCI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    const int TW = a.W < 64 ? a.W : 64;
-    const long ntiles = (long)a.B * a.H * (a.W / TW);
+    constexpr size_t smem = (size_t)(MAX_W * pitch(COUT) + (MAX_W + 2) * pitch(NCI)) * 2;
+    static_assert(smem <= 48 * 1024, "");
     const int per = 3 * (CIN / NCI);
     long nsplit = (4L * sms + per - 1) / per;
-    if (nsplit > ntiles) nsplit = ntiles;
+    if (nsplit > (long)a.B * a.H) nsplit = (long)a.B * a.H;
     if (nsplit < 1) nsplit = 1;
     k_wgrad<CIN, COUT, NCI><<<(int)(per * nsplit), COUT * 2, smem, s>>>(a);
     return cudaGetLastError();
@@ -308,30 +288,25 @@ static cudaError_t wgrad_t(const WgradArgs &a, int sms, cudaStream_t s)
 
 cudaError_t launch_conv(int cin, int cout, bool dgrad, const ConvArgs &a, int sms, cudaStream_t s)
 {
-#define NN_CONV(CI, CO)                                                              \
-    if (cin == CI && cout == CO)                                                     \
-        return dgrad ? conv_t<CI, CO, true>(a, sms, s) : conv_t<CI, CO, false>(a, sms, s);
-    NN_CONV(16, 32)   // c1 forward (4 inputs padded to 16); c6 input gradient (16 -> 32)
-    NN_CONV(32, 64)   // c2 forward
-    NN_CONV(64, 64)   // c3 forward and input gradient
-    NN_CONV(128, 64)  // c4 forward
-    NN_CONV(96, 32)   // c5 forward
-    NN_CONV(32, 16)   // c6 forward (1 output padded to 16)
-    NN_CONV(64, 32)   // c2 input gradient (64 -> 32)
-    NN_CONV(64, 128)  // c4 input gradient (64 -> 128)
-    NN_CONV(32, 96)   // c5 input gradient (32 -> 96)
+    if (a.W > MAX_W || a.W % 16) return cudaErrorInvalidValue;
+#define NN_CONV(CI, CO, DG) \
+    if (cin == CI && cout == CO && dgrad == DG) return conv_t<CI, CO, DG>(a, sms, s);
+    NN_CONV(32, 64, false)    // c2
+    NN_CONV(64, 64, false)    // c3
+    NN_CONV(128, 64, false)   // c4
+    NN_CONV(64, 32, true)     // c2 input gradient
+    NN_CONV(64, 64, true)     // c3 input gradient
+    NN_CONV(64, 128, true)    // c4 input gradient
 #undef NN_CONV
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_wgrad(int cin, int cout, const WgradArgs &a, int sms, cudaStream_t s)
 {
-    if (cin == 16 && cout == 32) return wgrad_t<16, 32, 16>(a, sms, s);
+    if (a.W > MAX_W || a.W % 16) return cudaErrorInvalidValue;
     if (cin == 32 && cout == 64) return wgrad_t<32, 64, 32>(a, sms, s);
     if (cin == 64 && cout == 64) return wgrad_t<64, 64, 64>(a, sms, s);
     if (cin == 128 && cout == 64) return wgrad_t<128, 64, 64>(a, sms, s);
-    if (cin == 96 && cout == 32) return wgrad_t<96, 32, 32>(a, sms, s);
-    if (cin == 32 && cout == 16) return wgrad_t<32, 16, 32>(a, sms, s);
     return cudaErrorInvalidValue;
 }
 

@@ -56,7 +56,7 @@ struct ConvArgs {
     int yf_c;
     const __nv_bfloat16 *xc;    // tcgen05: first input channels, from the coarser level [B][H/2][W/2][.]
     __nv_bfloat16 *yp;          // tcgen05: 2x2 mean of y [B][H/2][W/2][cout]
-    const __nv_bfloat16 *mask;  // [B][H][W][cout]: zero the output where mask <= 0 (ReLU derivative), or null
+    const __nv_bfloat16 *mask;  // tcgen05: [B][H][W][cout], zero the output where mask <= 0 (ReLU derivative)
     int B, H, W;
     int relu;
 };
@@ -70,11 +70,12 @@ struct WgradArgs {
     int B, H, W;
 };
 
+// c2, c3, c4 and their input gradients (dgrad) for rows of 16 and 32 points
 cudaError_t launch_conv(int cin, int cout, bool dgrad, const ConvArgs &a, int sms, cudaStream_t s);
 // the network's convolutions and input gradients on tcgen05 (nn_tc.cu), with
-// what follows them fused, for rows of a multiple of 64 points (the others
-// take launch_conv and the kernels of nn_ops.cu); err (device) is set if a
-// tensor-core wait ran out
+// what follows them fused, for rows of a multiple of 64 points: every row of
+// the finest level (the other levels' shorter ones take launch_conv and the
+// kernels of nn_ops.cu); err (device) is set if a tensor-core wait ran out
 enum ConvStep : int {
     CONV_C1, CONV_C2,   // x -> y, and its 2x2 mean -> yp
     CONV_C3,            // x -> y

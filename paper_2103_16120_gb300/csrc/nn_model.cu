@@ -29,14 +29,20 @@ typedef __nv_bfloat16 bf16;
 struct Acts {
     size_t cap_n0 = 0, cap_hw = 0;   // capacity: points of a batch, points of one sample
     void *mem = nullptr;
-    bf16 *x0b, *a1, *p1, *a2, *p2, *a3, *cat4, *a4, *cat5, *a5;
+    bf16 *x0b, *a1, *p1, *a2, *p2, *a3, *a4, *a5;
     float *y;
     bf16 *gy16, *gz5, *gz4, *gz3, *gz2, *gz1;
-    float *gcat5, *gcat4, *gp2, *gp1;    // input gradients of the convolutions, FP32
+    float *gp2, *gp1;            // input gradients of the convolutions, FP32
     float *gskip1, *gskip2;
     float *x0f;                  // one sample's FP32 inputs (sw_model_apply)
     float *ef;                   // one sample's preconditioner output (solver)
     double *scal;                // [0]: sum r^2 (apply), [1]: loss
+    // c4's concatenated input and its gradient, stored where the middle level's
+    // rows are 32 points (nx = 64) only
+    size_t cap_cat = 0;          // capacity: points of a batch at that level
+    void *cat_mem = nullptr;
+    bf16 *cat4;
+    float *gcat4;
 };
 
 } // namespace
@@ -71,8 +77,8 @@ sw_status check_shape(int B, int H, int W)
 {
     if (B < 1) return sw::api_fail(SW_ERR_INVALID_ARG, "batch must be >= 1");
     if (H < 8 || (H & 3)) return sw::api_fail(SW_ERR_INVALID_ARG, "ny must be a multiple of 4 and >= 8");
-    // every level's row splits into tiles of 64 points, or is one tile of a
-    // multiple of 16 points
+    // every level's row splits into tiles of 64 points, or is one of 16 or 32
+    // points (64 and 128 at the finest level, which so always has tiles)
     for (int l = 0; l < 3; ++l) {
         const int Wl = W >> l;
         if ((W & ((1 << l) - 1)) || (Wl <= 64 ? (Wl & 15) : (Wl & 63)))
@@ -85,13 +91,22 @@ sw_status check_shape(int B, int H, int W)
 sw_status ensure_acts(sw_model_s *M, int B, int H, int W)
 {
     Acts &A = M->A;
+    const size_t ncat = conv_tc_rows(W / 2) ? 0 : (size_t)B * H * W / 4;
+    if (A.cap_cat < ncat) {
+        if (A.cat_mem) { cudaFree(A.cat_mem); A.cat_mem = nullptr; A.cap_cat = 0; }
+        M->gen = next_model_gen();
+        NCK(cudaMalloc(&A.cat_mem, al256(ncat * 128 * 2) + ncat * 128 * 4));
+        A.cat4 = (bf16 *)A.cat_mem;
+        A.gcat4 = (float *)((char *)A.cat_mem + al256(ncat * 128 * 2));
+        A.cap_cat = ncat;
+    }
     if (A.mem && A.cap_n0 >= (size_t)B * H * W && A.cap_hw >= (size_t)H * W) return SW_OK;
     if (A.mem) { cudaFree(A.mem); A.mem = nullptr; }
     M->gen = next_model_gen();
     const size_t N0 = (size_t)B * H * W, N1 = N0 / 4, N2 = N0 / 16;
-    const size_t hb[] = {N0 * 16, N0 * 32, N1 * 32, N1 * 64, N2 * 64, N2 * 64, N1 * 128, N1 * 64, N0 * 96, N0 * 32,
+    const size_t hb[] = {N0 * 16, N0 * 32, N1 * 32, N1 * 64, N2 * 64, N2 * 64, N1 * 64, N0 * 32,
                          N0 * 16, N0 * 32, N1 * 64, N2 * 64, N1 * 64, N0 * 32};
-    const size_t hf[] = {N0 * 96, N1 * 128, N2 * 64, N1 * 32};
+    const size_t hf[] = {N2 * 64, N1 * 32};
     size_t bytes = 0;
     for (size_t h : hb) bytes += al256(h * 2);
     for (size_t h : hf) bytes += al256(h * 4);
@@ -99,11 +114,11 @@ sw_status ensure_acts(sw_model_s *M, int B, int H, int W)
              al256((size_t)H * W * 4) + al256(64);
     NCK(cudaMalloc(&A.mem, bytes));
     char *p = (char *)A.mem;
-    bf16 **slots[] = {&A.x0b, &A.a1, &A.p1, &A.a2, &A.p2, &A.a3, &A.cat4, &A.a4, &A.cat5, &A.a5,
+    bf16 **slots[] = {&A.x0b, &A.a1, &A.p1, &A.a2, &A.p2, &A.a3, &A.a4, &A.a5,
                       &A.gy16, &A.gz5, &A.gz4, &A.gz3, &A.gz2, &A.gz1};
-    for (int q = 0; q < 16; ++q) { *slots[q] = (bf16 *)p; p += al256(hb[q] * 2); }
-    float **fslots[] = {&A.gcat5, &A.gcat4, &A.gp2, &A.gp1};
-    for (int q = 0; q < 4; ++q) { *fslots[q] = (float *)p; p += al256(hf[q] * 4); }
+    for (int q = 0; q < 14; ++q) { *slots[q] = (bf16 *)p; p += al256(hb[q] * 2); }
+    float **fslots[] = {&A.gp2, &A.gp1};
+    for (int q = 0; q < 2; ++q) { *fslots[q] = (float *)p; p += al256(hf[q] * 4); }
     A.y = (float *)p; p += al256(N0 * 4);
     A.gskip1 = (float *)p; p += al256(N0 * 32 * 4);
     A.gskip2 = (float *)p; p += al256(N1 * 64 * 4);
@@ -145,35 +160,37 @@ sw_status forward(sw_model_s *M, int B, int H, int W, const float *x0, cudaStrea
 {
     Acts &A = M->A;
     const int H1 = H / 2, W1 = W / 2, H2 = H / 4, W2 = W / 4;
-    // a convolution and the pooling of its output
-    auto conv_pool = [&](ConvStep step, int l, const bf16 *x, bf16 *y, bf16 *yp, int h, int w) -> cudaError_t {
-        ConvArgs a = conv_args(x, M->wf[l], M->bias[l], y, B, h, w, 1);
-        a.yp = yp;
-        if (conv_tc_rows(w)) return launch_conv_tc(step, a, M->sms, M->err, s);
-        const cudaError_t e = launch_conv(LAYER[l].cin_pad, LAYER[l].cout_pad, false, a, M->sms, s);
-        return e != cudaSuccess ? e : launch_pool(y, yp, B, h, w, LAYER[l].cout_pad, s);
-    };
-    // a convolution of [up(coarse), skip]; cat: where it is stored for rows
-    // that the tcgen05 kernel does not take
-    auto conv_cat = [&](ConvStep step, int l, const bf16 *coarse, const bf16 *skip, int cs, bf16 *cat, bf16 *y, int h,
-                        int w) -> cudaError_t {
-        ConvArgs a = conv_args(skip, M->wf[l], M->bias[l], y, B, h, w, 1);
-        a.xc = coarse;
-        if (conv_tc_rows(w)) return launch_conv_tc(step, a, M->sms, M->err, s);
-        const cudaError_t e = launch_cat_up(coarse, 64, skip, cs, cat, B, h, w, s);
-        a.x = cat;
-        return e != cudaSuccess ? e : launch_conv(64 + cs, LAYER[l].cout_pad, false, a, M->sms, s);
-    };
+    const bool tc1 = conv_tc_rows(W1), tc2 = conv_tc_rows(W2);
     NCK(launch_pack_input(x0, A.x0b, B, H, W, s));
-    NCK(conv_pool(CONV_C1, 0, A.x0b, A.a1, A.p1, H, W));
-    NCK(conv_pool(CONV_C2, 1, A.p1, A.a2, A.p2, H1, W1));
+    ConvArgs c1 = conv_args(A.x0b, M->wf[0], M->bias[0], A.a1, B, H, W, 1);
+    c1.yp = A.p1;
+    NCK(launch_conv_tc(CONV_C1, c1, M->sms, M->err, s));
+    ConvArgs c2 = conv_args(A.p1, M->wf[1], M->bias[1], A.a2, B, H1, W1, 1);
+    c2.yp = A.p2;
+    if (tc1) {
+        NCK(launch_conv_tc(CONV_C2, c2, M->sms, M->err, s));
+    } else {
+        NCK(launch_conv(32, 64, false, c2, M->sms, s));
+        NCK(launch_pool(A.a2, A.p2, B, H1, W1, 64, s));
+    }
     const ConvArgs c3 = conv_args(A.p2, M->wf[2], M->bias[2], A.a3, B, H2, W2, 1);
-    NCK(conv_tc_rows(W2) ? launch_conv_tc(CONV_C3, c3, M->sms, M->err, s) : launch_conv(64, 64, false, c3, M->sms, s));
-    NCK(conv_cat(CONV_C4, 3, A.a3, A.a2, 64, A.cat4, A.a4, H1, W1));
-    NCK(conv_cat(CONV_C5, 4, A.a4, A.a1, 32, A.cat5, A.a5, H, W));
-    ConvArgs o = conv_args(A.a5, M->wf[5], M->bias[5], nullptr, B, H, W, 0);
-    o.yf = A.y; o.yf_c = 1;
-    NCK(conv_tc_rows(W) ? launch_conv_tc(CONV_C6, o, M->sms, M->err, s) : launch_conv(32, 16, false, o, M->sms, s));
+    NCK(tc2 ? launch_conv_tc(CONV_C3, c3, M->sms, M->err, s) : launch_conv(64, 64, false, c3, M->sms, s));
+    // of [up(a3), a2] and [up(a4), a1]
+    ConvArgs c4 = conv_args(A.a2, M->wf[3], M->bias[3], A.a4, B, H1, W1, 1);
+    if (tc1) {
+        c4.xc = A.a3;
+        NCK(launch_conv_tc(CONV_C4, c4, M->sms, M->err, s));
+    } else {
+        NCK(launch_cat_up(A.a3, 64, A.a2, 64, A.cat4, B, H1, W1, s));
+        c4.x = A.cat4;
+        NCK(launch_conv(128, 64, false, c4, M->sms, s));
+    }
+    ConvArgs c5 = conv_args(A.a1, M->wf[4], M->bias[4], A.a5, B, H, W, 1);
+    c5.xc = A.a4;
+    NCK(launch_conv_tc(CONV_C5, c5, M->sms, M->err, s));
+    ConvArgs c6 = conv_args(A.a5, M->wf[5], M->bias[5], nullptr, B, H, W, 0);
+    c6.yf = A.y;
+    NCK(launch_conv_tc(CONV_C6, c6, M->sms, M->err, s));
     return SW_OK;
 }
 
@@ -185,11 +202,9 @@ sw_status backward(sw_model_s *M, int B, int H, int W, const float *target, cuda
     NCK(cudaMemsetAsync(M->dw[0], 0, M->grad_bytes, s));        // every dw and db
     NCK(cudaMemsetAsync(A.scal + 1, 0, sizeof(double), s));
     NCK(launch_loss(A.y, target, A.gy16, A.scal + 1, B, H, W, s));
-    auto wg = [&](int l, const bf16 *g, const bf16 *x, int h_, int w_, const bf16 *coarse = nullptr,
-                  const bf16 *cat = nullptr) {
-        // a concatenated input is stored only where the forward pass stored it
-        WgradArgs a{g, x, coarse, M->dw[l], M->db[l], B, h_, w_};
-        if (cat && !conv_tc_rows(w_)) a.x = cat;
+    const bool tc1 = conv_tc_rows(W1);
+    auto wg = [&](int l, const bf16 *g, const bf16 *x, int h_, int w_, const bf16 *coarse = nullptr) {
+        const WgradArgs a{g, x, coarse, M->dw[l], M->db[l], B, h_, w_};
         return launch_wgrad_auto(LAYER[l].cin_pad, LAYER[l].cout_pad, a, M->sms, M->err, s);
     };
     // input gradient with FP32 output
@@ -199,31 +214,32 @@ sw_status backward(sw_model_s *M, int B, int H, int W, const float *target, cuda
         return conv_tc_rows(w) ? launch_conv_tc(step, a, M->sms, M->err, s)
                                : launch_conv(LAYER[l].cout_pad, co, true, a, M->sms, s);
     };
-    // input gradient of a convolution of [up(coarse), skip], split into the
-    // coarse level's gradient (times the ReLU derivative) and the skip's
-    auto dgrad_cat = [&](ConvStep step, int l, const bf16 *g, float *gcat, int cs, const bf16 *coarse, bf16 *gz,
-                         float *gskip, int h, int w) -> cudaError_t {
-        if (conv_tc_rows(w)) {
-            ConvArgs a = conv_args(g, M->wd[l], nullptr, gz, B, h, w, 0);
-            a.mask = coarse;
-            a.yf = gskip;
-            return launch_conv_tc(step, a, M->sms, M->err, s);
-        }
-        const cudaError_t e =
-            launch_conv(LAYER[l].cout_pad, 64 + cs, true, dgrad_args(g, M->wd[l], gcat, 64 + cs, B, h, w), M->sms, s);
-        return e != cudaSuccess ? e : launch_split_up_bwd(gcat, 64, cs, coarse, gz, gskip, B, h, w, s);
+    // input gradient of a convolution of [up(coarse), skip] on tcgen05, split
+    // into the coarse level's gradient (times the ReLU derivative) and the skip's
+    auto dgrad_cat = [&](ConvStep step, int l, const bf16 *g, const bf16 *coarse, bf16 *gz, float *gskip, int h, int w) {
+        ConvArgs a = conv_args(g, M->wd[l], nullptr, gz, B, h, w, 0);
+        a.mask = coarse;
+        a.yf = gskip;
+        return launch_conv_tc(step, a, M->sms, M->err, s);
     };
     // c6 (32 -> 1, padded to 16 outputs)
     NCK(wg(5, A.gy16, A.a5, H, W));
     ConvArgs d6 = conv_args(A.gy16, M->wd[5], nullptr, A.gz5, B, H, W, 0);
     d6.mask = A.a5;
-    NCK(conv_tc_rows(W) ? launch_conv_tc(CONV_D6, d6, M->sms, M->err, s) : launch_conv(16, 32, true, d6, M->sms, s));
+    NCK(launch_conv_tc(CONV_D6, d6, M->sms, M->err, s));
     // c5 (96 -> 32) on [up(a4), a1]
-    NCK(wg(4, A.gz5, A.a1, H, W, A.a4, A.cat5));
-    NCK(dgrad_cat(CONV_D5, 4, A.gz5, A.gcat5, 32, A.a4, A.gz4, A.gskip1, H, W));
-    // c4 (128 -> 64) on [up(a3), a2]
-    NCK(wg(3, A.gz4, A.a2, H1, W1, A.a3, A.cat4));
-    NCK(dgrad_cat(CONV_D4, 3, A.gz4, A.gcat4, 64, A.a3, A.gz3, A.gskip2, H1, W1));
+    NCK(wg(4, A.gz5, A.a1, H, W, A.a4));
+    NCK(dgrad_cat(CONV_D5, 4, A.gz5, A.a4, A.gz4, A.gskip1, H, W));
+    // c4 (128 -> 64) on [up(a3), a2]; the concatenation is stored only where the
+    // forward pass stored it
+    if (tc1) {
+        NCK(wg(3, A.gz4, A.a2, H1, W1, A.a3));
+        NCK(dgrad_cat(CONV_D4, 3, A.gz4, A.a3, A.gz3, A.gskip2, H1, W1));
+    } else {
+        NCK(wg(3, A.gz4, A.cat4, H1, W1));
+        NCK(launch_conv(64, 128, true, dgrad_args(A.gz4, M->wd[3], A.gcat4, 128, B, H1, W1), M->sms, s));
+        NCK(launch_split_up_bwd(A.gcat4, 64, 64, A.a3, A.gz3, A.gskip2, B, H1, W1, s));
+    }
     // c3 (64 -> 64) on pool(a2)
     NCK(wg(2, A.gz3, A.p2, H2, W2));
     NCK(dgrad(CONV_D3, 2, A.gz3, A.gp2, H2, W2));
@@ -431,6 +447,7 @@ extern "C" sw_status sw_model_destroy(sw_model M)
     if (!M) return sw::api_fail(SW_ERR_INVALID_ARG, "sw_model_destroy: NULL model");
     cudaFree(M->pmem);
     if (M->A.mem) cudaFree(M->A.mem);
+    if (M->A.cat_mem) cudaFree(M->A.cat_mem);
     delete M;
     return SW_OK;
 }
