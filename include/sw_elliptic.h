@@ -129,9 +129,10 @@ typedef struct {
     int row_mode;        /* launch shape of the solver kernel: 0 automatic (one
                             thread block per latitude row while the rows fit the
                             resident blocks, else, in the mixed precisions, one
-                            warp per row when nx is a power of two >= 128 and a
-                            single grid is solved without the learned
-                            preconditioner, else blocks cycling over rows);
+                            warp per row when every nx is a power of two >= 128,
+                            R and phi start on 16-byte boundaries and the
+                            preconditioner is not the learned one, else blocks
+                            cycling over rows);
                             1 thread blocks only; 2 one warp per row
                             (SW_ERR_INVALID_ARG where not possible).  The
                             results agree to rounding: the inner products sum
@@ -140,7 +141,8 @@ typedef struct {
                             residual r0 = L(Phi_0) - R in FP32 with the split
                             fluid thickness of Sec. 4.2, Eq. 14, from the
                             grid's last sw_split_refresh (SW_ERR_INVALID_ARG
-                            without one); 0 (default) computes it in FP64.
+                            without one, or where R or phi does not start on a
+                            16-byte boundary); 0 (default) computes it in FP64.
                             Every later true residual, and so the exit test,
                             stays FP64. */
 } sw_solve_opts;

@@ -542,14 +542,20 @@ static void fill_member(sw_grid g, const sw_solve_opts *o, const double *R, doub
     M.shat = g->shat; M.sdx = g->sdx; M.scx = g->scx; M.sdy = g->sdy; M.scy = g->scy;
 }
 
-// the split initial residual needs a mixed precision, a refresh of this grid
-// and rows of a multiple of 8 points
-static sw_status check_split(const sw_grid_s *g, const sw_solve_opts *o)
+// R and Phi start on 16-byte boundaries, as the vector loads of the warp-per-row
+// kernels and of the split initial residual need (the block-per-row kernels
+// look at the pointers and take any)
+static bool vector_fields(const double *R, const double *phi) { return (((uintptr_t)R | (uintptr_t)phi) & 15) == 0; }
+
+// the split initial residual needs a mixed precision, a refresh of this grid,
+// rows of a multiple of 8 points and fields that allow vector loads
+static sw_status check_split(const sw_grid_s *g, const sw_solve_opts *o, const double *R, const double *phi)
 {
     if (!o->split_r0) return SW_OK;
     if (o->prec == SW_PREC_FP64) return fail(SW_ERR_INVALID_ARG, "split_r0 is for the mixed precisions");
     if (!g->split_valid) return fail(SW_ERR_INVALID_ARG, "split_r0: call sw_split_refresh on the grid first");
     if (g->nx % 8) return fail(SW_ERR_INVALID_ARG, "split_r0: nx must be a multiple of 8");
+    if (!vector_fields(R, phi)) return fail(SW_ERR_INVALID_ARG, "split_r0: R and phi must be 16-byte aligned");
     return SW_OK;
 }
 
@@ -659,7 +665,8 @@ static int share_blocks(int n, const sw_grid *grids, int cap, int lanes, std::ve
     }
 }
 
-static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o, int max_nx, Plan &P)
+static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o, const double *const *R,
+                             double *const *phi, int max_nx, Plan &P)
 {
     const int sms = grids[0]->sms;
     P.threads = row_threads(max_nx, o->threads_per_row);
@@ -677,10 +684,11 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     // the learned preconditioner ends a launch before every application of
     // the network, so the owner-only vectors cannot live in shared memory
     bool warp_possible = o->pc != SW_PC_LEARNED;
-    for (int m = 0; m < n; ++m) warp_possible = warp_possible && grids[m]->lfT;
+    for (int m = 0; m < n; ++m) warp_possible = warp_possible && grids[m]->lfT && vector_fields(R[m], phi[m]);
     if (o->row_mode == 2 && !warp_possible)
-        return fail(SW_ERR_INVALID_ARG, "row_mode 2 (one warp per row) needs grids with nx a power of two >= 128 "
-                                        "and a preconditioner other than the learned one");
+        return fail(SW_ERR_INVALID_ARG, "row_mode 2 (one warp per row) needs grids with nx a power of two >= 128, "
+                                        "R and phi on 16-byte boundaries and a preconditioner other than the learned "
+                                        "one");
     // one row per block where that fits, with row_threads' four warps or else
     // with about four points a thread (members of an ensemble, or rows of few
     // points, then still get a block each)
@@ -845,7 +853,7 @@ static sw_status check_members(int n, const sw_grid *grids, const sw_solve_opts 
             if (grids[q] == g) return fail(SW_ERR_INVALID_ARG, "the member grids must be distinct");
         if (n > 1 && (o->res_history || o->row_residual))
             return fail(SW_ERR_INVALID_ARG, "res_history / row_residual are for single solves");
-        if (sw_status sst = check_split(g, o)) return sst;
+        if (sw_status sst = check_split(g, o, R[m], phi[m])) return sst;
         max_nx = std::max(max_nx, g->nx);
     }
     return SW_OK;
@@ -881,7 +889,7 @@ static sw_status solve_one_async(sw_grid g, const sw_solve_opts *o, const double
     }
     if (o->res_history) CK(launch_fill(o->res_history, (size_t)o->max_iters + 1, NAN, s));
     Plan P;
-    if ((st = plan_launch(1, &g, o, max_nx, P))) return st;
+    if ((st = plan_launch(1, &g, o, &R, &phi, max_nx, P))) return st;
     a.blk = g->blk;
     a.desc = g->desc;
     a.stats = stats_dev;
@@ -925,7 +933,7 @@ static sw_status solve_members(int n, const sw_grid *grids, const sw_solve_opts 
             if (grids[q] == g) return fail(SW_ERR_INVALID_ARG, "the member grids must be distinct");
         if (n > 1 && (o->res_history || o->row_residual))
             return fail(SW_ERR_INVALID_ARG, "res_history / row_residual are for single solves");
-        if (sw_status sst = check_split(g, o)) return sst;
+        if (sw_status sst = check_split(g, o, R[m], phi[m])) return sst;
         max_nx = std::max(max_nx, g->nx);
     }
     if (n == 1 && o->pc != SW_PC_LEARNED) {
@@ -955,7 +963,7 @@ static sw_status solve_members(int n, const sw_grid *grids, const sw_solve_opts 
     if (o->res_history) CK(launch_fill(o->res_history, (size_t)o->max_iters + 1, NAN, s));
 
     Plan P;
-    if ((st = plan_launch(n, grids, o, max_nx, P))) return st;
+    if ((st = plan_launch(n, grids, o, R, phi, max_nx, P))) return st;
     const int threads = P.threads, grid = P.grid, cc = P.cc, cs = P.cs;
     const size_t smem = P.smem;
     const std::vector<int> &nb = P.nb;
@@ -1183,7 +1191,7 @@ extern "C" sw_status sw_gcr_solve_noalloc(sw_grid g, const sw_solve_opts *o, con
     int dev = -1;
     CK(cudaGetDevice(&dev));
     if (g->device != dev) return fail(SW_ERR_INVALID_ARG, "sw_gcr_solve_noalloc: the grid belongs to another device");
-    if ((st = check_split(g, o))) return st;
+    if ((st = check_split(g, o, R, phi))) return st;
     const size_t need = ws_layout(g, o->prec, o->k).total;
     if (need > SW_NOALLOC_SCRATCH_BYTES) {
         char msg[200];
@@ -1220,7 +1228,7 @@ extern "C" sw_status sw_gcr_solve_noalloc(sw_grid g, const sw_solve_opts *o, con
 
     // the launch shape of sw_gcr_solve for this grid and these options
     Plan P;
-    if ((st = plan_launch(1, &g, o, g->nx, P))) return st;
+    if ((st = plan_launch(1, &g, o, &R, &phi, g->nx, P))) return st;
     fill_desc(*g->h_desc, 1, &g, P);
     CK(cudaMemcpyAsync(g->desc, g->h_desc, sizeof(EnsDesc), cudaMemcpyHostToDevice, s));
     CK(launch_gcr(o->prec, o->k, P.minb, P.warp, g->desc, P.grid, g->nx, P.threads, P.smem, s));
@@ -1304,7 +1312,7 @@ extern "C" sw_status sw_ensemble_solve_async(int n, const sw_grid *grids, const 
     }
     if (o->res_history) CK(launch_fill(o->res_history, (size_t)o->max_iters + 1, NAN, s));
     Plan P;
-    if ((st = plan_launch(n, grids, o, max_nx, P))) return st;
+    if ((st = plan_launch(n, grids, o, R, phi, max_nx, P))) return st;
     sw_grid lead = grids[0];
     EnsDesc *hd = recorded ? lead->h_desc
                            : (EnsDesc *)((unsigned char *)mdev_slot(lead) +
