@@ -646,7 +646,8 @@ struct Plan {
 // the 8 members of 512 x 256 in the 64-member ensemble got 26 blocks of 8 warps
 // for their 256 rows, and every phase lasted two rows: the
 // ensemble took 5.33 ms, 4.92 with this in blocks of 4 warps.
-static int share_blocks(int n, const sw_grid *grids, int cap, int lanes, std::vector<int> &nb)
+// Returns the blocks used; *slowest: the slowest member's time.
+static int share_blocks(int n, const sw_grid *grids, int cap, int lanes, std::vector<int> &nb, double *slowest)
 {
     auto rounds = [&](int m) { return (grids[m]->ny + lanes * nb[m] - 1) / (lanes * nb[m]); };
     auto cost = [&](int m) { return grids[m]->nx * (rounds(m) * (grids[m]->nx + 64.0) + 200.0); };
@@ -669,6 +670,8 @@ static int share_blocks(int n, const sw_grid *grids, int cap, int lanes, std::ve
         heap.push_back({cost(slow), -slow});
         std::push_heap(heap.begin(), heap.end());
     }
+    *slowest = 0.0;
+    for (int m = 0; m < n; ++m) *slowest = std::max(*slowest, cost(m));
     return used;
 }
 
@@ -741,12 +744,24 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
         for (int m = 0; m < n; ++m) need += (grids[m]->ny + warps - 1) / warps;
         // the register budget of one block per SM unless that leaves rows
         // without a warp and two blocks fit.  Ensembles with rows of more than
-        // 128 points keep it all the same: their passes spill a quarter of
-        // their registers with half the budget (64 members of 128 x 64 to 512 x
-        // 256 4.93 against 4.41 ms, 40 of 256 x 128 2.09 against 1.89; 64 of 128
-        // x 64 0.65 against 0.71)
+        // 128 points spill a quarter of their passes' registers at half the
+        // budget, and a round of rows takes about twice as long (1.9 times with
+        // 256 points), so they take it where the slowest member then needs that
+        // much less time by its rounds.  Full and half, ms (ratio by rounds): 64
+        // members of 128 x 64 to 512 x 256 4.04, 4.56 (0.53); 40 of 256 x 128 1.84, 1.97
+        // (0.64); 32 each of 128 x 64 and 256 x 128 1.96, 1.69 (0.513); 200 of 256 x 128
+        // 10.6, 7.9 (0.36); 152 of 512 x 256, 12 iterations, 10.7, 10.9 (0.505); 80
+        // 24.3, 22.7 (0.46); 100 each of three sizes 63, 36 (0.25); with rows of 128
+        // points alone 64 members 0.64, 0.58
         P.minb = 1;
-        if ((long)bps * sms < need && bps2 > bps && (n == 1 || max_nx <= 128)) { bps = bps2; P.minb = 2; }
+        bool half = (long)bps * sms < need && bps2 > bps;
+        if (half && n > 1 && max_nx > 128 && n <= bps * sms) {
+            double t1 = 0.0, t2 = 0.0;
+            share_blocks(n, grids, bps * sms, warps, P.nb, &t1);
+            share_blocks(n, grids, bps2 * sms, warps, P.nb, &t2);
+            half = t2 < (max_nx <= 256 ? 0.52 : 0.5) * t1;
+        }
+        if (half) { bps = bps2; P.minb = 2; }
         if (bps >= 1 && n <= bps * sms) {
             if (n == 1) {
                 // the same number of blocks on every SM, as few as give every
@@ -756,7 +771,8 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
                 P.grid = std::min(per_sm * sms, grids[0]->ny);
                 P.nb[0] = P.grid;
             } else {
-                P.grid = share_blocks(n, grids, bps * sms, warps, P.nb);
+                double slowest;
+                P.grid = share_blocks(n, grids, bps * sms, warps, P.nb, &slowest);
             }
             P.warp = 1;
             // every member with rows of 1024 or 2048 points (and GCR k <= 4,

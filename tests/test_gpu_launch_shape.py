@@ -17,23 +17,14 @@ class KernelNodeParams(C.Structure):
                 ("params", C.c_void_p), ("extra", C.c_void_p)]
 
 
-def solver_launch(nx, ny, **opts):
-    """(blocks, threads, dynamic shared memory) of the solver kernel for a grid:
-    of the recorded kernels the one with most shared memory"""
-    P = synth.problem(nx, ny, 7)
-    g = sw.sw_grid_create(nx, ny)
-    sw.sw_elliptic_set_coeffs(g, *[torch.as_tensor(P[k], device="cuda") for k in sw.COEFF_KEYS])
-    R = torch.as_tensor(P["R"], device="cuda")
-    phi = torch.zeros_like(R)
-    o = sw.sw_solve_opts_default(max_iters=1, **opts)
-    sw.sw_gcr_solve(g, o, R, phi)                      # the workspace exists from here on
-    torch.cuda.synchronize()
-    rt, s = C.CDLL("libcudart.so.13"), torch.cuda.Stream()
+def recorded_kernels(s, call):
+    """(dynamic shared memory, blocks, threads) of every kernel that call records on stream s"""
+    rt = C.CDLL("libcudart.so.13")
     graph, n, p = C.c_void_p(), C.c_size_t(), KernelNodeParams()
     st = C.c_void_p(s.cuda_stream)
     assert rt.cudaStreamBeginCapture(st, 2) == 0       # relaxed
     try:
-        sw.sw_ensemble_solve_async([g], o, [R], [phi], stream=s)
+        call()
     finally:
         assert rt.cudaStreamEndCapture(st, C.byref(graph)) == 0
     assert rt.cudaGraphGetNodes(graph, None, C.byref(n)) == 0
@@ -46,7 +37,22 @@ def solver_launch(nx, ny, **opts):
         if kind.value == 0 and rt.cudaGraphKernelNodeGetParams(C.c_void_p(q), C.byref(p)) == 0:
             found.append((p.smem, p.grid[0], p.block[0]))
     assert rt.cudaGraphDestroy(graph) == 0
-    smem, blocks, threads = max(found)
+    return found
+
+
+def solver_launch(nx, ny, **opts):
+    """(blocks, threads, dynamic shared memory) of the solver kernel for a grid:
+    of the recorded kernels the one with most shared memory"""
+    P = synth.problem(nx, ny, 7)
+    g = sw.sw_grid_create(nx, ny)
+    sw.sw_elliptic_set_coeffs(g, *[torch.as_tensor(P[k], device="cuda") for k in sw.COEFF_KEYS])
+    R = torch.as_tensor(P["R"], device="cuda")
+    phi = torch.zeros_like(R)
+    o = sw.sw_solve_opts_default(max_iters=1, **opts)
+    sw.sw_gcr_solve(g, o, R, phi)                      # the workspace exists from here on
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    smem, blocks, threads = max(recorded_kernels(s, lambda: sw.sw_ensemble_solve_async([g], o, [R], [phi], stream=s)))
     return blocks, threads, smem
 
 
@@ -68,3 +74,30 @@ def test_scan_products_are_kept_where_they_are_used():
         blocks, threads, smem3 = solver_launch(1024, ny, prec=sw.SW_PREC_FP64)
         assert blocks == ny
         assert smem3 - solver_launch(1024, ny, prec=sw.SW_PREC_FP64, pc=sw.SW_PC_DIAG)[2] == 14 * 8 * threads
+
+
+def ensemble_launch(sizes):
+    """(blocks, threads) of an ensemble's solver kernel, recorded"""
+    gs, Rs, phis = [], [], []
+    for q, (nx, ny) in enumerate(sizes):
+        P = synth.problem(nx, ny, 7)
+        g = sw.sw_grid_create(nx, ny)
+        sw.sw_elliptic_set_coeffs(g, *[torch.as_tensor(P[k], device="cuda") for k in sw.COEFF_KEYS])
+        gs.append(g)
+        Rs.append(torch.as_tensor(P["R"], device="cuda"))
+        phis.append(torch.zeros_like(Rs[-1]))
+    o = sw.sw_solve_opts_default(prec=sw.SW_PREC_MIXED_FP16, max_iters=1)
+    sw.sw_ensemble_solve_async(gs, o, Rs, phis)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    smem, blocks, threads = max(recorded_kernels(s, lambda: sw.sw_ensemble_solve_async(gs, o, Rs, phis, stream=s)))
+    return blocks, threads
+
+
+# 304 blocks at the full register budget, 608 at half of it
+@pytest.mark.parametrize("counts,half", [((8, 40), False), ((0, 40), False), ((32, 32), True), ((0, 200), True)])
+def test_ensembles_take_half_the_registers_where_rounds_pay(counts, half):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    blocks, threads = ensemble_launch([(128, 64)] * counts[0] + [(256, 128)] * counts[1])
+    assert threads == 128
+    assert (blocks > 2 * sms) == half and blocks <= 4 * sms
