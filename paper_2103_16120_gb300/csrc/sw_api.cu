@@ -699,12 +699,18 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
         return fail(SW_ERR_INVALID_ARG, "row_mode 2 (one warp per row) needs grids with nx a power of two >= 128, "
                                         "R and phi on 16-byte boundaries and a preconditioner other than the learned "
                                         "one");
-    // one row per block where that fits, with row_threads' four warps or else
-    // with about four points a thread (members of an ensemble, or rows of few
-    // points, then still get a block each)
-    const int narrow = o->threads_per_row > 0 ? P.threads : setup_threads(max_nx);
-    const int shapes[2] = {P.threads, narrow};
-    for (int sh = 0; sh < (narrow < P.threads ? 2 : 1) && !P.grid && o->row_mode != 2; ++sh) {
+    // one row per block where that fits: with four warps or, for rows of more
+    // than 512 points, the more that about four points a thread make, then with
+    // the other of the two (members of an ensemble, or rows of few points, still
+    // get a block each with fewer warps, and rows of 512 to 1024 points with four
+    // in twice as many blocks per SM).  us per iteration FP16 / FP64 with four
+    // points a thread and with four warps: 640 x 120 23.6, 26.2; 768 x 152 24.6 / 37.8,
+    // 27.8 / 44.8; 1000 x 64 22.1 / 40.1, 25.3 / 47.9; 1000 x 290 does not fit, 31.1 /
+    // 64.5
+    const int quarter = o->threads_per_row > 0 ? P.threads : setup_threads(max_nx);
+    const int shapes[2] = {std::max(P.threads, quarter), std::min(P.threads, quarter)};
+    const int nshape = shapes[1] < shapes[0] ? 2 : 1;
+    for (int sh = 0; sh < nshape && !P.grid && o->row_mode != 2; ++sh) {
         for (const int(&lv)[3] : levels) {
             if (P.grid || (lv[1] && o->pc == SW_PC_LEARNED) || (lv[2] && !scans)) continue;
             const size_t sm_l = gcr_smem_bytes(o->prec, max_nx, o->k, lv[0], lv[1], lv[2] ? shapes[sh] : 0);
@@ -796,12 +802,25 @@ static sw_status plan_launch(int n, const sw_grid *grids, const sw_solve_opts *o
     if (!P.grid) {
         // blocks own several rows: take the register budget that fits more
         // resident blocks
-        if (n > 1) P.threads = narrow;
         P.smem = gcr_smem_bytes(o->prec, max_nx, o->k, 0, 0, 0);
         P.cc = P.cs = 0;
         int bps = 0, bps2 = 0;
-        CK(gcr_occupancy(o->prec, o->k, 1, 0, P.threads, P.smem, &bps));
-        CK(gcr_occupancy(o->prec, o->k, 2, 0, P.threads, P.smem, &bps2));
+        auto occupancy = [&](int threads) {
+            cudaError_t e = gcr_occupancy(o->prec, o->k, 1, 0, threads, P.smem, &bps);
+            return e == cudaSuccess ? gcr_occupancy(o->prec, o->k, 2, 0, threads, P.smem, &bps2) : e;
+        };
+        // ensembles: four points a thread.  A single grid: the threads, in the
+        // order of above and three warps at least, with which every row still gets
+        // a block at the smaller budget; if none, the first.  us per FP16 iteration
+        // with 96, 128 and 160 threads: 360 x 640 41.5, 51.1; 640 x 320 36.3, 35.2, 32.4; 640
+        // x 500 46.9, 45.6, 54.1; 640 x 760 56.5, 64.1, 55.3
+        P.threads = n > 1 ? quarter : shapes[0];
+        for (int sh = 0; n == 1 && sh < nshape; ++sh) {
+            if (shapes[sh] < 96) break;
+            CK(occupancy(shapes[sh]));
+            if (rows_total <= (long)std::max(bps, bps2) * sms) { P.threads = shapes[sh]; break; }
+        }
+        CK(occupancy(P.threads));
         // FP64: two blocks on an SM take 1.6 times (rows of 3000 points and more
         // 1.9 times) one block's time for a round of rows, so the last round
         // decides, one against two, us per iteration: 2048 x 1024 437, 392; 2600 x

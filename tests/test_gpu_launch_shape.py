@@ -101,3 +101,14 @@ def test_ensembles_take_half_the_registers_where_rounds_pay(counts, half):
     blocks, threads = ensemble_launch([(128, 64)] * counts[0] + [(256, 128)] * counts[1])
     assert threads == 128
     assert (blocks > 2 * sms) == half and blocks <= 4 * sms
+
+
+# about four points a thread above 512
+# points where the rows have a block each with that, else four warps; three
+# where only those give every row a block
+@pytest.mark.parametrize("nx,ny,prec,threads", [(512, 256, 1, 128), (520, 64, 1, 160), (640, 320, 1, 160), (640, 500, 1, 128),
+                                                (640, 640, 1, 160), (768, 120, 0, 192), (768, 384, 1, 128),
+                                                (1000, 64, 0, 256), (1024, 512, 0, 128), (360, 640, 1, 96),
+                                                (1440, 400, 1, 256)])
+def test_threads_of_a_row(nx, ny, prec, threads):
+    assert solver_launch(nx, ny, prec=prec)[1] == threads
