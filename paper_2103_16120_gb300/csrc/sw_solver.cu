@@ -450,15 +450,32 @@ static cudaError_t launch_precond_t(const void *M, int nx, int ny, int nstages, 
     return cudaGetLastError();
 }
 
+// Three blocks per SM, two for FP64 rows in four warps.  With a zonal solve,
+// fewer where the shared memory of longer rows holds no more: registers held
+// down for blocks that do not fit only spill the solve's chunks.  One stage
+// with three and with that many, us: FP64 2600 x 1300 169, 151; 3600 x 1801 306, 271
+// (287 before there were budgets); 4096 x 512 107, 88; FP16 3600 x 1801 107, 97.
+// Without a solve three stay the better (option 2, FP64 2600 x 1300 496, 516).
+template <class Pol>
+static cudaError_t launch_precond_p(const void *M, int nx, int ny, int nstages, void *qout, int threads,
+                                    cudaStream_t s)
+{
+    const int want = !Pol::kMixed && threads <= 128 ? 2 : 3;
+    int fit = 3;
+    if (((const MemberDev<Pol> *)M)->pc >= 3) fit = (int)(227 * 1024 / (work_bytes<Pol>(nx) + 2048));
+    if (want == 3 && fit >= 3) return launch_precond_t<Pol, 3>(M, nx, ny, nstages, qout, threads, s);
+    return fit >= 2 ? launch_precond_t<Pol, 2>(M, nx, ny, nstages, qout, threads, s)
+                    : launch_precond_t<Pol, 1>(M, nx, ny, nstages, qout, threads, s);
+}
+
 // M: the member descriptor, host memory (read before the call returns)
 cudaError_t launch_precond(int prec, const void *M, int nx, int ny, int nstages, void *qout, int threads,
                            cudaStream_t s)
 {
     switch (prec) {
-    case 0: return threads > 128 ? launch_precond_t<PolFP64, 3>(M, nx, ny, nstages, qout, threads, s)
-                                 : launch_precond_t<PolFP64, 2>(M, nx, ny, nstages, qout, threads, s);
-    case 1: return launch_precond_t<PolF16, 3>(M, nx, ny, nstages, qout, threads, s);
-    case 2: return launch_precond_t<PolBF16, 3>(M, nx, ny, nstages, qout, threads, s);
+    case 0: return launch_precond_p<PolFP64>(M, nx, ny, nstages, qout, threads, s);
+    case 1: return launch_precond_p<PolF16>(M, nx, ny, nstages, qout, threads, s);
+    case 2: return launch_precond_p<PolBF16>(M, nx, ny, nstages, qout, threads, s);
     default: return cudaErrorInvalidValue;
     }
 }
