@@ -110,7 +110,8 @@ GridView sw::grid_view(const sw_grid_s *g)
 // FP64 / FP16 with 32-192 and with 128 threads: 128 x 64 48 / 36 and 31 / 28,
 // 256 x 128 42 / 32 and 32 / 27, 360 x 181 46 / 32 and 46 / 29, 768 x 384
 // 101 / 49 and 81 / 41, 1024 x 512 (FP64) 132 and 118.  2048 x 1024 (FP64)
-// takes 397 with 256 and 508 with 128; 1440 x 721 (FP16) 104 and 109.
+// takes 397 with 256 and 508 with 128; 1440 x 721 (FP16) 104 and 109.  The solver
+// takes more for rows of 512 to 1024 points where its blocks allow (plan_launch).
 static int row_threads(int nx, int requested = 0)
 {
     int t = requested > 0 ? requested : (nx <= 1024 ? 128 : MAX_THREADS);
@@ -121,8 +122,9 @@ static int row_threads(int nx, int requested = 0)
     return t;
 }
 
-// threads of the FP32 factorisation's blocks, one row each: about four points
-// a thread (the pivots' chunks set the rounding of the FP32 factors)
+// about four points a thread: the FP32 factorisation's blocks, one row each (the
+// pivots' chunks set the rounding of the FP32 factors), and a launch shape of
+// the solver
 static int setup_threads(int nx)
 {
     int t = ((nx / 4 + 31) / 32) * 32;
